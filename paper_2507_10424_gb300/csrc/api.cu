@@ -111,7 +111,8 @@ struct ldpc {
 static void free_graph(DevGraph& g) {
     void* ptrs[] = {g.row_ptr, g.col_idx, g.col_ptr, g.col_edge, g.packed, g.r_base,
                     g.r_deg, g.r_slot_pos, g.c_base, g.c_deg, g.c_slot, g.col_pos,
-                    g.col_class, g.r_slot_cls, g.ell_col, g.ell_deg, g.ell_cslot, g.ell_cls};
+                    g.col_class, g.r_slot_cls, g.ell_col, g.ell_deg, g.ell_cslot, g.ell_cls,
+                    g.col_row, g.col_k};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     g = DevGraph();
@@ -358,6 +359,19 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
                 return bail(rc);
             h->dg.ell_D = eg.D;
             h->dg.eta_slots = (int64_t)hg.M * eg.D;
+        } else if (hg.max_dc <= 255) {
+            std::vector<int32_t> col_row((size_t)hg.E), row_of((size_t)hg.E);
+            std::vector<uint8_t> col_k((size_t)hg.E);
+            for (int32_t i = 0; i < hg.M; i++)
+                for (int32_t e2 = hg.row_ptr[i]; e2 < hg.row_ptr[i + 1]; e2++) row_of[e2] = i;
+            for (int64_t q = 0; q < hg.E; q++) {
+                const int32_t e2 = hg.col_edge[q];
+                col_row[q] = row_of[e2];
+                col_k[q] = (uint8_t)(e2 - hg.row_ptr[row_of[e2]]);
+            }
+            if ((rc = upload(&h->dg.col_row, col_row.data(), col_row.size())) ||
+                (rc = upload(&h->dg.col_k, col_k.data(), col_k.size())))
+                return bail(rc);
         }
     }
     // edge classes (learned weights)

@@ -152,6 +152,10 @@ struct DevGraph {
     int32_t ell_D = 0;
     // message slots of the streaming workspace: M ell_D with the padded layout, else E
     int64_t eta_slots = 0;
+    // codes without the padded row layout: row of each CSC edge and its position in the row
+    // (rows of at most 255 edges)
+    int32_t* col_row = nullptr;  // E
+    uint8_t* col_k = nullptr;    // E
 };
 
 // Index arrays the debug checks cover (ids in the report of ldpc_debug_report).

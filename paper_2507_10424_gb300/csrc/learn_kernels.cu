@@ -35,7 +35,7 @@ using namespace ldpc_impl;
 
 struct TrainWork {
     int32_t Fp;
-    float *r, *s, *eta, *dlam, *ds;
+    float *r, *s, *eta, *ds;
     uint8_t* sg;     // [T][E][Fp] sign bit of lambda (rows of more than 16 edges only)
     float* mn0;      // [T][M][Fp]
     float* mn1;      // [T][M][Fp]
@@ -60,7 +60,7 @@ size_t carve(int32_t M, int32_t N, int64_t E, int32_t F, int32_t T, bool packed,
     char* r = take((size_t)N * Fp * 4);
     char* s = take((size_t)N * Fp * 4);
     char* eta = take((size_t)E * Fp * 4);
-    char* dlam = take((size_t)E * Fp * 4);
+    take((size_t)E * Fp * 4);  // the gradient pairs of the rows continue behind eta
     char* ds = take((size_t)N * Fp * 4);
     char* sg = packed ? nullptr : take((size_t)T * E * Fp);
     char* mn0 = take((size_t)T * M * Fp * 4);
@@ -71,7 +71,6 @@ size_t carve(int32_t M, int32_t N, int64_t E, int32_t F, int32_t T, bool packed,
         w->r = (float*)r;
         w->s = (float*)s;
         w->eta = (float*)eta;
-        w->dlam = (float*)dlam;
         w->ds = (float*)ds;
         w->sg = (uint8_t*)sg;
         w->mn0 = (float*)mn0;
@@ -119,10 +118,43 @@ __global__ void k_lw_out(const float* src, int Fp, int N, int F, float* dst) {
 struct LwArgs {
     const int32_t *row_ptr, *col_idx, *col_ptr, *col_edge;
     const uint8_t* col_class;
+    // row and position in the row of each CSC edge: ell_cslot on the padded row layout (rows
+    // of at most 16 edges), else the two arrays
+    const int32_t *ell_cslot, *col_row;
+    const uint8_t* col_k;
+    int32_t dshift;
     int32_t M, N, C, Fp;
+    int32_t vrow;  // entry of row i's gradient pair: 2 i (0), or row_ptr[i] (1)
     int64_t E;
     const float *alpha, *beta;  // [T][C]
 };
+
+// V consecutive frames of one row, edge or bit: a lane's share of a frame-interleaved row.
+template <typename T, int V>
+struct alignas(sizeof(T) * V) LV {
+    T x[V];
+};
+template <int V, typename T>
+__device__ __forceinline__ LV<T, V> ldv(const T* p) {
+    return *reinterpret_cast<const LV<T, V>*>(p);
+}
+template <int V, typename T>
+__device__ __forceinline__ void stv(T* p, const LV<T, V>& v) {
+    *reinterpret_cast<LV<T, V>*>(p) = v;
+}
+// Fields of a check's word.
+template <bool PK>
+__device__ __forceinline__ int info_loc(uint32_t info) {
+    return info & (PK ? 0xf : 0xff);
+}
+template <bool PK>
+__device__ __forceinline__ int info_loc2(uint32_t info) {
+    return (info >> (PK ? 4 : 8)) & (PK ? 0xf : 0xff);
+}
+template <bool PK>
+__device__ __forceinline__ uint32_t info_par(uint32_t info) {
+    return (info >> (PK ? 8 : 16)) & 1u;
+}
 
 // Forward check pass of iteration t with saving; block = 4 checks x 32 frames.
 // PK: the row's sign bits go to its word (rows of at most 16 edges).
@@ -183,74 +215,229 @@ __global__ void __launch_bounds__(128) k_lw_var(LwArgs a, TrainWork w) {
     w.s[(size_t)j * Fp + f] = acc;
 }
 
-// Adjoint of the check pass of iteration t; LAST: t = T (no dlambda^(t+1)).
-template <bool LAST, bool PK>
-__global__ void __launch_bounds__(128) k_lw_bwd_row(LwArgs a, TrainWork w, int t, int F,
-                                                    float* grad_alpha, float* grad_beta) {
-    extern __shared__ float gacc[];  // [2][C]
-    for (int q = threadIdx.x; q < 2 * a.C; q += blockDim.x) gacc[q] = 0.0f;
+// Adjoint of the check pass of iteration t; LAST: t = T (no dlambda^(t+1)). A warp covers
+// 32 V frames of one row after another, so the weight gradients collect over many rows
+// before they leave the block.
+//
+// dlambda^t of a row is zero but at the locations of its two minima, so a row keeps two values
+// per frame (at loc and at loc2, lambda's sign applied) instead of one per edge; the
+// locations are in the saved word. Row i's pair sits at entries 2 i and 2 i + 1 of the
+// message region, which the backward pass does not need otherwise (row_ptr[i] and
+// row_ptr[i] + 1 when the code has more rows than edges: a row with edges has at least two).
+//
+// Weight gradients: GM = 0 (one class) in two registers a lane; GM = 1 (at most kLwClasses
+// classes) in a shared-memory accumulator of the lane's own per class; GM = 2 by a warp
+// reduction and two shared-memory atomics per edge.
+//
+// One edge and frame a thread with a dense edge gradient and two shared-memory atomics per
+// edge was bound by those atomics (all lanes on one address) and by 4-byte loads. Measured,
+// whole training steps (forward and backward): N=576, 4096 frames, 10 iterations 3.89 -> 0.87
+// ms; N=64800, 256 frames, 20 iterations 38.4 -> 12.7 ms.
+constexpr int kLwClasses = 16;
+template <int V, bool LAST, bool PK, int GM>
+__global__ void __launch_bounds__(128) k_lw_bwd_row(LwArgs a, TrainWork w, int t, float* grad_alpha,
+                                                    float* grad_beta) {
+    extern __shared__ float gacc[];  // GM 0, 1: [2 C][128]; GM 2: [2 C]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int q = threadIdx.x; q < 2 * a.C * (GM == 2 ? 1 : 128); q += 128) gacc[q] = 0.0f;
     __syncthreads();
-    const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int f = blockIdx.y * 32 + (threadIdx.x & 31);
     const int Fp = a.Fp;
-    if (i < a.M && f < F) {
+    const int f0 = (blockIdx.y * 32 + lane) * V;
+    const bool on = f0 < Fp;  // lanes behind the last frame stay for the reductions
+    const int fo = on ? f0 : 0;
+    const float* al = a.alpha + (size_t)(t - 1) * a.C;
+    const float* be = a.beta + (size_t)(t - 1) * a.C;
+    const uint8_t* sg = PK ? nullptr : w.sg + (size_t)(t - 1) * (size_t)a.E * Fp;
+    float ga = 0.0f, gb = 0.0f;
+    for (int i = blockIdx.x * 4 + warp; i < a.M; i += gridDim.x * 4) {
         const int e0 = __ldg(a.row_ptr + i), d = __ldg(a.row_ptr + i + 1) - e0;
-        const uint8_t* sg = PK ? nullptr : w.sg + (size_t)(t - 1) * (size_t)a.E * Fp;
-        const size_t ri = (size_t)(t - 1) * a.M * Fp + (size_t)i * Fp + f;
-        const float min0 = w.mn0[ri], min1 = w.mn1[ri];
-        const uint32_t info = w.info[ri];
-        const int loc = PK ? info & 0xf : info & 0xff, loc2 = PK ? (info >> 4) & 0xf : (info >> 8) & 0xff;
-        const uint32_t par = (info >> (PK ? 8 : 16)) & 1u;
-        auto neg_of = [&](int k, int e) -> uint32_t {  // sign bit of lambda of the row's k-th edge
-            return PK ? (info >> (16 + k)) & 1u : sg[(size_t)e * Fp + f];
-        };
-        const float* al = a.alpha + (size_t)(t - 1) * a.C;
-        const float* be = a.beta + (size_t)(t - 1) * a.C;
-        float acc_loc = 0.0f, acc_loc2 = 0.0f;
-        for (int k = 0; k < d; k++) {
-            const int e = e0 + k, c = __ldg(a.col_idx + e);
-            const int cls = __ldg(a.col_class + c);
-            float deta = w.ds[(size_t)c * Fp + f];
-            if (!LAST) deta -= w.dlam[(size_t)e * Fp + f];
-            const float m = k == loc ? min1 : min0;
-            const float alpha = __ldg(al + cls);
-            const float g = __fmaf_rn(alpha, m, -__ldg(be + cls));
-            if (g > 0.0f) {
-                const float dg = (par ^ neg_of(k, e)) ? -deta : deta;
-                atomicAdd(&gacc[cls], dg * m);
-                atomicAdd(&gacc[a.C + cls], -dg);
-                if (k != loc) acc_loc += dg * alpha;
-                else acc_loc2 += dg * alpha;
+        if (d == 0) continue;
+        const size_t ri = ((size_t)(t - 1) * a.M + i) * Fp + fo;
+        const size_t rv = (a.vrow ? (size_t)e0 : 2 * (size_t)i) * Fp + fo;
+        const LV<float, V> m0 = ldv<V>(w.mn0 + ri), m1 = ldv<V>(w.mn1 + ri);
+        const LV<uint32_t, V> info = ldv<V>(w.info + ri);
+        LV<float, V> p1, p2;  // dlambda^(t+1) of the row, at that iteration's minima
+        LV<uint32_t, V> pinfo;
+        if (!LAST) {
+            p1 = ldv<V>(w.eta + rv);
+            p2 = ldv<V>(w.eta + rv + Fp);
+            pinfo = ldv<V>(w.info + ri + (size_t)a.M * Fp);
+        }
+        float acc1[V], acc2[V];
+        uint32_t neg1[V], neg2[V];  // lambda's sign at loc and loc2
+        uint32_t sx[V];             // PK: the sign of the message to edge k at bit k
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            acc1[v] = acc2[v] = 0.0f;
+            neg1[v] = neg2[v] = sx[v] = 0;
+            if (PK) {
+                const uint32_t x = info.x[v];
+                sx[v] = (x >> 16) ^ (info_par<PK>(x) ? 0xffffu : 0u);
+                neg1[v] = (x >> (16 + info_loc<PK>(x))) & 1u;
+                neg2[v] = (x >> (16 + info_loc2<PK>(x))) & 1u;
             }
         }
-        for (int k = 0; k < d; k++) {
-            const int e = e0 + k;
-            float v = 0.0f;
-            if (k == loc) v = acc_loc;
-            else if (k == loc2) v = acc_loc2;
-            if (neg_of(k, e)) v = -v;  // d|lambda| / dlambda = sign(lambda), sign(0) = +1
-            w.dlam[(size_t)e * Fp + f] = v;
+        constexpr int U = 4;  // gathers in flight together
+        for (int k0 = 0; k0 < d; k0 += U) {
+            int c[U];
+            LV<float, V> dv[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) c[u] = __ldg(a.col_idx + e0 + min(k0 + u, d - 1));
+#pragma unroll
+            for (int u = 0; u < U; u++) dv[u] = ldv<V>(w.ds + (size_t)c[u] * Fp + fo);
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int k = k0 + u;
+                if (k >= d) break;  // the same for the whole warp
+                const int cls = GM == 0 ? 0 : __ldg(a.col_class + c[u]);
+                const float alpha = __ldg(al + cls), beta = __ldg(be + cls);
+                LV<uint8_t, V> sv;
+                if (!PK) sv = ldv<V>(sg + (size_t)(e0 + k) * Fp + fo);
+                float xa = 0.0f, xb = 0.0f;
+#pragma unroll
+                for (int v = 0; v < V; v++) {
+                    float deta = dv[u].x[v];
+                    if (!LAST)
+                        deta -= k == info_loc<PK>(pinfo.x[v])    ? p1.x[v]
+                                : k == info_loc2<PK>(pinfo.x[v]) ? p2.x[v]
+                                                                 : 0.0f;
+                    const bool at0 = k == info_loc<PK>(info.x[v]);
+                    const float m = at0 ? m1.x[v] : m0.x[v];
+                    const bool pos = __fmaf_rn(alpha, m, -beta) > 0.0f;
+                    uint32_t flip;
+                    if (PK) {
+                        flip = sx[v] << (31 - k);
+                    } else {
+                        if (at0) neg1[v] = sv.x[v];
+                        if (k == info_loc2<PK>(info.x[v])) neg2[v] = sv.x[v];
+                        flip = (info_par<PK>(info.x[v]) ^ sv.x[v]) << 31;
+                    }
+                    const float dg = __uint_as_float(__float_as_uint(deta) ^ (flip & 0x80000000u));
+                    const float da = pos ? dg * alpha : 0.0f;
+                    acc1[v] += at0 ? 0.0f : da;
+                    acc2[v] += at0 ? da : 0.0f;
+                    xa += pos ? dg * m : 0.0f;
+                    xb -= pos ? dg : 0.0f;
+                }
+                if constexpr (GM == 0) {
+                    ga += xa;
+                    gb += xb;
+                } else if constexpr (GM == 1) {
+                    float* g = gacc + 2 * cls * 128 + threadIdx.x;
+                    g[0] += xa;
+                    g[128] += xb;
+                } else {
+                    xa = on ? xa : 0.0f;
+                    xb = on ? xb : 0.0f;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        xa += __shfl_xor_sync(0xffffffffu, xa, o);
+                        xb += __shfl_xor_sync(0xffffffffu, xb, o);
+                    }
+                    if (lane == 0) {
+                        atomicAdd(gacc + 2 * cls, xa);
+                        atomicAdd(gacc + 2 * cls + 1, xb);
+                    }
+                }
+            }
+        }
+        if (on) {
+            LV<float, V> o1, o2;
+#pragma unroll
+            for (int v = 0; v < V; v++) {  // d|lambda| / dlambda = sign(lambda), sign(0) = +1
+                o1.x[v] = neg1[v] ? -acc1[v] : acc1[v];
+                o2.x[v] = neg2[v] ? -acc2[v] : acc2[v];
+            }
+            stv<V>(w.eta + rv, o1);
+            stv<V>(w.eta + rv + Fp, o2);
         }
     }
+    if constexpr (GM == 0) {
+        gacc[threadIdx.x] = ga;
+        gacc[128 + threadIdx.x] = gb;
+    }
+    if (GM != 2 && !on)  // what the lanes behind the last frame added up is not theirs
+        for (int q = 0; q < 2 * a.C; q++) gacc[q * 128 + threadIdx.x] = 0.0f;
     __syncthreads();
-    for (int q = threadIdx.x; q < 2 * a.C; q += blockDim.x) {
-        const float v = gacc[q];
-        if (v != 0.0f) atomicAdd(q < a.C ? grad_alpha + (size_t)(t - 1) * a.C + q
-                                         : grad_beta + (size_t)(t - 1) * a.C + (q - a.C), v);
+    for (int q = GM == 2 ? (int)threadIdx.x : warp; q < 2 * a.C; q += GM == 2 ? 128 : 4) {
+        float x;
+        if constexpr (GM == 2) {
+            x = gacc[q];
+        } else {
+            const float* g = gacc + q * 128 + lane;
+            x = (g[0] + g[32]) + (g[64] + g[96]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        }
+        if (x != 0.0f && (GM == 2 || lane == 0))
+            atomicAdd((q & 1 ? grad_beta : grad_alpha) + (size_t)(t - 1) * a.C + q / 2, x);
     }
 }
 
-// ds^(t-1)_j = sum over the edges of bit j of dlambda^t.
-__global__ void __launch_bounds__(128) k_lw_bwd_col(LwArgs a, TrainWork w, int F) {
+// ds^(t-1)_j = sum over the edges of bit j of dlambda^t, ascending rows: the pair of each row,
+// picked by the row's locations.
+template <int V, bool PK>
+__global__ void __launch_bounds__(128) k_lw_bwd_col(LwArgs a, TrainWork w, int t) {
     const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int f = blockIdx.y * 32 + (threadIdx.x & 31);
-    if (j >= a.N) return;
+    const int f0 = (blockIdx.y * 32 + (threadIdx.x & 31)) * V;
     const int Fp = a.Fp;
-    float acc = 0.0f;
-    if (f < F)
-        for (int q = __ldg(a.col_ptr + j); q < __ldg(a.col_ptr + j + 1); q++)
-            acc += w.dlam[(size_t)__ldg(a.col_edge + q) * Fp + f];
-    w.ds[(size_t)j * Fp + f] = acc;
+    if (j >= a.N || f0 >= Fp) return;
+    const uint32_t* info = w.info + (size_t)(t - 1) * a.M * Fp;
+    LV<float, V> acc;
+#pragma unroll
+    for (int v = 0; v < V; v++) acc.x[v] = 0.0f;
+    const int q1 = __ldg(a.col_ptr + j + 1);
+#pragma unroll 2
+    for (int q = __ldg(a.col_ptr + j); q < q1; q++) {
+        int i, k;
+        if (PK) {
+            const int slot = __ldg(a.ell_cslot + q);
+            i = slot >> a.dshift;
+            k = slot & ((1 << a.dshift) - 1);
+        } else {
+            i = __ldg(a.col_row + q);
+            k = __ldg(a.col_k + q);
+        }
+        const size_t rv = (a.vrow ? (size_t)__ldg(a.row_ptr + i) : 2 * (size_t)i) * Fp + f0;
+        const LV<uint32_t, V> x = ldv<V>(info + (size_t)i * Fp + f0);
+        const LV<float, V> p1 = ldv<V>(w.eta + rv), p2 = ldv<V>(w.eta + rv + Fp);
+#pragma unroll
+        for (int v = 0; v < V; v++)
+            acc.x[v] += k == info_loc<PK>(x.x[v])    ? p1.x[v]
+                        : k == info_loc2<PK>(x.x[v]) ? p2.x[v]
+                                                     : 0.0f;
+    }
+    stv<V>(w.ds + (size_t)j * Fp + f0, acc);
+}
+
+// Frames a lane takes: the widest vector (16 bytes) that still gives the GPU eight warps per SM
+// over `rows` rows, and no lane group without frames. One frame when the caller's workspace
+// is not 16-byte aligned.
+int lane_frames(int32_t rows, int32_t Fp, int num_sms, const void* work) {
+    int V = ((uintptr_t)work & 15) ? 1 : 4;
+    while (V > 1 && (Fp < 32 * V || (int64_t)rows * ((Fp + 32 * V - 1) / (32 * V)) < 8ll * num_sms)) V /= 2;
+    return V;
+}
+
+template <int V, bool PK>
+void launch_bwd(const LwArgs& a, const TrainWork& w, int t, bool last, int num_sms, float* grad_alpha,
+                float* grad_beta, cudaStream_t st) {
+    const int fb = (a.Fp + 32 * V - 1) / (32 * V);
+    // about 16 blocks an SM (their warps take several rows each)
+    const int gx = std::max(1, std::min((a.M + 3) / 4, (16 * num_sms + fb - 1) / fb));
+    const int gm = a.C == 1 ? 0 : a.C <= kLwClasses ? 1 : 2;
+    const size_t sm = (size_t)2 * a.C * (gm == 2 ? 1 : 128) * sizeof(float);
+    auto go = [&](auto row) { row<<<dim3(gx, fb), 128, sm, st>>>(a, w, t, grad_alpha, grad_beta); };
+    if (last) {
+        if (gm == 0) go(k_lw_bwd_row<V, true, PK, 0>);
+        else if (gm == 1) go(k_lw_bwd_row<V, true, PK, 1>);
+        else go(k_lw_bwd_row<V, true, PK, 2>);
+    } else {
+        if (gm == 0) go(k_lw_bwd_row<V, false, PK, 0>);
+        else if (gm == 1) go(k_lw_bwd_row<V, false, PK, 1>);
+        else go(k_lw_bwd_row<V, false, PK, 2>);
+    }
+    if (t > 1) k_lw_bwd_col<V, PK><<<dim3((a.N + 3) / 4, fb), 128, 0, st>>>(a, w, t);
 }
 
 bool packed_signs(const HandleView& v) { return v.dg->max_dc <= kPackedSignsMaxRow; }
@@ -272,6 +459,11 @@ LwArgs make_args(const HandleView& v, int32_t Fp, const float* alpha, const floa
     a.col_ptr = v.dg->col_ptr;
     a.col_edge = v.dg->col_edge;
     a.col_class = v.dg->col_class;
+    a.ell_cslot = v.dg->ell_cslot;
+    a.col_row = v.dg->col_row;
+    a.col_k = v.dg->col_k;
+    a.dshift = v.dg->ell_D == 16 ? 4 : 3;
+    a.vrow = v.M > v.E;
     a.M = v.M;
     a.N = v.N;
     a.C = v.dg->n_classes;
@@ -352,22 +544,18 @@ int ldpc_train_backward(ldpc_t* h, int32_t frames, int32_t iters, const float* a
     // ds^T = the loss gradient of the last posteriors
     k_lw_in<<<gi, bi, 0, st>>>(grad_soft + (soft_every ? (size_t)(iters - 1) * plane : 0), frames,
                                v.N, w.ds, nullptr, w.Fp);
-    const dim3 gc((v.M + 3) / 4, w.Fp / 32), gv((v.N + 3) / 4, w.Fp / 32);
-    const size_t sm = 2 * a.C * sizeof(float);
+    const int V = lane_frames(v.M, w.Fp, v.num_sms, work);
     int launches = 1;
     for (int t = iters; t >= 1; t--) {
-        auto row = t == iters ? (pk ? k_lw_bwd_row<true, true> : k_lw_bwd_row<true, false>)
-                              : (pk ? k_lw_bwd_row<false, true> : k_lw_bwd_row<false, false>);
-        row<<<gc, 128, sm, st>>>(a, w, t, frames, grad_alpha, grad_beta);
-        launches++;
-        if (t > 1) {
-            k_lw_bwd_col<<<gv, 128, 0, st>>>(a, w, frames);  // ds^(t-1) through lambda^t
+        auto step = V == 4   ? (pk ? launch_bwd<4, true> : launch_bwd<4, false>)
+                    : V == 2 ? (pk ? launch_bwd<2, true> : launch_bwd<2, false>)
+                             : (pk ? launch_bwd<1, true> : launch_bwd<1, false>);
+        step(a, w, t, t == iters, v.num_sms, grad_alpha, grad_beta, st);
+        launches += t > 1 ? 2 : 1;
+        if (t > 1 && soft_every) {  // plus the loss gradient of the posteriors of iteration t-1
+            k_lw_in<<<gi, bi, 0, st>>>(grad_soft + (size_t)(t - 2) * plane, frames, v.N, w.ds, nullptr,
+                                       w.Fp, 1);
             launches++;
-            if (soft_every) {  // plus the loss gradient of the posteriors of iteration t-1
-                k_lw_in<<<gi, bi, 0, st>>>(grad_soft + (size_t)(t - 2) * plane, frames, v.N, w.ds,
-                                           nullptr, w.Fp, 1);
-                launches++;
-            }
         }
     }
     *v.last_launches = launches;
