@@ -19,7 +19,8 @@
 //   (a subgradient through min / argmin): dlambda^t = sign(lambda) * that sum, else 0;
 //   ds^(t-1)_j = sum of dlambda^t over the edges of bit j.
 // Layout: frame-interleaved, element (row/edge/bit x, frame f) at x * Fp + f; a warp
-// covers 32 consecutive frames of one check or bit. The saved state of a check is min0,
+// covers 32, 64 or 128 consecutive frames of one check or bit (1, 2 or 4 a lane). No pass
+// stores messages or their gradients per edge: both are rebuilt from what a row keeps. The saved state of a check is min0,
 // min1 and one word: for codes whose rows have at most 16 edges the word also holds the
 // row's sign bits (loc | loc2 << 4 | parity << 8 | sign of lambda_k << (16 + k)), so each
 // iteration keeps 12 bytes per check and frame; longer rows keep loc | loc2 << 8 |
@@ -80,9 +81,8 @@ size_t carve(int32_t M, int32_t N, int64_t E, int32_t F, int32_t T, bool packed,
     return o;
 }
 
-// [F][N] -> [N][Fp] (and the copy into s); frames past F are zero. acc: add into dst.
-__global__ void k_lw_in(const float* src, int F, int N, float* dst, float* dst2, int Fp,
-                        int acc = 0) {
+// [F][N] -> [N][Fp]; frames past F are zero.
+__global__ void k_lw_in(const float* src, int F, int N, float* dst, int Fp) {
     __shared__ float tile[32][33];
     const int j0 = blockIdx.x * 32, f0 = blockIdx.y * 32;
     for (int y = threadIdx.y; y < 32; y += blockDim.y) {
@@ -92,26 +92,7 @@ __global__ void k_lw_in(const float* src, int F, int N, float* dst, float* dst2,
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += blockDim.y) {
         const int j = j0 + y, f = f0 + threadIdx.x;
-        if (j < N && f < Fp) {
-            const size_t o = (size_t)j * Fp + f;
-            dst[o] = acc ? dst[o] + tile[threadIdx.x][y] : tile[threadIdx.x][y];
-            if (dst2) dst2[o] = tile[threadIdx.x][y];
-        }
-    }
-}
-
-// [N][Fp] -> [F][N]
-__global__ void k_lw_out(const float* src, int Fp, int N, int F, float* dst) {
-    __shared__ float tile[32][33];
-    const int j0 = blockIdx.x * 32, f0 = blockIdx.y * 32;
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int j = j0 + y, f = f0 + threadIdx.x;
-        tile[y][threadIdx.x] = (j < N && f < F) ? src[(size_t)j * Fp + f] : 0.0f;
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int f = f0 + y, j = j0 + threadIdx.x;
-        if (f < F && j < N) dst[(size_t)f * N + j] = tile[threadIdx.x][y];
+        if (j < N && f < Fp) dst[(size_t)j * Fp + f] = tile[threadIdx.x][y];
     }
 }
 
@@ -156,63 +137,193 @@ __device__ __forceinline__ uint32_t info_par(uint32_t info) {
     return (info >> (PK ? 8 : 16)) & 1u;
 }
 
-// Forward check pass of iteration t with saving; block = 4 checks x 32 frames.
-// PK: the row's sign bits go to its word (rows of at most 16 edges).
-template <bool FIRST, bool PK>
-__global__ void __launch_bounds__(128) k_lw_check(LwArgs a, TrainWork w, int t) {
-    const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int f = blockIdx.y * 32 + (threadIdx.x & 31);
-    if (i >= a.M) return;
-    const int Fp = a.Fp;
-    const int e0 = __ldg(a.row_ptr + i), d = __ldg(a.row_ptr + i + 1) - e0;
-    uint8_t* sg = PK ? nullptr : w.sg + (size_t)(t - 1) * (size_t)a.E * Fp;
-    float min0 = __int_as_float(0x7f800000), min1 = min0;
-    int loc = 0, loc2 = 0;
-    uint32_t par = 0, sgw = 0;
-    for (int k = 0; k < d; k++) {
-        const int e = e0 + k, c = __ldg(a.col_idx + e);
-        const float lam = FIRST ? w.s[(size_t)c * Fp + f] : w.s[(size_t)c * Fp + f] - w.eta[(size_t)e * Fp + f];
-        const float m = fabsf(lam);
-        const uint32_t neg = lam < 0.0f;
-        par ^= neg;
-        if (PK) sgw |= neg << k;
-        else sg[(size_t)e * Fp + f] = (uint8_t)neg;
-        if (m < min0) {
-            min1 = min0;
-            loc2 = loc;
-            min0 = m;
-            loc = k;
-        } else if (m < min1) {
-            min1 = m;
-            loc2 = k;
-        }
-    }
-    const size_t ri = (size_t)(t - 1) * a.M * Fp + (size_t)i * Fp + f;
-    w.mn0[ri] = min0;
-    w.mn1[ri] = min1;
-    w.info[ri] = PK ? (uint32_t)loc | ((uint32_t)loc2 << 4) | (par << 8) | (sgw << 16)
-                    : (uint32_t)loc | ((uint32_t)loc2 << 8) | (par << 16);
-    const float* al = a.alpha + (size_t)(t - 1) * a.C;
-    const float* be = a.beta + (size_t)(t - 1) * a.C;
-    for (int k = 0; k < d; k++) {
-        const int e = e0 + k, cls = __ldg(a.col_class + __ldg(a.col_idx + e));
-        const float g = __fmaf_rn(__ldg(al + cls), k == loc ? min1 : min0, -__ldg(be + cls));
-        const float mag = g > 0.0f ? g : 0.0f;
-        const uint32_t neg = PK ? (sgw >> k) & 1u : sg[(size_t)e * Fp + f];
-        w.eta[(size_t)e * Fp + f] = (par ^ neg) ? -mag : mag;
+// Row and position in the row of CSC edge q.
+template <bool PK>
+__device__ __forceinline__ void edge_at(const LwArgs& a, int q, int& i, int& k) {
+    if (PK) {
+        const int slot = __ldg(a.ell_cslot + q);
+        i = slot >> a.dshift;
+        k = slot & ((1 << a.dshift) - 1);
+    } else {
+        i = __ldg(a.col_row + q);
+        k = __ldg(a.col_k + q);
     }
 }
 
-// Forward bit pass: s = r + sum of eta in ascending row order.
-__global__ void __launch_bounds__(128) k_lw_var(LwArgs a, TrainWork w) {
-    const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int f = blockIdx.y * 32 + (threadIdx.x & 31);
-    if (j >= a.N) return;
+// max(fma(alpha, m, -beta), 0) with the sign bit of `flip`.
+__device__ __forceinline__ float lw_message(float m, float alpha, float beta, uint32_t flip) {
+    const float g = __fmaf_rn(alpha, m, -beta);
+    const float mag = g > 0.0f ? g : 0.0f;
+    return __uint_as_float(__float_as_uint(mag) ^ (flip & 0x80000000u));
+}
+
+// Forward check pass of iteration t with saving; a warp takes one row of 32 V frames. The
+// messages of iteration t - 1 are rebuilt from its saved state (12 bytes a row instead of 4
+// an edge, and no message is ever written), so the pass reads each edge's s, gathered, and
+// the row's state twice 12 bytes. PK: the row's sign bits go to its word (rows of at most 16
+// edges). Bound by the latency of its gathers (index, then s). With the posteriors written
+// by the bit pass itself, a training step went from 0.87 to 0.61 ms (N=576, 4096 frames, 10
+// iterations) and from 12.7 to 8.5 ms (N=64800, 256 frames, 20 iterations: this pass 167 ->
+// 108 us, the bit pass with its output 176 -> 84 us a launch).
+template <int V, bool FIRST, bool PK>
+__global__ void __launch_bounds__(128) k_lw_check(LwArgs a, TrainWork w, int t) {
+    const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int f0 = (blockIdx.y * 32 + (threadIdx.x & 31)) * V;
     const int Fp = a.Fp;
-    float acc = w.r[(size_t)j * Fp + f];
-    for (int q = __ldg(a.col_ptr + j); q < __ldg(a.col_ptr + j + 1); q++)
-        acc = acc + w.eta[(size_t)__ldg(a.col_edge + q) * Fp + f];
-    w.s[(size_t)j * Fp + f] = acc;
+    if (i >= a.M || f0 >= Fp) return;
+    const int e0 = __ldg(a.row_ptr + i), d = __ldg(a.row_ptr + i + 1) - e0;
+    const float* s = FIRST ? w.r : w.s;
+    const size_t ri = ((size_t)(t - 1) * a.M + i) * Fp + f0, rp = ri - (size_t)a.M * Fp;
+    uint8_t* sg = PK ? nullptr : w.sg + (size_t)(t - 1) * (size_t)a.E * Fp + (size_t)e0 * Fp + f0;
+    const float* al = a.alpha + (size_t)(FIRST ? 0 : t - 2) * a.C;
+    const float* be = a.beta + (size_t)(FIRST ? 0 : t - 2) * a.C;
+    const bool one = a.C == 1;
+    LV<float, V> om0, om1;
+    LV<uint32_t, V> oinfo;
+    uint32_t osx[V];  // PK: sign of the old message to edge k at bit k
+    float al1 = 1.0f, be1 = 0.0f;
+    if (!FIRST) {
+        om0 = ldv<V>(w.mn0 + rp);
+        om1 = ldv<V>(w.mn1 + rp);
+        oinfo = ldv<V>(w.info + rp);
+        al1 = __ldg(al);
+        be1 = __ldg(be);
+        if (PK) {
+#pragma unroll
+            for (int v = 0; v < V; v++) osx[v] = (oinfo.x[v] >> 16) ^ (info_par<PK>(oinfo.x[v]) ? 0xffffu : 0u);
+        }
+    }
+    LV<float, V> min0, min1;
+    int loc[V], loc2[V];
+    uint32_t par[V], sgw[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        min0.x[v] = min1.x[v] = __int_as_float(0x7f800000);
+        loc[v] = loc2[v] = 0;
+        par[v] = sgw[v] = 0;
+    }
+    constexpr int U = 4;  // gathers in flight together
+    for (int k0 = 0; k0 < d; k0 += U) {
+        int c[U];
+        LV<float, V> sv[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) c[u] = __ldg(a.col_idx + e0 + min(k0 + u, d - 1));
+#pragma unroll
+        for (int u = 0; u < U; u++) sv[u] = ldv<V>(s + (size_t)c[u] * Fp + f0);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int k = k0 + u;
+            if (k >= d) break;  // the same for the whole warp
+            float ak = al1, bk = be1;
+            LV<uint8_t, V> sb;
+            if (!FIRST) {
+                if (!one) {
+                    const int cls = __ldg(a.col_class + c[u]);
+                    ak = __ldg(al + cls);
+                    bk = __ldg(be + cls);
+                }
+                if (!PK) sb = ldv<V>(sg - (size_t)a.E * Fp + (size_t)k * Fp);
+            }
+            LV<uint8_t, V> nb;
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                float lam = sv[u].x[v];
+                if (!FIRST) {
+                    const float m = k == info_loc<PK>(oinfo.x[v]) ? om1.x[v] : om0.x[v];
+                    const uint32_t flip =
+                        PK ? osx[v] << (31 - k) : (info_par<PK>(oinfo.x[v]) ^ sb.x[v]) << 31;
+                    lam = lam - lw_message(m, ak, bk, flip);
+                }
+                const float m = fabsf(lam);
+                const uint32_t neg = lam < 0.0f;
+                if (PK) {
+                    sgw[v] |= neg << k;
+                } else {
+                    par[v] ^= neg;
+                    nb.x[v] = (uint8_t)neg;
+                }
+                const bool lt0 = m < min0.x[v], lt1 = m < min1.x[v];
+                loc2[v] = lt0 ? loc[v] : lt1 ? k : loc2[v];
+                min1.x[v] = lt0 ? min0.x[v] : lt1 ? m : min1.x[v];
+                loc[v] = lt0 ? k : loc[v];
+                min0.x[v] = lt0 ? m : min0.x[v];
+            }
+            if (!PK) stv<V>(sg + (size_t)k * Fp, nb);
+        }
+    }
+    LV<uint32_t, V> info;
+#pragma unroll
+    for (int v = 0; v < V; v++)
+        info.x[v] = PK ? (uint32_t)loc[v] | ((uint32_t)loc2[v] << 4) | ((__popc(sgw[v]) & 1u) << 8) | (sgw[v] << 16)
+                       : (uint32_t)loc[v] | ((uint32_t)loc2[v] << 8) | (par[v] << 16);
+    stv<V>(w.mn0 + ri, min0);
+    stv<V>(w.mn1 + ri, min1);
+    stv<V>(w.info + ri, info);
+}
+
+// Tile of 32 bits x 32 V frames between the frame-interleaved arrays (a warp holds one bit,
+// a lane V consecutive frames) and the caller's frame-major [F][N] ones: frame lane V + v of
+// a bit sits at column v 32 + lane, so neither side has bank conflicts.
+template <int V>
+struct LwTile {
+    float x[32][32 * V + 1];
+    __device__ __forceinline__ void put(int c, int lane, const LV<float, V>& a) {
+#pragma unroll
+        for (int v = 0; v < V; v++) x[c][v * 32 + lane] = a.x[v];
+    }
+    __device__ __forceinline__ LV<float, V> get(int c, int lane) const {
+        LV<float, V> a;
+#pragma unroll
+        for (int v = 0; v < V; v++) a.x[v] = x[c][v * 32 + lane];
+        return a;
+    }
+    __device__ __forceinline__ float& at(int c, int f) { return x[c][(f % V) * 32 + f / V]; }
+};
+
+// Forward bit pass: s = r + sum of eta in ascending row order, the messages rebuilt from the
+// rows' states; a block takes 32 bits, 8 warps of 4. soft (nullable): also written to
+// soft [F][N], from the tile in shared memory, so that s is not read again to transpose it;
+// keep: s is needed by a later iteration.
+template <int V, bool PK>
+__global__ void __launch_bounds__(256) k_lw_var(LwArgs a, TrainWork w, int t, float* soft, int F, int keep) {
+    __shared__ LwTile<V> tile;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j0 = blockIdx.x * 32, fb = blockIdx.y * 32 * V, f0 = fb + lane * V;
+    const int Fp = a.Fp;
+    const size_t base = (size_t)(t - 1) * a.M * Fp + f0;
+    for (int b = warp; b < 32 && j0 + b < a.N; b += 8) {
+        if (f0 >= Fp) break;
+        const int j = j0 + b;
+        const int cls = a.C == 1 ? 0 : __ldg(a.col_class + j);
+        const float al = __ldg(a.alpha + (size_t)(t - 1) * a.C + cls);
+        const float be = __ldg(a.beta + (size_t)(t - 1) * a.C + cls);
+        LV<float, V> acc = ldv<V>(w.r + (size_t)j * Fp + f0);
+        const int q1 = __ldg(a.col_ptr + j + 1);
+#pragma unroll 2
+        for (int q = __ldg(a.col_ptr + j); q < q1; q++) {
+            int i, k;
+            edge_at<PK>(a, q, i, k);
+            const size_t o = base + (size_t)i * Fp;
+            const LV<float, V> m0 = ldv<V>(w.mn0 + o), m1 = ldv<V>(w.mn1 + o);
+            const LV<uint32_t, V> x = ldv<V>(w.info + o);
+            LV<uint8_t, V> sb;
+            if (!PK)
+                sb = ldv<V>(w.sg + ((size_t)(t - 1) * a.E + __ldg(a.col_edge + q)) * Fp + f0);
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                const float m = k == info_loc<PK>(x.x[v]) ? m1.x[v] : m0.x[v];
+                const uint32_t neg = PK ? x.x[v] >> (16 + k) : (uint32_t)sb.x[v];
+                acc.x[v] = acc.x[v] + lw_message(m, al, be, (info_par<PK>(x.x[v]) ^ neg) << 31);
+            }
+        }
+        if (keep) stv<V>(w.s + (size_t)j * Fp + f0, acc);
+        if (soft) tile.put(b, lane, acc);
+    }
+    if (!soft) return;
+    __syncthreads();
+    if (j0 + lane >= a.N) return;
+    for (int y = warp; y < 32 * V && fb + y < F; y += 8)
+        soft[(size_t)(fb + y) * a.N + j0 + lane] = tile.at(lane, y);
 }
 
 // Adjoint of the check pass of iteration t; LAST: t = T (no dlambda^(t+1)). A warp covers
@@ -374,40 +485,51 @@ __global__ void __launch_bounds__(128) k_lw_bwd_row(LwArgs a, TrainWork w, int t
     }
 }
 
-// ds^(t-1)_j = sum over the edges of bit j of dlambda^t, ascending rows: the pair of each row,
-// picked by the row's locations.
+// ds^(t-1)_j = sum over the edges of bit j of dlambda^t, ascending rows (the pair of each
+// row, picked by the row's locations), plus the loss gradient of the posteriors of iteration
+// t - 1 (grad [F][N], nullable), read through the tile: a block takes 32 bits. Measured
+// against a pass of its own that adds the gradient: 137 + 52 -> 82 us a launch (N=64800, 256
+// frames).
 template <int V, bool PK>
-__global__ void __launch_bounds__(128) k_lw_bwd_col(LwArgs a, TrainWork w, int t) {
-    const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int f0 = (blockIdx.y * 32 + (threadIdx.x & 31)) * V;
+__global__ void __launch_bounds__(256) k_lw_bwd_col(LwArgs a, TrainWork w, int t, const float* grad, int F) {
+    __shared__ LwTile<V> tile;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j0 = blockIdx.x * 32, fb = blockIdx.y * 32 * V, f0 = fb + lane * V;
     const int Fp = a.Fp;
-    if (j >= a.N || f0 >= Fp) return;
-    const uint32_t* info = w.info + (size_t)(t - 1) * a.M * Fp;
-    LV<float, V> acc;
-#pragma unroll
-    for (int v = 0; v < V; v++) acc.x[v] = 0.0f;
-    const int q1 = __ldg(a.col_ptr + j + 1);
-#pragma unroll 2
-    for (int q = __ldg(a.col_ptr + j); q < q1; q++) {
-        int i, k;
-        if (PK) {
-            const int slot = __ldg(a.ell_cslot + q);
-            i = slot >> a.dshift;
-            k = slot & ((1 << a.dshift) - 1);
-        } else {
-            i = __ldg(a.col_row + q);
-            k = __ldg(a.col_k + q);
-        }
-        const size_t rv = (a.vrow ? (size_t)__ldg(a.row_ptr + i) : 2 * (size_t)i) * Fp + f0;
-        const LV<uint32_t, V> x = ldv<V>(info + (size_t)i * Fp + f0);
-        const LV<float, V> p1 = ldv<V>(w.eta + rv), p2 = ldv<V>(w.eta + rv + Fp);
-#pragma unroll
-        for (int v = 0; v < V; v++)
-            acc.x[v] += k == info_loc<PK>(x.x[v])    ? p1.x[v]
-                        : k == info_loc2<PK>(x.x[v]) ? p2.x[v]
-                                                     : 0.0f;
+    if (grad) {
+#pragma unroll 4
+        for (int y = warp; y < 32 * V; y += 8)
+            tile.at(lane, y) = (fb + y < F && j0 + lane < a.N) ? grad[(size_t)(fb + y) * a.N + j0 + lane] : 0.0f;
+        __syncthreads();
     }
-    stv<V>(w.ds + (size_t)j * Fp + f0, acc);
+    if (f0 >= Fp) return;
+    const uint32_t* info = w.info + (size_t)(t - 1) * a.M * Fp;
+    for (int b = warp; b < 32 && j0 + b < a.N; b += 8) {
+        const int j = j0 + b;
+        LV<float, V> acc;
+#pragma unroll
+        for (int v = 0; v < V; v++) acc.x[v] = 0.0f;
+        const int q1 = __ldg(a.col_ptr + j + 1);
+#pragma unroll 2
+        for (int q = __ldg(a.col_ptr + j); q < q1; q++) {
+            int i, k;
+            edge_at<PK>(a, q, i, k);
+            const size_t rv = (a.vrow ? (size_t)__ldg(a.row_ptr + i) : 2 * (size_t)i) * Fp + f0;
+            const LV<uint32_t, V> x = ldv<V>(info + (size_t)i * Fp + f0);
+            const LV<float, V> p1 = ldv<V>(w.eta + rv), p2 = ldv<V>(w.eta + rv + Fp);
+#pragma unroll
+            for (int v = 0; v < V; v++)
+                acc.x[v] += k == info_loc<PK>(x.x[v])    ? p1.x[v]
+                            : k == info_loc2<PK>(x.x[v]) ? p2.x[v]
+                                                         : 0.0f;
+        }
+        if (grad) {
+            const LV<float, V> g = tile.get(b, lane);
+#pragma unroll
+            for (int v = 0; v < V; v++) acc.x[v] = acc.x[v] + g.x[v];
+        }
+        stv<V>(w.ds + (size_t)j * Fp + f0, acc);
+    }
 }
 
 // Frames a lane takes: the widest vector (16 bytes) that still gives the GPU eight warps per SM
@@ -420,8 +542,19 @@ int lane_frames(int32_t rows, int32_t Fp, int num_sms, const void* work) {
 }
 
 template <int V, bool PK>
-void launch_bwd(const LwArgs& a, const TrainWork& w, int t, bool last, int num_sms, float* grad_alpha,
-                float* grad_beta, cudaStream_t st) {
+void launch_fwd(const LwArgs& a, const TrainWork& w, int t, float* soft, int frames, bool keep,
+                cudaStream_t st) {
+    const int fb = (a.Fp + 32 * V - 1) / (32 * V);
+    const dim3 gc((a.M + 3) / 4, fb);
+    if (t == 1) k_lw_check<V, true, PK><<<gc, 128, 0, st>>>(a, w, t);
+    else k_lw_check<V, false, PK><<<gc, 128, 0, st>>>(a, w, t);
+    k_lw_var<V, PK><<<dim3((a.N + 31) / 32, fb), 256, 0, st>>>(a, w, t, soft, frames, keep);
+}
+
+// grad_prev (nullable): the loss gradient of the posteriors of iteration t - 1.
+template <int V, bool PK>
+void launch_bwd(const LwArgs& a, const TrainWork& w, int t, bool last, int num_sms, const float* grad_prev,
+                int frames, float* grad_alpha, float* grad_beta, cudaStream_t st) {
     const int fb = (a.Fp + 32 * V - 1) / (32 * V);
     // about 16 blocks an SM (their warps take several rows each)
     const int gx = std::max(1, std::min((a.M + 3) / 4, (16 * num_sms + fb - 1) / fb));
@@ -437,7 +570,7 @@ void launch_bwd(const LwArgs& a, const TrainWork& w, int t, bool last, int num_s
         else if (gm == 1) go(k_lw_bwd_row<V, false, PK, 1>);
         else go(k_lw_bwd_row<V, false, PK, 2>);
     }
-    if (t > 1) k_lw_bwd_col<V, PK><<<dim3((a.N + 3) / 4, fb), 128, 0, st>>>(a, w, t);
+    if (t > 1) k_lw_bwd_col<V, PK><<<dim3((a.N + 31) / 32, fb), 256, 0, st>>>(a, w, t, grad_prev, frames);
 }
 
 bool packed_signs(const HandleView& v) { return v.dg->max_dc <= kPackedSignsMaxRow; }
@@ -498,25 +631,16 @@ int ldpc_train_forward(ldpc_t* h, const float* llr, int32_t frames, int32_t iter
     carve(v.M, v.N, v.E, frames, iters, pk, (char*)work, &w);
     const LwArgs a = make_args(v, w.Fp, alpha, beta);
     cudaStream_t st = v.stream;
-    k_lw_in<<<dim3((v.N + 31) / 32, w.Fp / 32), dim3(32, 8), 0, st>>>(llr, frames, v.N, w.r, w.s, w.Fp);
-    const dim3 gc((v.M + 3) / 4, w.Fp / 32), gv((v.N + 3) / 4, w.Fp / 32);
-    const dim3 go((v.N + 31) / 32, (frames + 31) / 32), bo(32, 8);
+    k_lw_in<<<dim3((v.N + 31) / 32, w.Fp / 32), dim3(32, 8), 0, st>>>(llr, frames, v.N, w.r, w.Fp);
+    const int V = lane_frames(v.M, w.Fp, v.num_sms, work);
+    auto step = V == 4   ? (pk ? launch_fwd<4, true> : launch_fwd<4, false>)
+                : V == 2 ? (pk ? launch_fwd<2, true> : launch_fwd<2, false>)
+                         : (pk ? launch_fwd<1, true> : launch_fwd<1, false>);
     int launches = 1;
     for (int t = 1; t <= iters; t++) {
-        if (pk) {
-            if (t == 1) k_lw_check<true, true><<<gc, 128, 0, st>>>(a, w, t);
-            else k_lw_check<false, true><<<gc, 128, 0, st>>>(a, w, t);
-        } else {
-            if (t == 1) k_lw_check<true, false><<<gc, 128, 0, st>>>(a, w, t);
-            else k_lw_check<false, false><<<gc, 128, 0, st>>>(a, w, t);
-        }
-        k_lw_var<<<gv, 128, 0, st>>>(a, w);
+        float* out = soft_every ? soft + (size_t)(t - 1) * frames * v.N : t == iters ? soft : nullptr;
+        step(a, w, t, out, frames, t < iters, st);
         launches += 2;
-        if (soft_every || t == iters) {
-            k_lw_out<<<go, bo, 0, st>>>(w.s, w.Fp, v.N, frames,
-                                        soft + (soft_every ? (size_t)(t - 1) * frames * v.N : 0));
-            launches++;
-        }
     }
     *v.last_launches = launches;
     return cudaGetLastError() == cudaSuccess ? LDPC_OK : LDPC_ERR_CUDA;
@@ -543,20 +667,16 @@ int ldpc_train_backward(ldpc_t* h, int32_t frames, int32_t iters, const float* a
     const size_t plane = (size_t)frames * v.N;
     // ds^T = the loss gradient of the last posteriors
     k_lw_in<<<gi, bi, 0, st>>>(grad_soft + (soft_every ? (size_t)(iters - 1) * plane : 0), frames,
-                               v.N, w.ds, nullptr, w.Fp);
+                               v.N, w.ds, w.Fp);
     const int V = lane_frames(v.M, w.Fp, v.num_sms, work);
     int launches = 1;
     for (int t = iters; t >= 1; t--) {
         auto step = V == 4   ? (pk ? launch_bwd<4, true> : launch_bwd<4, false>)
                     : V == 2 ? (pk ? launch_bwd<2, true> : launch_bwd<2, false>)
                              : (pk ? launch_bwd<1, true> : launch_bwd<1, false>);
-        step(a, w, t, t == iters, v.num_sms, grad_alpha, grad_beta, st);
+        step(a, w, t, t == iters, v.num_sms, soft_every && t > 1 ? grad_soft + (size_t)(t - 2) * plane : nullptr,
+             frames, grad_alpha, grad_beta, st);
         launches += t > 1 ? 2 : 1;
-        if (t > 1 && soft_every) {  // plus the loss gradient of the posteriors of iteration t-1
-            k_lw_in<<<gi, bi, 0, st>>>(grad_soft + (size_t)(t - 2) * plane, frames, v.N, w.ds, nullptr,
-                                       w.Fp, 1);
-            launches++;
-        }
     }
     *v.last_launches = launches;
     return cudaGetLastError() == cudaSuccess ? LDPC_OK : LDPC_ERR_CUDA;
