@@ -163,6 +163,7 @@ static void apply_staging(const ldpc_t* h, StreamWork& w) {
     w.stage_warps = stage_warps_of(h);
     w.stages = h->st_stages < 0 ? 0 : (h->st_stages > 0 ? h->st_stages : kStagesDefault);
     w.stage_vw = h->st_vw;
+    w.auto_staging = h->st_warps == 0 && h->st_stages == 0 && h->st_vw == 0;
     w.wait_limit = h->wait_limit;
     w.msg_compressed = h->st_msg;
 }
@@ -427,6 +428,7 @@ int ldpc_impl::handle_view(ldpc_t* h, HandleView* v) {
     v->stage_warps = stage_warps_of(h);
     v->stages = h->st_stages < 0 ? 0 : (h->st_stages > 0 ? h->st_stages : kStagesDefault);
     v->stage_vw = h->st_vw;
+    v->auto_staging = h->st_warps == 0 && h->st_stages == 0 && h->st_vw == 0;
     v->wait_limit = h->wait_limit;
     v->msg_compressed = h->st_msg;
     return LDPC_OK;
@@ -582,12 +584,15 @@ int ldpc_decode_ex(ldpc_t* h, const void* llr, int32_t llr_dtype, int32_t frames
                 n = k < 0 ? k : n + k;
             }
         } else {
-            int rc = ensure_stream_work(h, frames, max_iter);
+            apply_staging(h, h->sw);
+            const int vw = stream_lane_frames(h->dg, frames, h->sw);
+            int rc = ensure_stream_work(h, frames, max_iter, vw ? 32 * vw : 256);
             if (rc != LDPC_OK) return rc;
             int32_t used_cmp = 0;
             StreamWork w = h->sw;
+            stream_narrow(w, frames, vw);
             w.used_compressed = &used_cmp;
-            n = stream_decode(h->mode, h->dg, a, w, h->stream);
+            n = stream_decode(h->mode, h->dg, a, w, h->stream, vw);
             if (n >= 0 && !a.early_stop) {  // no compaction: position = frame
                 h->msg_frames = frames;
                 h->msg_mode = h->mode;
@@ -793,8 +798,9 @@ static int autotune_stream(ldpc_t* h, int32_t frames, int32_t max_iter, float* b
     const int32_t keep[3] = {h->st_warps, h->st_stages, h->st_vw};
     // (warps, stages, frames per lane): full and half-width lanes (half-width stages let rows
     // of 16 slots fit more warps), and the unstaged kernel
-    // (shapes whose shared memory does not fit run the unstaged kernel and lose)
-    static const int32_t shapes[][3] = {{8, 3, 0}, {12, 2, 0}, {6, 3, 0}, {4, 4, 0}, {8, 2, 0},
+    // (shapes whose shared memory does not fit run the unstaged kernel and lose); first the
+    // automatic choice, which small batches run with narrow lanes
+    static const int32_t shapes[][3] = {{0, 0, 0}, {8, 3, 0}, {12, 2, 0}, {6, 3, 0}, {4, 4, 0}, {8, 2, 0},
                                         {12, 3, 0}, {8, 4, 0}, {4, 2, 0}, {6, 2, 0}, {12, 2, 2},
                                         {8, 3, 2}, {0, -1, 0}};
     constexpr int n_shapes = (int)(sizeof(shapes) / sizeof(shapes[0]));

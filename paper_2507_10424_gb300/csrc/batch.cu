@@ -185,7 +185,10 @@ static int batch_enqueue(ldpc_batch_t* b) {
         for (size_t k = 0; k < b->streamed.size(); k++) {
             const auto& x = b->streamed[k];
             if (x.a.frames == 0) continue;
-            const int n = stream_decode(kModeFP32, *b->views[x.code].dg, x.a, x.w, (k & 1) ? b->side2 : b->side);
+            StreamWork w = x.w;
+            const int vw = stream_lane_frames(*b->views[x.code].dg, x.a.frames, w);
+            stream_narrow(w, x.a.frames, vw);
+            const int n = stream_decode(kModeFP32, *b->views[x.code].dg, x.a, w, (k & 1) ? b->side2 : b->side, vw);
             if (n < 0) return n;
             launches += n;
         }
@@ -376,6 +379,7 @@ int ldpc_batch_prepare(ldpc_batch_t* b, int32_t max_iter, int32_t early_stop) {
             x.w.stage_warps = v.stage_warps;
             x.w.stages = v.stages;
             x.w.stage_vw = v.stage_vw;
+            x.w.auto_staging = v.auto_staging;
             x.w.wait_limit = v.wait_limit;
             x.w.msg_compressed = v.msg_compressed;
             DecodeArgs& a = x.a;

@@ -216,6 +216,7 @@ struct StreamWork {
     int32_t* err = nullptr;
     int32_t stage_warps = 0, stages = 0;
     int32_t stage_vw = 0;  // frames per lane of the staged kernel (0: the run's vector width)
+    int32_t auto_staging = 0;  // no shape was asked for: small batches may take narrow lanes
     uint32_t wait_limit = 1u << 16;
     int32_t num_sms = 0;
     // FP32 codes on the padded row layout: keep each row's messages compressed (min0,
@@ -238,6 +239,13 @@ inline size_t staged_smem_bytes(int mode, int vw, int D, bool cmp, int warps, in
     const size_t meta = (size_t)32 * 4 + (size_t)D * 4;
     return (size_t)warps * stages * (stage + meta + 8) + (weights ? (size_t)2 * 256 * 4 : 0);
 }
+
+// Frames a lane takes in the streaming passes of a batch: 0 = the full 16-byte vector of the
+// mode on a frame stride of whole 256-frame blocks, else 1 or 2 frames with the register
+// kernels and per-edge messages, on a stride of whole 32- or 64-frame blocks.
+int stream_lane_frames(const DevGraph& g, int32_t frames, const StreamWork& w);
+// Sets w's frame stride, staging and message format for lanes of vw frames.
+void stream_narrow(StreamWork& w, int32_t frames, int vw);
 
 // Launchers; return the number of kernels enqueued, or a negative status.
 // vw: frames per lane (0: a 16-byte vector, 4 fp32 / 8 int16; else 1, 2, 4 or 8 with the
@@ -306,6 +314,7 @@ struct HandleView {
     int32_t* err = nullptr;  // device error word of the handle
     int32_t stage_warps = 0, stages = 0;  // staged streaming check pass (stages 0 = off)
     int32_t stage_vw = 0;
+    int32_t auto_staging = 0;
     uint32_t wait_limit = 0;
     int32_t msg_compressed = 1;  // ldpc_set_stream_messages
 };

@@ -128,6 +128,7 @@ extern "C" int ldpc_decode_noalloc(ldpc_t* h, const void* llr, int32_t llr_dtype
     w.stage_warps = v.stage_warps;
     w.stages = v.stages;
     w.stage_vw = v.stage_vw;
+    w.auto_staging = v.auto_staging;
     w.wait_limit = v.wait_limit;
     w.msg_compressed = v.msg_compressed;
     DecodeArgs a;
@@ -152,7 +153,9 @@ extern "C" int ldpc_decode_noalloc(ldpc_t* h, const void* llr, int32_t llr_dtype
         a.w_beta = v.w_alpha + (size_t)v.w_rows * v.dg->n_classes;
     }
     // the kernels clear the done counter and the syndrome flags and set the frame state
-    const int n = stream_decode(v.mode, *v.dg, a, w, v.stream);
+    const int vw = stream_lane_frames(*v.dg, frames, w);
+    stream_narrow(w, frames, vw);
+    const int n = stream_decode(v.mode, *v.dg, a, w, v.stream, vw);
     if (n < 0) {  // a failed launch leaves its error pending: clear it and report it
         const cudaError_t e = cudaGetLastError();
         return e != cudaSuccess ? LDPC_ERR_CUDA : n;

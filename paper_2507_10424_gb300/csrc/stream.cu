@@ -12,6 +12,29 @@ namespace ldpc_impl {
 int stream_decode_fp32(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_t st, int vw);
 int stream_decode_fixed(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_t st, int vw);
 
+// Few frames: a 16-byte lane vector makes blocks of 128 (FP32) or 256 (fixed point) frames that
+// are mostly padding, and the staged pass's pipeline has nothing to overlap; the passes are
+// then chains of dependent loads, which the register kernels on one or two frames a lane
+// shorten (a row's, or four of a column's, messages requested together). Measured, 20
+// iterations, full vectors / one frame / two frames a lane, us a decode:
+//   32 frames: N=576 282 / 190 / 194, N=16200 (rows of 20-21) 722 / 360 / 434, N=64800 1484 /
+//     797 / 893;
+//   64 frames: N=12288 493 / 458 / 375, N=16200 732 / 529 / 465, N=64800 1529 / 1425 / 1047;
+//   128 frames: N=12288 503 / 692 / 536, N=64800 1631 / 2737 / 2066, but N=16200 792 / 869 /
+//     659: rows of more than 16 edges have no staged pass.
+int stream_lane_frames(const DevGraph& g, int32_t frames, const StreamWork& w) {
+    if (!w.auto_staging) return 0;
+    if (frames <= 32) return 1;
+    return frames <= (g.ell_D == 0 && g.max_dc <= 32 ? 128 : 64) ? 2 : 0;
+}
+
+void stream_narrow(StreamWork& w, int32_t frames, int vw) {
+    if (!vw) return;
+    w.Fp = (frames + 32 * vw - 1) / (32 * vw) * (32 * vw);
+    w.stages = 0;
+    w.msg_compressed = 0;
+}
+
 size_t stream_bytes(int mode, int32_t N, int64_t slots, int32_t Fp, int32_t L) {
     size_t tb = mode == kModeFP32 ? 4 : 2, rb = mode == kModeFP32 ? 4 : 1;
     return (size_t)slots * Fp * tb + (size_t)N * Fp * (tb + rb) + (size_t)N * (Fp / 4) + (size_t)Fp * 13 +

@@ -56,6 +56,14 @@ __device__ __forceinline__ float lam_of(float s, float e) { return s - e; }
 __device__ __forceinline__ int32_t lam_of(int32_t s, int32_t e) { return sat16(s - e); }
 __device__ __forceinline__ float absval(float x) { return fabsf(x); }
 __device__ __forceinline__ int32_t absval(int32_t x) { return abs(x); }
+// max for the second minimum: NaN when b is NaN, so that a NaN magnitude (infinite channel
+// values can produce one) leaves both minima as they are.
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ int32_t max_nan(int32_t a, int32_t b) { return max(a, b); }
 __device__ __forceinline__ float big(float) { return __int_as_float(0x7f800000); }
 __device__ __forceinline__ int32_t big(int32_t) { return 0x7fffffff; }
 template <typename A>
@@ -440,6 +448,20 @@ __device__ __forceinline__ VT ld_nc(const VT* p) {
     return v;
 }
 
+// The D columns of a padded row (16-byte loads).
+template <int D>
+__device__ __forceinline__ void load_cols(const int32_t* __restrict__ p, int (&c)[D]) {
+    static_assert(D % 4 == 0, "columns load as 16-byte vectors");
+#pragma unroll
+    for (int q = 0; q < D / 4; q++) {
+        const int4 v = __ldg(reinterpret_cast<const int4*>(p) + q);
+        c[4 * q] = v.x;
+        c[4 * q + 1] = v.y;
+        c[4 * q + 2] = v.z;
+        c[4 * q + 3] = v.w;
+    }
+}
+
 template <int MODE, int VW>
 struct RowVec {  // per-frame values
     using VT = Vec<typename Tr<MODE>::T, VW>;
@@ -525,7 +547,7 @@ __device__ __forceinline__ uint32_t row_update(Row& row, int d, typename Tr<MODE
                     if (SYN) zx[v] ^= PAPER ? sbits(A(0) - sa) : sbits(sa);
                     const A l = FIRST ? sa : lam_of(sa, (A)ev.x[v]);
                     const A m = absval(l);
-                    min1[v] = min(min1[v], max(min0[v], m));
+                    min1[v] = min(min1[v], max_nan(min0[v], m));
                     min0[v] = min(min0[v], m);
                     sx[v] ^= sbits(l);
                     lv.x[v] = (T)l;  // exact: lambda is saturated to the storage range
@@ -606,9 +628,12 @@ __device__ __forceinline__ uint32_t row_update(Row& row, int d, typename Tr<MODE
     return z;
 }
 
-template <int MODE, bool FIRST, bool W, int VW, int D>
+// CSR: the same on CSR order (rows of at most D edges; slots are CSR edge ids), one round trip
+// more, for the row's offset.
+template <int MODE, bool FIRST, bool W, int VW, int D, bool CSR = false>
 __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
-    k_check_ell(const int32_t* __restrict__ ell_col, const uint8_t* __restrict__ ell_deg, int M,
+    k_check_row(const int32_t* __restrict__ col, const uint8_t* __restrict__ ell_deg,
+                const int32_t* __restrict__ row_ptr, int M,
                 const typename Tr<MODE>::T* __restrict__ s, typename Tr<MODE>::T* __restrict__ eta,
                 int Fp, const uint8_t* __restrict__ state, uint8_t* __restrict__ unsat, int do_syn,
                 int paper, IterWeights wt = IterWeights()) {
@@ -616,28 +641,29 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
     using VT = typename RowVec<MODE, VW>::VT;
     using VS = Vec<uint8_t, VW>;
     static_assert(sizeof(VT) == sizeof(T) * VW, "one vector = VW frames");
-    static_assert(D % 4 == 0, "columns load as 16-byte vectors");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 4 + warp;
     const int f0 = (blockIdx.y * 32 + lane) * VW;
     if (i >= M) return;
     const VS st = *reinterpret_cast<const VS*>(state + f0);
-    const int d = __ldg(ell_deg + i);
-    int c[D];
+    int d, c[D];
+    size_t e0;
+    if constexpr (CSR) {
+        e0 = (size_t)__ldg(row_ptr + i);
+        d = __ldg(row_ptr + i + 1) - (int)e0;
 #pragma unroll
-    for (int q = 0; q < D / 4; q++) {
-        const int4 v = __ldg(reinterpret_cast<const int4*>(ell_col + (size_t)i * D) + q);
-        c[4 * q] = v.x;
-        c[4 * q + 1] = v.y;
-        c[4 * q + 2] = v.z;
-        c[4 * q + 3] = v.w;
+        for (int t = 0; t < D; t++) c[t] = t < d ? __ldg(col + e0 + t) : 0;
+    } else {
+        e0 = (size_t)i * D;
+        d = __ldg(ell_deg + i);
+        load_cols<D>(col + e0, c);
     }
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < VW; v++) act |= (uint32_t)(st.x[v] != 0) << v;
     if (!act) return;
 
-    T* const erow = eta + (size_t)i * D * Fp + f0;
+    T* const erow = eta + e0 * Fp + f0;
     RegRow<VT, D> row;
     row.cols = c;
 #pragma unroll
@@ -657,9 +683,10 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
 // Final syndrome pass on the padded row layout (status of frames that never stopped): the
 // XOR of the decisions of a row's bits (eq. 1-2), every load of the row issued at once.
 // ------------------------------------------------------------------------------------
-template <int MODE, int VW, int D>
-__global__ void __launch_bounds__(128) k_syn_ell(const int32_t* __restrict__ ell_col,
-                                                 const uint8_t* __restrict__ ell_deg, int M,
+template <int MODE, int VW, int D, bool CSR = false>
+__global__ void __launch_bounds__(128) k_syn_row(const int32_t* __restrict__ col,
+                                                 const uint8_t* __restrict__ ell_deg,
+                                                 const int32_t* __restrict__ row_ptr, int M,
                                                  const typename Tr<MODE>::T* __restrict__ s, int Fp,
                                                  const uint8_t* __restrict__ state,
                                                  uint8_t* __restrict__ unsat, int paper) {
@@ -671,15 +698,15 @@ __global__ void __launch_bounds__(128) k_syn_ell(const int32_t* __restrict__ ell
     const int f0 = (blockIdx.y * 32 + lane) * VW;
     if (i >= M) return;
     const VS st = *reinterpret_cast<const VS*>(state + f0);
-    const int d = __ldg(ell_deg + i);
-    int c[D];
+    int d, c[D];
+    if constexpr (CSR) {
+        const int e0 = __ldg(row_ptr + i);
+        d = __ldg(row_ptr + i + 1) - e0;
 #pragma unroll
-    for (int q = 0; q < D / 4; q++) {
-        const int4 v = __ldg(reinterpret_cast<const int4*>(ell_col + (size_t)i * D) + q);
-        c[4 * q] = v.x;
-        c[4 * q + 1] = v.y;
-        c[4 * q + 2] = v.z;
-        c[4 * q + 3] = v.w;
+        for (int t = 0; t < D; t++) c[t] = t < d ? __ldg(col + e0 + t) : 0;
+    } else {
+        d = __ldg(ell_deg + i);
+        load_cols<D>(col + (size_t)i * D, c);
     }
     uint32_t act = 0;
 #pragma unroll
@@ -1093,6 +1120,13 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
     using VR = Vec<R, V>;
     using VS = Vec<uint8_t, V>;
     const VS st = *reinterpret_cast<const VS*>(state + f0);
+    int t0, t1;
+    VR rv;
+    if constexpr (V <= 2) {  // one round trip less
+        t0 = __ldg(col_ptr + j);
+        t1 = __ldg(col_ptr + j + 1);
+        rv = *reinterpret_cast<const VR*>(r + (size_t)j * Fp + f0);
+    }
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
@@ -1116,8 +1150,11 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
         }
     }
     if (!upd) return;
-    const int t0 = __ldg(col_ptr + j), t1 = __ldg(col_ptr + j + 1);
-    const VR rv = *reinterpret_cast<const VR*>(r + (size_t)j * Fp + f0);
+    if constexpr (V > 2) {
+        t0 = __ldg(col_ptr + j);
+        t1 = __ldg(col_ptr + j + 1);
+        rv = *reinterpret_cast<const VR*>(r + (size_t)j * Fp + f0);
+    }
     A acc[V];
 #pragma unroll
     for (int v = 0; v < V; v++) acc[v] = (A)rv.x[v];
@@ -1148,6 +1185,24 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
                 if constexpr (W) m = cmsg_weight(m, wa, wb);
                 acc[v] = acc[v] + (A)cmsg_signed(m, w.x[v], tp);
             }
+        }
+    } else if constexpr (V <= 2) {
+        // few frames: the pass is one chain of dependent loads, so four messages are
+        // gathered at once (the registers are there: one or two frames a lane)
+        constexpr int U = 4;
+        for (int q = t0; q < t1; q += U) {
+            int e[U];
+            VT ev[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) e[u] = __ldg(col_edge + min(q + u, t1 - 1));
+#pragma unroll
+            for (int u = 0; u < U; u++) ev[u] = ld_nc(reinterpret_cast<const VT*>(eta + (size_t)e[u] * Fp + f0));
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (q + u < t1) {
+#pragma unroll
+                    for (int v = 0; v < V; v++) acc[v] = acc[v] + (A)ev[u].x[v];
+                }
         }
     } else if constexpr (MODE == kModeFixed && V % 2 == 0) {
         // int16 pairs: each lane of a word added by one two-way dot product (dp2a)
@@ -1211,7 +1266,7 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
 // (CTAs that loop over strided tasks drift apart: 20 % slower on the N=64800 code); with
 // per-edge messages the looping form measured 1.7 % slower on the QC N=2304 code.
 template <int MODE, int VW = Tr<MODE>::V, bool CMP = false, bool W = false, bool HD = false>
-__global__ void __launch_bounds__(128, 16) k_var(const int32_t* __restrict__ col_ptr,
+__global__ void __launch_bounds__(128, VW <= 2 ? 8 : 16) k_var(const int32_t* __restrict__ col_ptr,
                                              const int32_t* __restrict__ col_edge, int N,
                                              const typename Tr<MODE>::R* __restrict__ r,
                                              typename Tr<MODE>::T* s,
@@ -1528,15 +1583,22 @@ void check_pass_t(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, d
     const int Fp = w.Fp;
     if (g.ell_D == 8) {
         if (staged<MODE, V, FIRST, W, 8>(g, a, w, s, eta, un, test_prev, wt, st)) return;
-        k_check_ell<MODE, FIRST, W, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, eta, Fp,
+        k_check_row<MODE, FIRST, W, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, eta, Fp,
                                                               w.state, un, test_prev, a.paper_slicer, wt);
         return;
     }
     if (g.ell_D == 16) {
         if (staged<MODE, V, FIRST, W, 16>(g, a, w, s, eta, un, test_prev, wt, st)) return;
-        k_check_ell<MODE, FIRST, W, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, eta, Fp,
+        k_check_row<MODE, FIRST, W, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, eta, Fp,
                                                                w.state, un, test_prev, a.paper_slicer, wt);
         return;
+    }
+    if constexpr (V <= 2) {
+        if (g.max_dc <= 32) {
+            k_check_row<MODE, FIRST, W, V, 32, true><<<gc, 128, 0, st>>>(
+                g.col_idx, nullptr, g.row_ptr, a.M, s, eta, Fp, w.state, un, test_prev, a.paper_slicer, wt);
+            return;
+        }
     }
     k_check<MODE, FIRST, false, W, V><<<gc, 128, 0, st>>>(g.row_ptr, g.col_idx, a.M, s, eta, Fp,
                                                           w.state, un, test_prev, w.n_done, a.frames,
@@ -1657,6 +1719,8 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
         }
         return wt;
     };
+    // a batch of one frame block has no block to free: its frames stop in place
+    const bool may_compact = a.early_stop && w.comp && a.frames > 32 * V;
     for (int k = 1; k <= a.L; k++) {
         const int test_prev = a.early_stop && ((k - 1) % a.check_every == 0);
         uint8_t* un = w.unsat + (size_t)k * Fp;
@@ -1679,7 +1743,7 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
                         var_pass<MODE, V, true, false>(g, a, w, gv, g.ell_cslot, un, test_prev, k, hd && k == a.L,
                                                        cs, dshift, wt, st);
                     launches += 2;
-                    if (a.early_stop && k < a.L && k % kCompactEvery == 0 && w.comp)
+                    if (may_compact && k < a.L && k % kCompactEvery == 0)
                         launches += compact<MODE>(g, a, w, st, true);
                     continue;
                 }
@@ -1691,7 +1755,7 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
         var_pass<MODE, V, false, false>(g, a, w, gv, cslot, un, test_prev, k, hd && k == a.L, CState{}, 0,
                                         IterWeights(), st);
         launches += 2;
-        if (a.early_stop && k < a.L && k % kCompactEvery == 0 && w.comp)
+        if (may_compact && k < a.L && k % kCompactEvery == 0)
             launches += compact<MODE>(g, a, w, st, false);
     }
     if (w.used_compressed) *w.used_compressed = cmp ? 1 : 0;
@@ -1713,12 +1777,16 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
     if (!syn_done) {
         if (g.ell_D == 8) {
             if (!launch_staged<MODE, V, true, false, 8, true>(g, a, w, s, eta, unf, 1, IterWeights(), st))
-                k_syn_ell<MODE, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf,
-                                                          a.paper_slicer);
+                k_syn_row<MODE, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, Fp, state,
+                                                          unf, a.paper_slicer);
         } else if (g.ell_D == 16) {
             if (!launch_staged<MODE, V, true, false, 16, true>(g, a, w, s, eta, unf, 1, IterWeights(), st))
-                k_syn_ell<MODE, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf,
-                                                           a.paper_slicer);
+                k_syn_row<MODE, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, Fp, state,
+                                                           unf, a.paper_slicer);
+        } else if (V <= 2 && g.max_dc <= 32) {
+            if constexpr (V <= 2)
+                k_syn_row<MODE, V, 32, true><<<gc, 128, 0, st>>>(g.col_idx, nullptr, g.row_ptr, a.M, s, Fp,
+                                                                 state, unf, a.paper_slicer);
         } else
             k_check<MODE, false, true, false, V><<<gc, 128, 0, st>>>(g.row_ptr, g.col_idx, a.M, s, eta, Fp,
                                                                      state, unf, 1, w.n_done, a.frames,
