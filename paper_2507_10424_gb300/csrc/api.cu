@@ -70,7 +70,7 @@ struct ldpc {
     StreamWork sw;
     int32_t sw_cap = 0, sw_cap_L = -1;
     void* sw_big = nullptr;
-    uint8_t* sw_unsat = nullptr;
+    uint32_t* sw_unsat = nullptr;
     void* dense_work = nullptr;  // dense variant workspace
     size_t dense_cap = 0;
     int32_t stream_group = -1;   // streaming: -1 no frame groups, 0 L2-sized groups, > 0 group size
@@ -214,7 +214,7 @@ static int ensure_stream_work(ldpc_t* h, int32_t frames, int32_t L, int32_t gran
             cudaFree(h->sw_unsat);
             h->sw_unsat = nullptr;
         }
-        cudaError_t e = cudaMalloc((void**)&h->sw_unsat, (size_t)(L + 2) * h->sw_cap);
+        cudaError_t e = cudaMalloc((void**)&h->sw_unsat, (size_t)(L + 2) * (h->sw_cap / 32) * 4);
         if (e != cudaSuccess) {
             h->sw_unsat = nullptr;
             h->sw_cap_L = -1;

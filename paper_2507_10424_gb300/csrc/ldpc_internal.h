@@ -205,7 +205,7 @@ struct StreamWork {
     int32_t* pos2frame = nullptr;  // [Fp]
     int32_t* new_pos = nullptr;    // [Fp]
     int32_t* comp = nullptr;       // [4]
-    uint8_t* unsat = nullptr;      // [(L+2)][Fp]
+    uint32_t* unsat = nullptr;     // [(L+2)][Fp / 32]: bit p of word p / 32, position p fails a check
     int32_t* n_done = nullptr;     // [1]
     // decisions of the last bit pass, one byte per lane of 4 or 8 frames: [N][Fp / 4] bytes
     // (nullable: the final syndrome and the output bits are then taken from s)

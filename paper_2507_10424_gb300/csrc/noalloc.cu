@@ -118,7 +118,7 @@ extern "C" int ldpc_decode_noalloc(ldpc_t* h, const void* llr, int32_t llr_dtype
     w.r = base + o_r;
     w.done_iter = (int32_t*)(base + o_done);
     w.state = (uint8_t*)(base + o_state);
-    w.unsat = (uint8_t*)(base + o_unsat);
+    w.unsat = (uint32_t*)(base + o_unsat);
     w.n_done = (int32_t*)(base + o_count);
     w.pos2frame = (int32_t*)(base + o_p2f);
     w.new_pos = (int32_t*)(base + o_newpos);

@@ -63,7 +63,7 @@ StreamWork stream_carve(int mode, void* mem, int32_t N, int64_t slots, int32_t F
     p += (size_t)Fp * 4;
     w.state = (uint8_t*)p;
     p += (size_t)Fp;
-    w.unsat = (uint8_t*)p;
+    w.unsat = (uint32_t*)p;
     p += (size_t)(L + 2) * Fp;
     w.n_done = (int32_t*)p;  // the last 256 bytes: counters
     w.err = w.n_done + 1;

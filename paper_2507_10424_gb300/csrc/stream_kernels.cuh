@@ -79,22 +79,23 @@ __device__ __forceinline__ int8_t quantize(float x) {
     return (int8_t)__float2int_rn(t);
 }
 
-// Mark frames f0 + v (bit v of z) as having an unsatisfied check. Every check of a frame
-// reports to the same byte, so the flags are read first and only the missing ones are
-// written: after the first failing row, the other rows find the byte set and leave it
-// (tens of thousands of stores to the same few L2 lines otherwise serialise the pass).
+// Unsatisfied checks, one bit per position: bit p % 32 of word p / 32. Every check of a frame
+// reports to the same bit, so a warp first brings the bits of its 32 VW positions together in
+// VW words, and its leading lanes set only the bits that `have`, the word read earlier, does
+// not show: after the first failing rows the others find theirs set. (Byte flags, written
+// lane by lane, serialised the pass on a few L2 lines. Check pass with the syndrome, us a
+// launch, bytes against bits: N=12288, 64 frames, 48 against 11; N=64800 in fixed point, 1000
+// frames, 337 against 208.)
+// z: bit v = position f0 + v, f0 = (32 y + lane) VW; all lanes of the warp take part.
 template <int VW>
-__device__ __forceinline__ void flag_unsat(uint8_t* unsat, int f0, uint32_t z) {
-    if (!z) return;
-    uint32_t have = 0;
+__device__ __forceinline__ void flag_unsat(uint32_t* unsat, int f0, uint32_t z, uint32_t have) {
+    uint32_t x = z << (f0 & 31);
 #pragma unroll
-    for (int v = 0; v < VW; v++) have |= (uint32_t)(((volatile const uint8_t*)unsat)[f0 + v] != 0) << v;
-    const uint32_t need = z & ~have;
-    if (need) {
-#pragma unroll
-        for (int v = 0; v < VW; v++)
-            if ((need >> v) & 1) unsat[f0 + v] = 1;
-    }
+    for (int o = 1; o < 32 / VW; o <<= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
+    if ((x & ~have) && (threadIdx.x & (32 / VW - 1)) == 0) atomicOr(unsat + (f0 >> 5), x);
+}
+__device__ __forceinline__ uint32_t unsat_now(const uint32_t* unsat, int f0) {
+    return __ldcg(unsat + (f0 >> 5));
 }
 
 // ------------------------------------------------------------------------------------
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(128) k_check(const int32_t* __restrict__ row_p
                                                const int32_t* __restrict__ col_idx, int M,
                                                const typename Tr<MODE>::T* __restrict__ s,
                                                typename Tr<MODE>::T* eta, int Fp,
-                                               const uint8_t* __restrict__ state, uint8_t* unsat,
+                                               const uint8_t* __restrict__ state, uint32_t* unsat,
                                                int do_syn, const int* n_done, int frames,
                                                int paper, IterWeights wt = IterWeights()) {
     using T = typename Tr<MODE>::T;
@@ -332,12 +333,13 @@ __global__ void __launch_bounds__(128) k_check(const int32_t* __restrict__ row_p
     if (i >= M) return;
     if (*(volatile const int*)n_done >= frames) return;
     const VS st = *reinterpret_cast<const VS*>(state + f0);
+    const uint32_t have = do_syn ? unsat_now(unsat, f0) : 0u;
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
-    if (!act) return;
+    if (!__any_sync(0xffffffffu, act != 0)) return;
 
-    const int e0 = __ldg(row_ptr + i), d = __ldg(row_ptr + i + 1) - e0;
+    const int e0 = __ldg(row_ptr + i), d = act ? __ldg(row_ptr + i + 1) - e0 : 0;
     A min0[V], min1[V];
     int loc[V];
     uint32_t msk[V];
@@ -378,7 +380,7 @@ __global__ void __launch_bounds__(128) k_check(const int32_t* __restrict__ row_p
         }
         if (!SYN_ONLY && longrow) *reinterpret_cast<VT*>(ep) = lv;  // stash lambda in place
     }
-    if (do_syn) flag_unsat<V>(unsat, f0, z & act);
+    if (do_syn) flag_unsat<V>(unsat, f0, z & act, have);
     if constexpr (!SYN_ONLY) {
     for (int t = 0; t < d; t++) {
         T* ep = eta + (size_t)(e0 + t) * Fp + f0;
@@ -635,7 +637,7 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
     k_check_row(const int32_t* __restrict__ col, const uint8_t* __restrict__ ell_deg,
                 const int32_t* __restrict__ row_ptr, int M,
                 const typename Tr<MODE>::T* __restrict__ s, typename Tr<MODE>::T* __restrict__ eta,
-                int Fp, const uint8_t* __restrict__ state, uint8_t* __restrict__ unsat, int do_syn,
+                int Fp, const uint8_t* __restrict__ state, uint32_t* unsat, int do_syn,
                 int paper, IterWeights wt = IterWeights()) {
     using T = typename Tr<MODE>::T;
     using VT = typename RowVec<MODE, VW>::VT;
@@ -658,25 +660,27 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
         d = __ldg(ell_deg + i);
         load_cols<D>(col + e0, c);
     }
+    const uint32_t have = do_syn ? unsat_now(unsat, f0) : 0u;
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < VW; v++) act |= (uint32_t)(st.x[v] != 0) << v;
-    if (!act) return;
-
-    T* const erow = eta + e0 * Fp + f0;
-    RegRow<VT, D> row;
-    row.cols = c;
-#pragma unroll
-    for (int t = 0; t < D; t++)
-        if (t < d) {
-            row.sv[t] = ld_nc(reinterpret_cast<const VT*>(s + (size_t)c[t] * Fp + f0));
-            if (!FIRST) row.ev[t] = *reinterpret_cast<const VT*>(erow + (size_t)t * Fp);
-        }
     uint32_t z = 0;
-    if (!do_syn) z = row_update<MODE, FIRST, false, false, W, VW, D>(row, d, erow, Fp, wt);
-    else if (!paper) z = row_update<MODE, FIRST, true, false, W, VW, D>(row, d, erow, Fp, wt);
-    else z = row_update<MODE, FIRST, true, true, W, VW, D>(row, d, erow, Fp, wt);
-    if (do_syn) flag_unsat<VW>(unsat, f0, z & act);
+    if (act) {  // lanes whose frames have all stopped touch nothing
+        T* const erow = eta + e0 * Fp + f0;
+        RegRow<VT, D> row;
+        row.cols = c;
+#pragma unroll
+        for (int t = 0; t < D; t++)
+            if (t < d) {
+                row.sv[t] = ld_nc(reinterpret_cast<const VT*>(s + (size_t)c[t] * Fp + f0));
+                if (!FIRST) row.ev[t] = *reinterpret_cast<const VT*>(erow + (size_t)t * Fp);
+            }
+        if (!do_syn) z = row_update<MODE, FIRST, false, false, W, VW, D>(row, d, erow, Fp, wt);
+        else if (!paper) z = row_update<MODE, FIRST, true, false, W, VW, D>(row, d, erow, Fp, wt);
+        else z = row_update<MODE, FIRST, true, true, W, VW, D>(row, d, erow, Fp, wt);
+    }
+    __syncwarp();
+    if (do_syn) flag_unsat<VW>(unsat, f0, z & act, have);
 }
 
 // ------------------------------------------------------------------------------------
@@ -689,7 +693,7 @@ __global__ void __launch_bounds__(128) k_syn_row(const int32_t* __restrict__ col
                                                  const int32_t* __restrict__ row_ptr, int M,
                                                  const typename Tr<MODE>::T* __restrict__ s, int Fp,
                                                  const uint8_t* __restrict__ state,
-                                                 uint8_t* __restrict__ unsat, int paper) {
+                                                 uint32_t* unsat, int paper) {
     using A = typename Tr<MODE>::A;
     using VT = Vec<typename Tr<MODE>::T, VW>;
     using VS = Vec<uint8_t, VW>;
@@ -711,19 +715,22 @@ __global__ void __launch_bounds__(128) k_syn_row(const int32_t* __restrict__ col
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < VW; v++) act |= (uint32_t)(st.x[v] != 0) << v;
-    if (!act) return;
-    VT sv[D];
-#pragma unroll
-    for (int t = 0; t < D; t++)
-        if (t < d) sv[t] = ld_nc(reinterpret_cast<const VT*>(s + (size_t)c[t] * Fp + f0));
+    const uint32_t have = unsat_now(unsat, f0);
     uint32_t z = 0;
+    if (act) {
+        VT sv[D];
 #pragma unroll
-    for (int t = 0; t < D; t++)
-        if (t < d) {
+        for (int t = 0; t < D; t++)
+            if (t < d) sv[t] = ld_nc(reinterpret_cast<const VT*>(s + (size_t)c[t] * Fp + f0));
 #pragma unroll
-            for (int v = 0; v < VW; v++) z ^= slice((A)sv[t].x[v], paper) << v;
-        }
-    flag_unsat<VW>(unsat, f0, z & act);
+        for (int t = 0; t < D; t++)
+            if (t < d) {
+#pragma unroll
+                for (int v = 0; v < VW; v++) z ^= slice((A)sv[t].x[v], paper) << v;
+            }
+    }
+    __syncwarp();
+    flag_unsat<VW>(unsat, f0, z & act, have);
 }
 
 // ------------------------------------------------------------------------------------
@@ -882,7 +889,7 @@ struct StagedArgs {
     int M, Fp, n_fblocks, stages, paper, n_classes;
     uint32_t wait_limit;
     const uint8_t* state;
-    uint8_t* unsat;
+    uint32_t* unsat;
     int32_t* err;
     const int32_t* comp;  // [1]: positions in use (frame blocks behind them get no task)
 };
@@ -1079,7 +1086,8 @@ __global__ void __launch_bounds__(kStagedMaxThreads) k_check_staged(const Staged
             cy++;
         }
         if ((SYN || SYN_ONLY) && cy != py) {  // the warp's rows of this frame block are done
-            flag_unsat<VW>(a.unsat, py * FB + lane * VW, zacc);
+            const int f0 = py * FB + lane * VW;
+            flag_unsat<VW>(a.unsat, f0, zacc, unsat_now(a.unsat, f0));
             zacc = 0;
         }
     }
@@ -1109,7 +1117,7 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
                                          const typename Tr<MODE>::T* __restrict__ eta, int Fp,
                                          uint8_t* state, int32_t* done_iter,
                                          const int32_t* __restrict__ pos2frame,
-                                         const uint8_t* __restrict__ unsat, int test_prev, int k,
+                                         const uint32_t* __restrict__ unsat, int test_prev, int k,
                                          int* n_done, const CState& cs, int dshift,
                                          const IterWeights& wt, uint8_t* hd, int paper) {
     using T = typename Tr<MODE>::T;
@@ -1133,11 +1141,7 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
     if (!act) return;
     uint32_t upd = act;
     if (test_prev) {
-        const VS un = *reinterpret_cast<const VS*>(unsat + f0);
-        uint32_t conv = 0;
-#pragma unroll
-        for (int v = 0; v < V; v++) conv |= (uint32_t)(un.x[v] == 0) << v;
-        conv &= act;
+        const uint32_t conv = ~(__ldg(unsat + (f0 >> 5)) >> (f0 & 31)) & act;
         upd = act & ~conv;
         if (j == 0 && conv) {  // one designated thread per frame records the stop
 #pragma unroll
@@ -1273,7 +1277,7 @@ __global__ void __launch_bounds__(128, VW <= 2 ? 8 : 16) k_var(const int32_t* __
                                              const typename Tr<MODE>::T* __restrict__ eta, int Fp,
                                              uint8_t* state, int32_t* done_iter,
                                              const int32_t* __restrict__ pos2frame,
-                                             const uint8_t* __restrict__ unsat, int test_prev,
+                                             const uint32_t* __restrict__ unsat, int test_prev,
                                              int k, int* n_done, int frames, const int32_t* comp,
                                              CState cs = CState{}, int dshift = 0,
                                              IterWeights wt = IterWeights(), uint8_t* hd = nullptr,
@@ -1472,18 +1476,16 @@ __global__ void __launch_bounds__(256) k_store_hd(const uint8_t* __restrict__ hd
     }
 }
 
-// Status of the frames in the final layout (positions in use).
-// ubits (nullable): the final syndrome as a bit array (k_syn_hd) instead of unsat_final.
+// Status of the frames in the final layout (positions in use); unsat: the final syndrome.
 __global__ void k_finish(const int32_t* done_iter, const int32_t* pos2frame, const int32_t* comp,
-                         const uint8_t* unsat_final, int Fp, int L, int32_t* out_iters,
-                         uint8_t* out_ok, const uint32_t* ubits = nullptr) {
+                         const uint32_t* unsat, int Fp, int L, int32_t* out_iters, uint8_t* out_ok) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= Fp || p >= comp[1]) return;
     const int f = pos2frame[p];
     if (f < 0) return;
     const int d = done_iter[f];
     out_iters[f] = d >= 0 ? d : L;
-    const int fails = ubits ? (int)((ubits[p >> 5] >> (p & 31)) & 1u) : (unsat_final[p] != 0);
+    const int fails = (int)((unsat[p >> 5] >> (p & 31)) & 1u);
     if (out_ok) out_ok[f] = d >= 0 ? 1 : !fails;
 }
 
@@ -1491,7 +1493,7 @@ __global__ void k_finish(const int32_t* done_iter, const int32_t* pos2frame, con
 // task count does not fit 32 bits (the caller then runs the unstaged kernel).
 template <int MODE, int V, bool FIRST, bool W, int D, bool SYN_ONLY = false, bool CMP = false>
 bool launch_staged(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
-                   const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint8_t* un,
+                   const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint32_t* un,
                    int test_prev, const IterWeights& wt, cudaStream_t st) {
     if (w.stages <= 0 || w.stage_warps <= 0 || w.num_sms <= 0 || !w.err) return false;
     using LY = StagedLayout<MODE, V, D, CMP>;
@@ -1542,7 +1544,7 @@ bool launch_staged(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
 // works on the same frame stride.
 template <int MODE, int V, bool FIRST, bool W, int D, bool CMP = false>
 bool staged(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
-            const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint8_t* un, int test_prev,
+            const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint32_t* un, int test_prev,
             const IterWeights& wt, cudaStream_t st) {
     switch (w.stage_vw) {
         case 0: return launch_staged<MODE, V, FIRST, W, D, false, CMP>(g, a, w, s, eta, un, test_prev, wt, st);
@@ -1568,7 +1570,7 @@ bool staged(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
 // can only happen on the first iteration, before any state exists).
 template <int V, bool FIRST, bool W>
 bool check_pass_cmp(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, const float* s,
-                    float* state, uint8_t* un, int test_prev, const IterWeights& wt_prev, cudaStream_t st) {
+                    float* state, uint32_t* un, int test_prev, const IterWeights& wt_prev, cudaStream_t st) {
     if (g.ell_D == 8) return staged<kModeFP32, V, FIRST, W, 8, true>(g, a, w, s, state, un, test_prev, wt_prev, st);
     if (g.ell_D == 16) return staged<kModeFP32, V, FIRST, W, 16, true>(g, a, w, s, state, un, test_prev, wt_prev, st);
     return false;
@@ -1578,7 +1580,7 @@ bool check_pass_cmp(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
 // staging is on) or the register kernel; else the general kernel on the CSR order.
 template <int MODE, int V, bool FIRST, bool W>
 void check_pass_t(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, dim3 gc,
-                  const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint8_t* un,
+                  const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint32_t* un,
                   int test_prev, const IterWeights& wt, cudaStream_t st) {
     const int Fp = w.Fp;
     if (g.ell_D == 8) {
@@ -1607,7 +1609,7 @@ void check_pass_t(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, d
 
 template <int MODE, int V>
 void check_pass(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, dim3 gc,
-                const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint8_t* un,
+                const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint32_t* un,
                 int test_prev, bool first, const IterWeights& wt, cudaStream_t st) {
     if constexpr (MODE == kModeFP32) {  // learned weights exist in FP32 mode only
         if (wt.alpha != nullptr) {
@@ -1651,7 +1653,7 @@ int compact(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStr
 // One bit pass of iteration k; hd: the HD variant (the last iteration, decisions packed).
 template <int MODE, int V, bool CMP, bool W>
 void var_pass(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, dim3 gv, const int32_t* cslot,
-              uint8_t* un, int test_prev, int k, bool hd, const CState& cs, int dshift,
+              uint32_t* un, int test_prev, int k, bool hd, const CState& cs, int dshift,
               const IterWeights& wt, cudaStream_t st) {
     using T = typename Tr<MODE>::T;
     using R = typename Tr<MODE>::R;
@@ -1682,7 +1684,8 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
     R* r = (R*)w.r;
     int launches = 0;
     if (cudaMemsetAsync(w.n_done, 0, sizeof(int32_t), st) != cudaSuccess) return LDPC_ERR_CUDA;
-    if (cudaMemsetAsync(w.unsat, 0, (size_t)(a.L + 2) * Fp, st) != cudaSuccess) return LDPC_ERR_CUDA;
+    const int uw = Fp / 32;  // words of unsatisfied-check bits per pass
+    if (cudaMemsetAsync(w.unsat, 0, (size_t)(a.L + 2) * uw * 4, st) != cudaSuccess) return LDPC_ERR_CUDA;
     uint8_t* state = w.state;
     k_init_state<<<(Fp + 255) / 256, 256, 0, st>>>(state, w.done_iter, w.pos2frame, w.comp, Fp,
                                                     a.frames);
@@ -1723,7 +1726,7 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
     const bool may_compact = a.early_stop && w.comp && a.frames > 32 * V;
     for (int k = 1; k <= a.L; k++) {
         const int test_prev = a.early_stop && ((k - 1) % a.check_every == 0);
-        uint8_t* un = w.unsat + (size_t)k * Fp;
+        uint32_t* un = w.unsat + (size_t)k * uw;
         const IterWeights wt = weights_of(k);
         if constexpr (MODE == kModeFP32) {
             if (cmp) {
@@ -1759,18 +1762,16 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
             launches += compact<MODE>(g, a, w, st, false);
     }
     if (w.used_compressed) *w.used_compressed = cmp ? 1 : 0;
-    uint8_t* unf = w.unsat + (size_t)(a.L + 1) * Fp;
+    uint32_t* unf = w.unsat + (size_t)(a.L + 1) * uw;
     bool syn_done = false;
-    uint32_t* ubits = nullptr;  // the final syndrome as bits, in the (cleared) unf region
     if constexpr (V == 4 || V == 8) {
         if (hd && (g.ell_D == 8 || g.ell_D == 16)) {
             const int runs = (a.M + kSynRows - 1) / kSynRows;
             const dim3 gs((unsigned)((runs + 7) / 8), (unsigned)((Fp / (4 * V) + 31) / 32));
-            ubits = reinterpret_cast<uint32_t*>(unf);  // Fp / 8 of its Fp bytes, 256-byte aligned
             if (g.ell_D == 8)
-                k_syn_hd<V, 8><<<gs, 256, 0, st>>>(g.ell_col, g.ell_deg, a.M, w.hd, Fp, ubits);
+                k_syn_hd<V, 8><<<gs, 256, 0, st>>>(g.ell_col, g.ell_deg, a.M, w.hd, Fp, unf);
             else
-                k_syn_hd<V, 16><<<gs, 256, 0, st>>>(g.ell_col, g.ell_deg, a.M, w.hd, Fp, ubits);
+                k_syn_hd<V, 16><<<gs, 256, 0, st>>>(g.ell_col, g.ell_deg, a.M, w.hd, Fp, unf);
             syn_done = true;
         }
     }
@@ -1805,8 +1806,8 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
     if (!stored)
         k_store<MODE><<<dim3((a.N + kStoreTJ - 1) / kStoreTJ, Fp / kStoreTF), 256, 0, st>>>(
             s, Fp, a.N, w.pos2frame, w.comp, a.out_bits, a.out_soft, a.paper_slicer);
-    k_finish<<<(Fp + 255) / 256, 256, 0, st>>>(w.done_iter, w.pos2frame, w.comp, unf, Fp, a.L,
-                                               a.out_iters, a.out_ok, ubits);
+    k_finish<<<(Fp + 255) / 256, 256, 0, st>>>(w.done_iter, w.pos2frame, w.comp, unf, Fp, a.L, a.out_iters,
+                                               a.out_ok);
     launches += 3;
     if (cudaGetLastError() != cudaSuccess) return LDPC_ERR_CUDA;
     return launches;
