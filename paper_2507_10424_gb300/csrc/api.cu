@@ -585,7 +585,7 @@ int ldpc_decode_ex(ldpc_t* h, const void* llr, int32_t llr_dtype, int32_t frames
             }
         } else {
             apply_staging(h, h->sw);
-            const int vw = stream_lane_frames(h->dg, frames, h->sw);
+            const int vw = stream_lane_frames(frames, h->sw);
             int rc = ensure_stream_work(h, frames, max_iter, vw ? 32 * vw : 256);
             if (rc != LDPC_OK) return rc;
             int32_t used_cmp = 0;

@@ -186,7 +186,7 @@ static int batch_enqueue(ldpc_batch_t* b) {
             const auto& x = b->streamed[k];
             if (x.a.frames == 0) continue;
             StreamWork w = x.w;
-            const int vw = stream_lane_frames(*b->views[x.code].dg, x.a.frames, w);
+            const int vw = stream_lane_frames(x.a.frames, w);
             stream_narrow(w, x.a.frames, vw);
             const int n = stream_decode(kModeFP32, *b->views[x.code].dg, x.a, w, (k & 1) ? b->side2 : b->side, vw);
             if (n < 0) return n;

@@ -243,7 +243,7 @@ inline size_t staged_smem_bytes(int mode, int vw, int D, bool cmp, int warps, in
 // Frames a lane takes in the streaming passes of a batch: 0 = the full 16-byte vector of the
 // mode on a frame stride of whole 256-frame blocks, else 1 or 2 frames with the register
 // kernels and per-edge messages, on a stride of whole 32- or 64-frame blocks.
-int stream_lane_frames(const DevGraph& g, int32_t frames, const StreamWork& w);
+int stream_lane_frames(int32_t frames, const StreamWork& w);
 // Sets w's frame stride, staging and message format for lanes of vw frames.
 void stream_narrow(StreamWork& w, int32_t frames, int vw);
 

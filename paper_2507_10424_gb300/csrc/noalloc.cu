@@ -153,7 +153,7 @@ extern "C" int ldpc_decode_noalloc(ldpc_t* h, const void* llr, int32_t llr_dtype
         a.w_beta = v.w_alpha + (size_t)v.w_rows * v.dg->n_classes;
     }
     // the kernels clear the done counter and the syndrome flags and set the frame state
-    const int vw = stream_lane_frames(*v.dg, frames, w);
+    const int vw = stream_lane_frames(frames, w);
     stream_narrow(w, frames, vw);
     const int n = stream_decode(v.mode, *v.dg, a, w, v.stream, vw);
     if (n < 0) {  // a failed launch leaves its error pending: clear it and report it

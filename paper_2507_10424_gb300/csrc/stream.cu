@@ -15,17 +15,16 @@ int stream_decode_fixed(const DevGraph& g, const DecodeArgs& a, const StreamWork
 // Few frames: a 16-byte lane vector makes blocks of 128 (FP32) or 256 (fixed point) frames that
 // are mostly padding, and the staged pass's pipeline has nothing to overlap; the passes are
 // then chains of dependent loads, which the register kernels on one or two frames a lane
-// shorten (a row's, or four of a column's, messages requested together). Measured, 20
-// iterations, full vectors / one frame / two frames a lane, us a decode:
-//   32 frames: N=576 282 / 190 / 194, N=16200 (rows of 20-21) 722 / 360 / 434, N=64800 1484 /
-//     797 / 893;
-//   64 frames: N=12288 493 / 458 / 375, N=16200 732 / 529 / 465, N=64800 1529 / 1425 / 1047;
-//   128 frames: N=12288 503 / 692 / 536, N=64800 1631 / 2737 / 2066, but N=16200 792 / 869 /
-//     659: rows of more than 16 edges have no staged pass.
-int stream_lane_frames(const DevGraph& g, int32_t frames, const StreamWork& w) {
+// shorten (eight messages requested together). Measured, 20 iterations with early stop, full
+// vectors / one frame / two frames a lane, us a decode:
+//   32 frames: N=576 282 / 232 / 233, N=16200 (rows of 20-21) 710 / 412 / 441, N=64800 1547 /
+//     981 / 1146;
+//   64 frames: N=12288 504 / 634 / 395, N=16200 712 / 740 / 439, N=64800 1611 / 2034 / 1401;
+//   128 frames: N=12288 514 / 958 / 718, N=16200 749 / 1065 / 831.
+int stream_lane_frames(int32_t frames, const StreamWork& w) {
     if (!w.auto_staging) return 0;
     if (frames <= 32) return 1;
-    return frames <= (g.ell_D == 0 && g.max_dc <= 32 ? 128 : 64) ? 2 : 0;
+    return frames <= 64 ? 2 : 0;
 }
 
 void stream_narrow(StreamWork& w, int32_t frames, int vw) {

@@ -56,14 +56,6 @@ __device__ __forceinline__ float lam_of(float s, float e) { return s - e; }
 __device__ __forceinline__ int32_t lam_of(int32_t s, int32_t e) { return sat16(s - e); }
 __device__ __forceinline__ float absval(float x) { return fabsf(x); }
 __device__ __forceinline__ int32_t absval(int32_t x) { return abs(x); }
-// max for the second minimum: NaN when b is NaN, so that a NaN magnitude (infinite channel
-// values can produce one) leaves both minima as they are.
-__device__ __forceinline__ float max_nan(float a, float b) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ int32_t max_nan(int32_t a, int32_t b) { return max(a, b); }
 __device__ __forceinline__ float big(float) { return __int_as_float(0x7f800000); }
 __device__ __forceinline__ int32_t big(int32_t) { return 0x7fffffff; }
 template <typename A>
@@ -549,7 +541,7 @@ __device__ __forceinline__ uint32_t row_update(Row& row, int d, typename Tr<MODE
                     if (SYN) zx[v] ^= PAPER ? sbits(A(0) - sa) : sbits(sa);
                     const A l = FIRST ? sa : lam_of(sa, (A)ev.x[v]);
                     const A m = absval(l);
-                    min1[v] = min(min1[v], max_nan(min0[v], m));
+                    min1[v] = min(min1[v], max(min0[v], m));
                     min0[v] = min(min0[v], m);
                     sx[v] ^= sbits(l);
                     lv.x[v] = (T)l;  // exact: lambda is saturated to the storage range
@@ -630,12 +622,9 @@ __device__ __forceinline__ uint32_t row_update(Row& row, int d, typename Tr<MODE
     return z;
 }
 
-// CSR: the same on CSR order (rows of at most D edges; slots are CSR edge ids), one round trip
-// more, for the row's offset.
-template <int MODE, bool FIRST, bool W, int VW, int D, bool CSR = false>
+template <int MODE, bool FIRST, bool W, int VW, int D>
 __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
-    k_check_row(const int32_t* __restrict__ col, const uint8_t* __restrict__ ell_deg,
-                const int32_t* __restrict__ row_ptr, int M,
+    k_check_ell(const int32_t* __restrict__ ell_col, const uint8_t* __restrict__ ell_deg, int M,
                 const typename Tr<MODE>::T* __restrict__ s, typename Tr<MODE>::T* __restrict__ eta,
                 int Fp, const uint8_t* __restrict__ state, uint32_t* unsat, int do_syn,
                 int paper, IterWeights wt = IterWeights()) {
@@ -648,25 +637,16 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
     const int f0 = (blockIdx.y * 32 + lane) * VW;
     if (i >= M) return;
     const VS st = *reinterpret_cast<const VS*>(state + f0);
-    int d, c[D];
-    size_t e0;
-    if constexpr (CSR) {
-        e0 = (size_t)__ldg(row_ptr + i);
-        d = __ldg(row_ptr + i + 1) - (int)e0;
-#pragma unroll
-        for (int t = 0; t < D; t++) c[t] = t < d ? __ldg(col + e0 + t) : 0;
-    } else {
-        e0 = (size_t)i * D;
-        d = __ldg(ell_deg + i);
-        load_cols<D>(col + e0, c);
-    }
+    const int d = __ldg(ell_deg + i);
+    int c[D];
+    load_cols<D>(ell_col + (size_t)i * D, c);
     const uint32_t have = do_syn ? unsat_now(unsat, f0) : 0u;
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < VW; v++) act |= (uint32_t)(st.x[v] != 0) << v;
     uint32_t z = 0;
     if (act) {  // lanes whose frames have all stopped touch nothing
-        T* const erow = eta + e0 * Fp + f0;
+        T* const erow = eta + (size_t)i * D * Fp + f0;
         RegRow<VT, D> row;
         row.cols = c;
 #pragma unroll
@@ -687,10 +667,9 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
 // Final syndrome pass on the padded row layout (status of frames that never stopped): the
 // XOR of the decisions of a row's bits (eq. 1-2), every load of the row issued at once.
 // ------------------------------------------------------------------------------------
-template <int MODE, int VW, int D, bool CSR = false>
-__global__ void __launch_bounds__(128) k_syn_row(const int32_t* __restrict__ col,
-                                                 const uint8_t* __restrict__ ell_deg,
-                                                 const int32_t* __restrict__ row_ptr, int M,
+template <int MODE, int VW, int D>
+__global__ void __launch_bounds__(128) k_syn_ell(const int32_t* __restrict__ ell_col,
+                                                 const uint8_t* __restrict__ ell_deg, int M,
                                                  const typename Tr<MODE>::T* __restrict__ s, int Fp,
                                                  const uint8_t* __restrict__ state,
                                                  uint32_t* unsat, int paper) {
@@ -702,16 +681,9 @@ __global__ void __launch_bounds__(128) k_syn_row(const int32_t* __restrict__ col
     const int f0 = (blockIdx.y * 32 + lane) * VW;
     if (i >= M) return;
     const VS st = *reinterpret_cast<const VS*>(state + f0);
-    int d, c[D];
-    if constexpr (CSR) {
-        const int e0 = __ldg(row_ptr + i);
-        d = __ldg(row_ptr + i + 1) - e0;
-#pragma unroll
-        for (int t = 0; t < D; t++) c[t] = t < d ? __ldg(col + e0 + t) : 0;
-    } else {
-        d = __ldg(ell_deg + i);
-        load_cols<D>(col + (size_t)i * D, c);
-    }
+    const int d = __ldg(ell_deg + i);
+    int c[D];
+    load_cols<D>(ell_col + (size_t)i * D, c);
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < VW; v++) act |= (uint32_t)(st.x[v] != 0) << v;
@@ -731,6 +703,248 @@ __global__ void __launch_bounds__(128) k_syn_row(const int32_t* __restrict__ col
     }
     __syncwarp();
     flag_unsat<VW>(unsat, f0, z & act, have);
+}
+
+// ------------------------------------------------------------------------------------
+// Few frames (one or two a lane; stream_lane_frames): rows of at most 32 edges on either
+// slot order (ell_deg: padded rows of D slots, else CSR). Such a pass is about one wave of
+// warps, each a chain of dependent loads, so the chain is kept short (the row's columns in
+// one load, the gathers of U edges together), the registers few, so that the wave holds
+// every row (a row keeps its minima, the first location and one sign bit per edge, not its
+// lambdas), and the instructions few: with 18 warps an SM the pass is bound by issue
+// latency. Lanes whose frames have all stopped read what the first running lane reads and
+// store nothing. Same results as k_check, NaN included (no lambda is ever -0.0, so its sign
+// bit is [lambda < 0]). Against kernels that hold all operands of a row in registers (128 to
+// 226 of them): graph replay of 25 iterations on 64 frames, N=12288 409 -> 356 us, N=16200
+// (rows of 20-21 edges) 521 -> 444 us.
+// ------------------------------------------------------------------------------------
+template <int V>
+struct FewRow {
+    int i, lane, f0, fo, d, mycol;
+    size_t e0;
+    bool on;
+    uint32_t act, have;
+    // false: no frame of the warp is being decoded
+    __device__ __forceinline__ bool load(const int32_t* __restrict__ col, const uint8_t* __restrict__ ell_deg,
+                                         const int32_t* __restrict__ row_ptr, int D, const uint8_t* state,
+                                         const uint32_t* unsat, int do_syn) {
+        const Vec<uint8_t, V> st = *reinterpret_cast<const Vec<uint8_t, V>*>(state + f0);
+        have = do_syn ? unsat_now(unsat, f0) : 0u;
+        if (ell_deg) {
+            e0 = (size_t)i * D;
+            d = __ldg(ell_deg + i);
+            mycol = lane < D ? __ldg(col + e0 + lane) : 0;
+        } else {
+            e0 = (size_t)__ldg(row_ptr + i);
+            d = __ldg(row_ptr + i + 1) - (int)e0;
+            mycol = lane < d ? __ldg(col + e0 + lane) : 0;
+        }
+        act = 0;
+#pragma unroll
+        for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
+        on = act != 0;
+        const uint32_t m = __ballot_sync(0xffffffffu, on);
+        fo = on ? f0 : f0 + (__ffs(m) - 1 - lane) * V;
+        return m != 0;
+    }
+};
+// The sign bit of the hard decision of s, paper's slicer when pm = -1 (fma: +0 stays +0).
+__device__ __forceinline__ uint32_t dec_sign(float s, float pm) { return __float_as_uint(__fmaf_rn(s, pm, 0.0f)); }
+__device__ __forceinline__ uint32_t dec_sign(int32_t s, int32_t pm) { return (uint32_t)(s * pm); }
+
+template <int MODE, bool FIRST, bool W, int V>
+__global__ void __launch_bounds__(128, 8)
+    k_check_few(const int32_t* __restrict__ col, const uint8_t* __restrict__ ell_deg,
+                const int32_t* __restrict__ row_ptr, int D, int M,
+                const typename Tr<MODE>::T* __restrict__ s, typename Tr<MODE>::T* eta, int Fp,
+                const uint8_t* __restrict__ state, uint32_t* unsat, int do_syn, int paper,
+                IterWeights wt = IterWeights()) {
+    using T = typename Tr<MODE>::T;
+    using A = typename Tr<MODE>::A;
+    using VT = Vec<T, V>;
+    FewRow<V> row;
+    row.lane = threadIdx.x & 31;
+    row.i = blockIdx.x * 4 + (threadIdx.x >> 5);
+    row.f0 = (blockIdx.y * 32 + row.lane) * V;
+    if (row.i >= M || !row.load(col, ell_deg, row_ptr, D, state, unsat, do_syn)) return;
+    const int d = row.d;
+    const T* const sp = s + row.fo;
+    T* const er = eta + row.e0 * Fp + row.fo;
+    const A pm = paper ? A(-1) : A(1);
+    A min0[V], min1[V];
+    int loc[V];
+    uint32_t sg[V], zx[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        min0[v] = min1[v] = big(A());
+        loc[v] = 0;
+        sg[v] = zx[v] = 0;
+    }
+    constexpr int U = 8;
+    for (int k0 = 0; k0 < d; k0 += U) {
+        VT sv[U], ev[U];
+        const T* ep = er + (size_t)k0 * Fp;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int c = __shfl_sync(0xffffffffu, row.mycol, (k0 + u) & 31);  // (0 past the row)
+            sv[u] = ld_nc(reinterpret_cast<const VT*>(sp + (size_t)c * Fp));
+            if (!FIRST && k0 + u < d) ev[u] = *reinterpret_cast<const VT*>(ep + (size_t)u * Fp);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int k = k0 + u;
+            if (k >= d) break;  // the same for the whole warp
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                const A sa = (A)sv[u].x[v];
+                zx[v] ^= dec_sign(sa, pm);
+                const A lam = FIRST ? sa : lam_of(sa, (A)ev[u].x[v]);
+                const A a = absval(lam);
+                const bool lt0 = a < min0[v];  // strict: the first location of min0 stays
+                min1[v] = lt0 ? min0[v] : min(min1[v], a);
+                min0[v] = min(min0[v], a);
+                loc[v] = lt0 ? k : loc[v];
+                sg[v] = __funnelshift_l(sbits(lam), sg[v], 1);  // (sg << 1) | sign of lambda
+            }
+        }
+    }
+    uint32_t z = 0;
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        z |= (zx[v] >> 31) << v;
+        // message signs (the row's parity XOR lambda's own), edge 0 in bit 31
+        const uint32_t p = (__popc(sg[v]) & 1) ? 0xffffffffu : 0u;
+        sg[v] = d ? (sg[v] ^ p) << (32 - d) : 0u;
+    }
+    if (do_syn) flag_unsat<V>(unsat, row.f0, z & row.act, row.have);
+    T* ep = er;
+#pragma unroll 4
+    for (int k = 0; k < d; k++, ep += Fp) {
+        float wa = 1.0f, wb = 0.0f;
+        if constexpr (W) {
+            const int c = __ldg(wt.col_class + __shfl_sync(0xffffffffu, row.mycol, k));
+            wa = __ldg(wt.alpha + c);
+            wb = __ldg(wt.beta + c);
+        }
+        VT out;
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            A m = k == loc[v] ? min1[v] : min0[v];
+            if constexpr (W) {
+                const float x = __fmaf_rn(wa, (float)m, -wb);
+                m = (A)(x > 0.0f ? x : 0.0f);
+            }
+            out.x[v] = (T)signed_mag(m, sg[v]);
+            sg[v] <<= 1;
+        }
+        if (row.on) *reinterpret_cast<VT*>(ep) = out;
+    }
+}
+
+// The final syndrome of few frames.
+template <int MODE, int V>
+__global__ void __launch_bounds__(128) k_syn_few(const int32_t* __restrict__ col,
+                                                 const uint8_t* __restrict__ ell_deg,
+                                                 const int32_t* __restrict__ row_ptr, int D, int M,
+                                                 const typename Tr<MODE>::T* __restrict__ s, int Fp,
+                                                 const uint8_t* __restrict__ state, uint32_t* unsat,
+                                                 int paper) {
+    using A = typename Tr<MODE>::A;
+    using VT = Vec<typename Tr<MODE>::T, V>;
+    FewRow<V> row;
+    row.lane = threadIdx.x & 31;
+    row.i = blockIdx.x * 4 + (threadIdx.x >> 5);
+    row.f0 = (blockIdx.y * 32 + row.lane) * V;
+    if (row.i >= M || !row.load(col, ell_deg, row_ptr, D, state, unsat, 1)) return;
+    const typename Tr<MODE>::T* const sp = s + row.fo;
+    const A pm = paper ? A(-1) : A(1);
+    uint32_t zx[V], z = 0;
+#pragma unroll
+    for (int v = 0; v < V; v++) zx[v] = 0;
+#pragma unroll 8
+    for (int k = 0; k < row.d; k++) {
+        const int c = __shfl_sync(0xffffffffu, row.mycol, k);
+        const VT sv = ld_nc(reinterpret_cast<const VT*>(sp + (size_t)c * Fp));
+#pragma unroll
+        for (int v = 0; v < V; v++) zx[v] ^= dec_sign((A)sv.x[v], pm);
+    }
+#pragma unroll
+    for (int v = 0; v < V; v++) z |= (zx[v] >> 31) << v;
+    flag_unsat<V>(unsat, row.f0, z & row.act, row.have);
+}
+
+// The bit pass of few frames, a warp per column: state, channel value and edge range in one
+// round trip, the edges' slots in the next (one load), eight messages in the next.
+template <int MODE, int V>
+__global__ void __launch_bounds__(128, 12)
+    k_var_few(const int32_t* __restrict__ col_ptr, const int32_t* __restrict__ col_edge, int N,
+              const typename Tr<MODE>::R* __restrict__ r, typename Tr<MODE>::T* s,
+              const typename Tr<MODE>::T* __restrict__ eta, int Fp, uint8_t* state, int32_t* done_iter,
+              const int32_t* __restrict__ pos2frame, const uint32_t* __restrict__ unsat, int test_prev, int k,
+              int* n_done) {
+    using T = typename Tr<MODE>::T;
+    using A = typename Tr<MODE>::A;
+    using VT = Vec<T, V>;
+    const int lane = threadIdx.x & 31;
+    const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int f0 = (blockIdx.y * 32 + lane) * V;
+    if (j >= N) return;
+    const Vec<uint8_t, V> st = *reinterpret_cast<const Vec<uint8_t, V>*>(state + f0);
+    const uint32_t un = test_prev ? __ldg(unsat + (f0 >> 5)) : ~0u;
+    const int t0 = __ldg(col_ptr + j), t1 = __ldg(col_ptr + j + 1);
+    const Vec<typename Tr<MODE>::R, V> rv = *reinterpret_cast<const Vec<typename Tr<MODE>::R, V>*>(r + (size_t)j * Fp + f0);
+    uint32_t act = 0;
+#pragma unroll
+    for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
+    const uint32_t conv = ~(un >> (f0 & 31)) & act, upd = act & ~conv;
+    if (j == 0 && conv) {  // one designated thread per frame records the stop
+#pragma unroll
+        for (int v = 0; v < V; v++)
+            if ((conv >> v) & 1) {
+                done_iter[pos2frame[f0 + v]] = k - 1;
+                state[f0 + v] = 0;
+                atomicAdd(n_done, 1);
+            }
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, upd != 0);
+    if (!m) return;
+    const T* const ep = eta + (upd ? f0 : f0 + (__ffs(m) - 1 - lane) * V);
+    A acc[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) acc[v] = (A)rv.x[v];
+    constexpr int U = 8;
+    for (int q0 = t0; q0 < t1; q0 += 32) {
+        const int slot = __ldg(col_edge + min(q0 + lane, t1 - 1));
+        const int n = min(32, t1 - q0);
+        for (int b = 0; b < n; b += U) {
+            VT ev[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int e = __shfl_sync(0xffffffffu, slot, (b + u) & 31);
+                if (b + u < n) ev[u] = ld_nc(reinterpret_cast<const VT*>(ep + (size_t)e * Fp));
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (b + u >= n) break;
+#pragma unroll
+                for (int v = 0; v < V; v++) acc[v] = acc[v] + (A)ev[u].x[v];
+            }
+        }
+    }
+    T* sp = s + (size_t)j * Fp + f0;
+#pragma unroll
+    for (int v = 0; v < V; v++)
+        if (MODE == kModeFixed) acc[v] = sat16((int32_t)acc[v]);
+    if (upd == (1u << V) - 1u) {
+        VT out;
+#pragma unroll
+        for (int v = 0; v < V; v++) out.x[v] = (T)acc[v];
+        *reinterpret_cast<VT*>(sp) = out;
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; v++)
+            if ((upd >> v) & 1) sp[v] = (T)acc[v];
+    }
 }
 
 // ------------------------------------------------------------------------------------
@@ -1128,13 +1342,6 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
     using VR = Vec<R, V>;
     using VS = Vec<uint8_t, V>;
     const VS st = *reinterpret_cast<const VS*>(state + f0);
-    int t0, t1;
-    VR rv;
-    if constexpr (V <= 2) {  // one round trip less
-        t0 = __ldg(col_ptr + j);
-        t1 = __ldg(col_ptr + j + 1);
-        rv = *reinterpret_cast<const VR*>(r + (size_t)j * Fp + f0);
-    }
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
@@ -1154,11 +1361,8 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
         }
     }
     if (!upd) return;
-    if constexpr (V > 2) {
-        t0 = __ldg(col_ptr + j);
-        t1 = __ldg(col_ptr + j + 1);
-        rv = *reinterpret_cast<const VR*>(r + (size_t)j * Fp + f0);
-    }
+    const int t0 = __ldg(col_ptr + j), t1 = __ldg(col_ptr + j + 1);
+    const VR rv = *reinterpret_cast<const VR*>(r + (size_t)j * Fp + f0);
     A acc[V];
 #pragma unroll
     for (int v = 0; v < V; v++) acc[v] = (A)rv.x[v];
@@ -1189,24 +1393,6 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
                 if constexpr (W) m = cmsg_weight(m, wa, wb);
                 acc[v] = acc[v] + (A)cmsg_signed(m, w.x[v], tp);
             }
-        }
-    } else if constexpr (V <= 2) {
-        // few frames: the pass is one chain of dependent loads, so four messages are
-        // gathered at once (the registers are there: one or two frames a lane)
-        constexpr int U = 4;
-        for (int q = t0; q < t1; q += U) {
-            int e[U];
-            VT ev[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) e[u] = __ldg(col_edge + min(q + u, t1 - 1));
-#pragma unroll
-            for (int u = 0; u < U; u++) ev[u] = ld_nc(reinterpret_cast<const VT*>(eta + (size_t)e[u] * Fp + f0));
-#pragma unroll
-            for (int u = 0; u < U; u++)
-                if (q + u < t1) {
-#pragma unroll
-                    for (int v = 0; v < V; v++) acc[v] = acc[v] + (A)ev[u].x[v];
-                }
         }
     } else if constexpr (MODE == kModeFixed && V % 2 == 0) {
         // int16 pairs: each lane of a word added by one two-way dot product (dp2a)
@@ -1270,7 +1456,7 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
 // (CTAs that loop over strided tasks drift apart: 20 % slower on the N=64800 code); with
 // per-edge messages the looping form measured 1.7 % slower on the QC N=2304 code.
 template <int MODE, int VW = Tr<MODE>::V, bool CMP = false, bool W = false, bool HD = false>
-__global__ void __launch_bounds__(128, VW <= 2 ? 8 : 16) k_var(const int32_t* __restrict__ col_ptr,
+__global__ void __launch_bounds__(128, 16) k_var(const int32_t* __restrict__ col_ptr,
                                              const int32_t* __restrict__ col_edge, int N,
                                              const typename Tr<MODE>::R* __restrict__ r,
                                              typename Tr<MODE>::T* s,
@@ -1583,22 +1769,24 @@ void check_pass_t(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, d
                   const typename Tr<MODE>::T* s, typename Tr<MODE>::T* eta, uint32_t* un,
                   int test_prev, const IterWeights& wt, cudaStream_t st) {
     const int Fp = w.Fp;
-    if (g.ell_D == 8) {
-        if (staged<MODE, V, FIRST, W, 8>(g, a, w, s, eta, un, test_prev, wt, st)) return;
-        k_check_row<MODE, FIRST, W, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, eta, Fp,
-                                                              w.state, un, test_prev, a.paper_slicer, wt);
-        return;
-    }
-    if (g.ell_D == 16) {
-        if (staged<MODE, V, FIRST, W, 16>(g, a, w, s, eta, un, test_prev, wt, st)) return;
-        k_check_row<MODE, FIRST, W, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, eta, Fp,
-                                                               w.state, un, test_prev, a.paper_slicer, wt);
-        return;
-    }
+    if (g.ell_D == 8 && staged<MODE, V, FIRST, W, 8>(g, a, w, s, eta, un, test_prev, wt, st)) return;
+    if (g.ell_D == 16 && staged<MODE, V, FIRST, W, 16>(g, a, w, s, eta, un, test_prev, wt, st)) return;
     if constexpr (V <= 2) {
         if (g.max_dc <= 32) {
-            k_check_row<MODE, FIRST, W, V, 32, true><<<gc, 128, 0, st>>>(
-                g.col_idx, nullptr, g.row_ptr, a.M, s, eta, Fp, w.state, un, test_prev, a.paper_slicer, wt);
+            k_check_few<MODE, FIRST, W, V><<<gc, 128, 0, st>>>(
+                g.ell_D ? g.ell_col : g.col_idx, g.ell_D ? g.ell_deg : nullptr, g.row_ptr, g.ell_D, a.M, s, eta,
+                Fp, w.state, un, test_prev, a.paper_slicer, wt);
+            return;
+        }
+    } else {
+        if (g.ell_D == 8) {
+            k_check_ell<MODE, FIRST, W, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, eta, Fp, w.state,
+                                                                  un, test_prev, a.paper_slicer, wt);
+            return;
+        }
+        if (g.ell_D == 16) {
+            k_check_ell<MODE, FIRST, W, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, eta, Fp, w.state,
+                                                                   un, test_prev, a.paper_slicer, wt);
             return;
         }
     }
@@ -1660,18 +1848,22 @@ void var_pass(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, dim3 
     const R* r = (const R*)w.r;
     T* s = (T*)w.s;
     const T* eta = (const T*)w.eta;
-    if constexpr (V == 4 || V == 8) {
-        if (hd) {
-            k_var<MODE, V, CMP, W, true><<<gv, 128, 0, st>>>(g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state,
-                                                             w.done_iter, w.pos2frame, un, test_prev, k,
-                                                             w.n_done, a.frames, w.comp, cs, dshift, wt,
-                                                             w.hd, a.paper_slicer);
-            return;
+    if constexpr (V <= 2 && !CMP) {
+        k_var_few<MODE, V><<<dim3((a.N + 3) / 4, w.Fp / (32 * V)), 128, 0, st>>>(
+            g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state, w.done_iter, w.pos2frame, un, test_prev, k, w.n_done);
+    } else {
+        if constexpr (V == 4 || V == 8) {
+            if (hd) {
+                k_var<MODE, V, CMP, W, true><<<gv, 128, 0, st>>>(
+                    g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state, w.done_iter, w.pos2frame, un, test_prev, k,
+                    w.n_done, a.frames, w.comp, cs, dshift, wt, w.hd, a.paper_slicer);
+                return;
+            }
         }
+        k_var<MODE, V, CMP, W><<<gv, 128, 0, st>>>(g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state, w.done_iter,
+                                                   w.pos2frame, un, test_prev, k, w.n_done, a.frames, w.comp, cs,
+                                                   dshift, wt);
     }
-    k_var<MODE, V, CMP, W><<<gv, 128, 0, st>>>(g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state, w.done_iter,
-                                               w.pos2frame, un, test_prev, k, w.n_done, a.frames, w.comp, cs,
-                                               dshift, wt);
 }
 
 template <int MODE, int V>
@@ -1776,19 +1968,22 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
         }
     }
     if (!syn_done) {
-        if (g.ell_D == 8) {
-            if (!launch_staged<MODE, V, true, false, 8, true>(g, a, w, s, eta, unf, 1, IterWeights(), st))
-                k_syn_row<MODE, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, Fp, state,
-                                                          unf, a.paper_slicer);
-        } else if (g.ell_D == 16) {
-            if (!launch_staged<MODE, V, true, false, 16, true>(g, a, w, s, eta, unf, 1, IterWeights(), st))
-                k_syn_row<MODE, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, nullptr, a.M, s, Fp, state,
-                                                           unf, a.paper_slicer);
-        } else if (V <= 2 && g.max_dc <= 32) {
-            if constexpr (V <= 2)
-                k_syn_row<MODE, V, 32, true><<<gc, 128, 0, st>>>(g.col_idx, nullptr, g.row_ptr, a.M, s, Fp,
-                                                                 state, unf, a.paper_slicer);
-        } else
+        bool done = (g.ell_D == 8 && launch_staged<MODE, V, true, false, 8, true>(g, a, w, s, eta, unf, 1, IterWeights(), st)) ||
+                    (g.ell_D == 16 && launch_staged<MODE, V, true, false, 16, true>(g, a, w, s, eta, unf, 1, IterWeights(), st));
+        if constexpr (V <= 2) {
+            if (!done && g.max_dc <= 32) {
+                k_syn_few<MODE, V><<<gc, 128, 0, st>>>(g.ell_D ? g.ell_col : g.col_idx, g.ell_D ? g.ell_deg : nullptr,
+                                                       g.row_ptr, g.ell_D, a.M, s, Fp, state, unf, a.paper_slicer);
+                done = true;
+            }
+        } else if (!done && g.ell_D == 8) {
+            k_syn_ell<MODE, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf, a.paper_slicer);
+            done = true;
+        } else if (!done && g.ell_D == 16) {
+            k_syn_ell<MODE, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf, a.paper_slicer);
+            done = true;
+        }
+        if (!done)
             k_check<MODE, false, true, false, V><<<gc, 128, 0, st>>>(g.row_ptr, g.col_idx, a.M, s, eta, Fp,
                                                                      state, unf, 1, w.n_done, a.frames,
                                                                      a.paper_slicer);
