@@ -59,6 +59,8 @@ struct ldpc {
     int64_t E = 0;
     DevGraph dg;
     ResidentPlan plan[2];
+    ResidentPlan narrow[2][2];  // [mode]: one and two frames per tile, for few frames
+    ResidentPlan wide[2];       // [mode]: two frames per tile, index arrays in global memory
     ResidentTuning tuning;
     std::vector<int32_t> class_degree;
     // learned weights (FP32 mode)
@@ -112,7 +114,7 @@ static void free_graph(DevGraph& g) {
     void* ptrs[] = {g.row_ptr, g.col_idx, g.col_ptr, g.col_edge, g.packed, g.r_base,
                     g.r_deg, g.r_slot_pos, g.c_base, g.c_deg, g.c_slot, g.col_pos,
                     g.col_class, g.r_slot_cls, g.ell_col, g.ell_deg, g.ell_cslot, g.ell_cls,
-                    g.col_row, g.col_k};
+                    g.col_row, g.col_k, g.idx_blob};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     g = DevGraph();
@@ -233,9 +235,32 @@ static int ensure_stream_work(ldpc_t* h, int32_t frames, int32_t L, int32_t gran
 static void replan(ldpc_t* h) {
     h->cl_valid[0] = h->cl_valid[1] = 0;
     if (!h->dg.sliced) return;
-    const int we = h->w_rows * h->dg.n_classes;
-    h->plan[kModeFP32] = resident_plan(kModeFP32, h->dg, h->N, h->device, h->tuning, we);
-    h->plan[kModeFixed] = resident_plan(kModeFixed, h->dg, h->N, h->device, h->tuning, 0);
+    const ResidentTuning& t = h->tuning;
+    for (int mode : {kModeFP32, kModeFixed}) {
+        const int we = mode == kModeFP32 ? h->w_rows * h->dg.n_classes : 0;
+        h->plan[mode] = resident_plan(mode, h->dg, h->N, h->device, t, we);
+        for (int ft = 1; ft <= 2; ft++) {  // (a shape that was asked for is used for any batch)
+            ResidentTuning n;
+            n.FT = ft;
+            h->narrow[mode][ft - 1] = t.FT || t.threads || t.idx ? ResidentPlan()
+                                                                 : resident_plan(mode, h->dg, h->N, h->device, n, we);
+        }
+        ResidentTuning wd;
+        wd.FT = 2;
+        wd.idx = 2;
+        h->wide[mode] = t.FT || t.threads || t.idx ? ResidentPlan()
+                                                   : resident_plan(mode, h->dg, h->N, h->device, wd, we);
+    }
+}
+
+// The plan of a decode of `frames` frames.
+static ResidentPlan& plan_of(ldpc_t* h, int32_t frames, int early_stop) {
+    ResidentPlan& p = h->plan[h->mode];
+    if (h->w_rows == 0 && h->wide[h->mode].ok &&
+        resident_wide(h->mode, p, h->dg.max_dc, frames, early_stop, h->num_sms))
+        return h->wide[h->mode];
+    const int ft = resident_narrow(h->mode, p.FT, h->narrow[h->mode], frames, early_stop, h->num_sms);
+    return ft ? h->narrow[h->mode][ft - 1] : p;
 }
 
 // The cluster layout for cluster size 2^li, built and uploaded on first use.
@@ -406,9 +431,19 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
             (rc = upload(&d.col_pos, sg.col_pos.data(), sg.col_pos.size())) ||
             (rc = upload(&d.r_slot_cls, sg.r_slot_cls.data(), sg.r_slot_cls.size())))
             return bail(rc);
+        const IdxLayout I = idx_layout(sg.E_pad, sg.Ec_pad, sg.n_rslices, sg.n_cslices, hg.N);
+        std::vector<uint8_t> blob(I.total, 0);
+        auto put = [&](uint32_t at, const auto& v) { std::memcpy(blob.data() + at, v.data(), v.size() * sizeof(v[0])); };
+        put(I.rpos, sg.r_slot_pos);
+        put(I.cslot, sg.c_slot);
+        put(I.cpos, sg.col_pos);
+        put(I.rdeg, sg.r_deg);
+        put(I.cdeg, sg.c_deg);
+        put(I.rbase, sg.r_base);
+        put(I.cbase, sg.c_base);
+        if ((rc = upload(&d.idx_blob, blob.data(), blob.size()))) return bail(rc);
         d.sliced = 1;
-        h->plan[kModeFP32] = resident_plan(kModeFP32, d, hg.N, h->device);
-        h->plan[kModeFixed] = resident_plan(kModeFixed, d, hg.N, h->device);
+        replan(h);
     }
     e = cudaMalloc((void**)&h->counters, 8 * sizeof(int32_t));
     if (e != cudaSuccess) return bail(alloc_fail(e));
@@ -549,7 +584,7 @@ int ldpc_decode_ex(ldpc_t* h, const void* llr, int32_t llr_dtype, int32_t frames
         n = dense_decode(h->dg, a, h->dense_work, h->stream);
     } else if (resolved_variant(h) == LDPC_VARIANT_RESIDENT) {
         if (!h->plan[h->mode].ok) return fail(LDPC_ERR_UNSUPPORTED);
-        n = resident_decode(h->mode, h->dg, h->plan[h->mode], a, h->counters, h->num_sms, h->stream);
+        n = resident_decode(h->mode, h->dg, plan_of(h, frames, a.early_stop), a, h->counters, h->num_sms, h->stream);
     } else if (resolved_variant(h) == LDPC_VARIANT_CLUSTER) {
         const ClusterPlan& p = cluster_plan_of(h, h->mode);
         if (!p.ok) return fail(LDPC_ERR_UNSUPPORTED);

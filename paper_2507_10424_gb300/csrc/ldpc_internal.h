@@ -63,6 +63,33 @@ struct SlicedGraph {
 // Returns false when the code cannot use 16-bit slot ids or 8-bit degrees.
 bool build_sliced(const HostGraph& g, SlicedGraph& sg);
 
+// The index arrays of the resident kernel one after the other, each on a 16-byte boundary: the
+// order and offsets they have in shared memory and, as one array, in global memory.
+struct IdxLayout {
+    uint32_t rpos, cslot, cpos, rdeg, cdeg, rbase, cbase, total;
+};
+__host__ __device__ inline IdxLayout idx_layout(int E_pad, int Ec_pad, int n_rsl, int n_csl, int N) {
+    auto al = [](uint32_t x) { return (x + 15u) & ~15u; };
+    IdxLayout I{};
+    uint32_t o = 0;
+    I.rpos = o;
+    o = al(o + (uint32_t)E_pad * 2);
+    I.cslot = o;
+    o = al(o + (uint32_t)Ec_pad * 2);
+    I.cpos = o;
+    o = al(o + (uint32_t)N * 2);
+    I.rdeg = o;
+    o = al(o + (uint32_t)n_rsl * 32);
+    I.cdeg = o;
+    o = al(o + (uint32_t)n_csl * 32);
+    I.rbase = o;
+    o = al(o + (uint32_t)(n_rsl + 1) * 4);
+    I.cbase = o;
+    o = al(o + (uint32_t)(n_csl + 1) * 4);
+    I.total = o;
+    return I;
+}
+
 // ---------------------------------------------------------------------------------------
 // Padded row layout of the streaming kernels (codes whose rows have at most 16 edges):
 // every row owns D = 8 or 16 message slots, the t-th edge of row i at slot i D + t, so a
@@ -142,6 +169,7 @@ struct DevGraph {
     uint16_t* col_pos = nullptr;
     uint8_t* r_slot_cls = nullptr;
     int32_t n_rslices = 0, n_cslices = 0, E_pad = 0, Ec_pad = 0;
+    uint8_t* idx_blob = nullptr;  // the arrays above but r_slot_cls, laid out by idx_layout
     int32_t sliced = 0;  // the sliced layout exists
     int32_t max_dc = 0;  // longest row (set for every code)
     // padded row layout (streaming kernels); ell_D = 0 when absent
@@ -286,6 +314,12 @@ ResidentPlan resident_plan(int mode, const DevGraph& dg, int32_t N, int device,
                            const ResidentTuning& tune = ResidentTuning(), int w_entries = 0);
 int resident_decode(int mode, const DevGraph& dg, const ResidentPlan& p, const DecodeArgs& a,
                     int32_t* tile_counter, int num_sms, cudaStream_t st);
+// Whether two frames per tile with the index arrays in global memory serve a batch better than
+// the automatic plan p.
+bool resident_wide(int mode, const ResidentPlan& p, int32_t max_dc, int32_t frames, int early_stop, int num_sms);
+// Frames per tile of the narrower plan that serves a batch of `frames` frames better than the
+// automatic plan of width FT (0: none).
+int resident_narrow(int mode, int FT, const ResidentPlan narrow[2], int32_t frames, int early_stop, int num_sms);
 
 // Cluster variant: C CTAs (a thread-block cluster) per tile of FT frames.
 struct ClusterPlan {

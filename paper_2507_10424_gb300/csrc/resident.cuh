@@ -88,20 +88,15 @@ __host__ __device__ inline ResLayout res_layout(int tb, int FT, int E_pad, int E
     L.r = o;
     o = al16(o + (uint32_t)n_csl * 32 * FT * tb);
     if (idx) {
-        L.rpos = o;
-        o = al16(o + (uint32_t)E_pad * 2);
-        L.cslot = o;
-        o = al16(o + (uint32_t)Ec_pad * 2);
-        L.cpos = o;
-        o = al16(o + (uint32_t)N * 2);
-        L.rdeg = o;
-        o = al16(o + (uint32_t)n_rsl * 32);
-        L.cdeg = o;
-        o = al16(o + (uint32_t)n_csl * 32);
-        L.rbase = o;
-        o = al16(o + (uint32_t)(n_rsl + 1) * 4);
-        L.cbase = o;
-        o = al16(o + (uint32_t)(n_csl + 1) * 4);
+        const IdxLayout I = idx_layout(E_pad, Ec_pad, n_rsl, n_csl, N);
+        L.rpos = o + I.rpos;
+        L.cslot = o + I.cslot;
+        L.cpos = o + I.cpos;
+        L.rdeg = o + I.rdeg;
+        L.cdeg = o + I.cdeg;
+        L.rbase = o + I.rbase;
+        L.cbase = o + I.cbase;
+        o += I.total;
         if (w_entries > 0) {  // learned weights: class of each row slot, alpha and beta tables
             L.wcls = o;
             o = al16(o + (uint32_t)E_pad);
@@ -134,6 +129,7 @@ struct ResArgs {
     uint8_t* out_ok;
     float* out_soft;
     int32_t* tile_counter;
+    const uint8_t* idx_blob;  // the index arrays as one (idx_layout)
 };
 
 struct Idx {
@@ -941,6 +937,24 @@ __device__ __forceinline__ void copy_to_smem(T* dst, const T* src, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
 }
 
+// `bytes` (a multiple of 16; both sides 16-byte aligned) to shared memory, four loads in flight
+// a thread. The index arrays used to be copied one after the other by their elements, each
+// copy waiting for its own loads: about 4 us of a decode of one frame.
+__device__ __forceinline__ void copy16_to_smem(void* dst, const void* src, uint32_t bytes) {
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    const uint4* g = reinterpret_cast<const uint4*>(src);
+    const int n = (int)(bytes / 16), nth = blockDim.x;
+    for (int i = threadIdx.x; i < n; i += 4 * nth) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (i + u * nth < n) v[u] = __ldg(g + i + u * nth);
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (i + u * nth < n) d[i + u * nth] = v[u];
+    }
+}
+
 // Every iteration of one tile of nf frames (frames fbase .. fbase + nf - 1 of a.llr) with
 // eta, s and r at the given addresses (shared memory, or a CTA's slot of global scratch),
 // ending with the decisions of every frame written out. unsat_w: two words reset to 0.
@@ -1106,7 +1120,7 @@ __device__ __forceinline__ void decode_refill(const ResArgs& a, const Idx& ix, V
     constexpr bool kPacked = MODE == kModeFixed && FT % 2 == 0;
     constexpr uint32_t kAll = (1u << FT) - 1u;
     const int N = a.N;
-    if (threadIdx.x == 0) sl->next = atomicAdd(a.tile_counter, FT);
+    if (threadIdx.x == 0) sl->next = (int)blockIdx.x * FT;
     for (;;) {  // fresh tiles
         __syncthreads();
         const int fbase = sl->next;
@@ -1159,7 +1173,12 @@ __device__ __forceinline__ void decode_refill(const ResArgs& a, const Idx& ix, V
                 if (fin) {  // s still holds the decisions these frames end with
                     active &= ~fin;
                     // the counter's answer comes while the frames are written out
-                    if (threadIdx.x == 0) sl->next = atomicAdd(a.tile_counter, active ? __popc(fin) : FT);
+                    if (threadIdx.x == 0) {
+                        if (a.tile_counter)
+                            sl->next = (int)gridDim.x * FT + atomicAdd(a.tile_counter, active ? __popc(fin) : FT);
+                        else
+                            sl->next = a.frames;  // every frame was in a first tile
+                    }
                     for (int j = threadIdx.x; j < N; j += blockDim.x) {
                         const auto v = s[ix.col_pos[j]];
 #pragma unroll
@@ -1214,12 +1233,17 @@ __device__ __forceinline__ void decode_refill(const ResArgs& a, const Idx& ix, V
     }
 }
 
-template <int MODE, int FT, bool IDX_SMEM, bool PAPER, bool W, bool ES>
+// ONE: no more tiles than CTAs, CTA b decodes tile b (plain Min-Sum, standard slicer, no early
+// stop): no work counter, and the index arrays arrive in one copy. The kernels of full batches
+// keep the loop over the counter and the copies array by array, which the compiler turned into
+// a faster iteration (QC N=2304, 65536 frames: 8350 us against 8420).
+template <int MODE, int FT, bool IDX_SMEM, bool PAPER, bool W, bool ES, bool ONE = false>
 __global__ void __launch_bounds__(kMaxThreads, 1) k_resident(const ResArgs a) {
     using T = typename RT<MODE>::T;
     using VT = VecR<T, FT>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t unsat_w[2];
+    __shared__ int tile_sh;
     const int w_entries = W ? a.w_rows * a.n_classes : 0;
     const ResLayout lay = res_layout((int)sizeof(T), FT, a.E_pad, a.Ec_pad, a.n_rsl, a.n_csl, a.N,
                                      IDX_SMEM, w_entries);
@@ -1244,13 +1268,21 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_resident(const ResArgs a) {
         uint8_t* cdeg = smem_raw + lay.cdeg;
         int32_t* rbase = reinterpret_cast<int32_t*>(smem_raw + lay.rbase);
         int32_t* cbase = reinterpret_cast<int32_t*>(smem_raw + lay.cbase);
-        if (!kDec) copy_to_smem(rpos, a.r_slot_pos, a.E_pad);  // (kDec: the decision bytes' region)
-        copy_to_smem(cslot, a.c_slot, a.Ec_pad);
-        copy_to_smem(cpos, a.col_pos, a.N);
-        copy_to_smem(rdeg, a.r_deg, a.n_rsl * 32);
-        copy_to_smem(cdeg, a.c_deg, a.n_csl * 32);
-        copy_to_smem(rbase, a.r_base, a.n_rsl + 1);
-        copy_to_smem(cbase, a.c_base, a.n_csl + 1);
+        if constexpr (ONE || (ES && !W)) {
+            // all index arrays in one copy of 16-byte vectors (kDec: not the slot positions,
+            // whose region holds the decision bytes)
+            const uint32_t from = kDec ? lay.cslot - lay.rpos : 0u;
+            copy16_to_smem(smem_raw + lay.rpos + from, a.idx_blob + from,
+                           idx_layout(a.E_pad, a.Ec_pad, a.n_rsl, a.n_csl, a.N).total - from);
+        } else {
+            if (!kDec) copy_to_smem(rpos, a.r_slot_pos, a.E_pad);  // (kDec: the decision bytes' region)
+            copy_to_smem(cslot, a.c_slot, a.Ec_pad);
+            copy_to_smem(cpos, a.col_pos, a.N);
+            copy_to_smem(rdeg, a.r_deg, a.n_rsl * 32);
+            copy_to_smem(cdeg, a.c_deg, a.n_csl * 32);
+            copy_to_smem(rbase, a.r_base, a.n_rsl + 1);
+            copy_to_smem(cbase, a.c_base, a.n_csl + 1);
+        }
         ix = Idx{rbase, rdeg, kDec ? a.r_slot_pos : rpos, cbase, cdeg, cslot, cpos, nullptr, nullptr, nullptr};
         dec = reinterpret_cast<uint8_t*>(rpos);
         if (W) {
@@ -1275,8 +1307,14 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_resident(const ResArgs a) {
         __shared__ Slots slots;
         __syncthreads();  // the index arrays are in shared memory
         decode_refill<MODE, FT, VT, kDec>(a, ix, eta, s, r, unsat_w, &slots, n_rtasks, dec);
+    } else if constexpr (ONE) {
+        const int fbase = blockIdx.x * FT;
+        if (threadIdx.x < 2) unsat_w[threadIdx.x] = 0;
+        __syncthreads();
+        decode_tile<MODE, FT, PAPER, W, VT, true, ES, kDec>(a, ix, eta, s, r, unsat_w, fbase,
+                                                            min(FT, a.frames - fbase), walpha0, wbeta0,
+                                                            n_rtasks, dec);
     } else {
-        __shared__ int tile_sh;
         for (;;) {
             if (threadIdx.x == 0) {
                 tile_sh = atomicAdd(a.tile_counter, 1);
@@ -1297,7 +1335,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_resident(const ResArgs a) {
 
 template <int MODE, int FT, bool IDX, bool PAPER, bool W, bool ES>
 int launch(const ResArgs& ra, const ResidentPlan& p, int num_sms, cudaStream_t st) {
-    auto kern = k_resident<MODE, FT, IDX, PAPER, W, ES>;
+    void (*kern)(const ResArgs) = k_resident<MODE, FT, IDX, PAPER, W, ES>;
+    // no more tiles than SMs: as many CTAs as tiles run at once
+    constexpr bool kOne = !ES && !PAPER && !W;
+    const bool one = kOne && ra.n_tiles <= num_sms;
+    if constexpr (kOne)
+        if (one) kern = k_resident<MODE, FT, IDX, PAPER, W, ES, true>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess)
         return LDPC_ERR_CUDA;
     int per_sm = 0;
@@ -1305,7 +1348,11 @@ int launch(const ResArgs& ra, const ResidentPlan& p, int num_sms, cudaStream_t s
         return LDPC_ERR_CUDA;
     if (per_sm < 1) return LDPC_ERR_UNSUPPORTED;
     const int grid = std::max(1, std::min(ra.n_tiles, num_sms * per_sm));
-    kern<<<grid, p.threads, p.smem, st>>>(ra);
+    ResArgs r = ra;
+    // early stop: the first tile of CTA b is tile b, and without more there is no counter
+    if (one || (ES && !W && ra.n_tiles <= grid)) r.tile_counter = nullptr;
+    else if (cudaMemsetAsync(ra.tile_counter, 0, sizeof(int32_t), st) != cudaSuccess) return LDPC_ERR_CUDA;
+    kern<<<grid, p.threads, p.smem, st>>>(r);
     return cudaGetLastError() == cudaSuccess ? 1 : LDPC_ERR_CUDA;
 }
 
