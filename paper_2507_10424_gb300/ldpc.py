@@ -120,6 +120,20 @@ def load(path: str = LIB_PATH):
     return _lib
 
 
+_torch_module = None
+_LLR_TYPES = {}  # torch dtype of the channel values -> LDPC_LLR_*
+
+
+def _torch():
+    """torch, imported on first use."""
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _LLR_TYPES.update({torch.float32: LDPC_LLR_F32, torch.int8: LDPC_LLR_I8})
+        _torch_module = torch
+    return _torch_module
+
+
 class LdpcError(RuntimeError):
     def __init__(self, status: int, what: str = ""):
         msg = load().ldpc_strerror(status).decode()
@@ -518,28 +532,30 @@ class Decoder:
         Returns (bits uint8 [F][N], iters int32 [F], ok uint8 [F] or None, soft float32
         [F][N] or None), allocated on the tensor's device unless ``out`` gives them.
         """
-        import torch
-
-        if not llr.is_cuda or not llr.is_contiguous() or llr.dim() != 2 or llr.shape[1] != self.N:
+        # a decode of one frame takes the GPU about 15 us: the host side is kept as short
+        torch = _torch()
+        shape = llr.shape
+        if not llr.is_cuda or len(shape) != 2 or shape[1] != self.N or not llr.is_contiguous():
             raise ValueError("llr must be a contiguous CUDA tensor [F][N]")
-        dt = {torch.float32: LDPC_LLR_F32, torch.int8: LDPC_LLR_I8}[llr.dtype]
-        F = llr.shape[0]
+        dt = _LLR_TYPES[llr.dtype]
+        F = shape[0]
         dev = llr.device
         if out is None:
-            bits = torch.empty((F, self.N), dtype=torch.uint8, device=dev)
-            iters = torch.empty(F, dtype=torch.int32, device=dev)
-            ok = torch.empty(F, dtype=torch.uint8, device=dev) if want_ok else None
-            soft = torch.empty((F, self.N), dtype=torch.float32, device=dev) if want_soft else None
+            empty = torch.empty
+            bits = empty(shape, dtype=torch.uint8, device=dev)
+            iters = empty(F, dtype=torch.int32, device=dev)
+            ok = empty(F, dtype=torch.uint8, device=dev) if want_ok else None
+            soft = empty(shape, dtype=torch.float32, device=dev) if want_soft else None
         else:
             bits, iters, ok, soft = out
-        lib = load()
-        _check(lib.ldpc_set_stream(self.h, ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream)),
-               "ldpc_set_stream")
-        st = lib.ldpc_decode_ex(self.h, ctypes.c_void_p(llr.data_ptr()), dt, F, max_iter,
-                                int(bool(early_stop)), check_every, ctypes.c_void_p(bits.data_ptr()),
-                                ctypes.c_void_p(iters.data_ptr()),
-                                ctypes.c_void_p(ok.data_ptr()) if ok is not None else None,
-                                ctypes.c_void_p(soft.data_ptr()) if soft is not None else None)
+        lib = _lib or load()
+        h = self.h
+        st = lib.ldpc_set_stream(h, torch._C._cuda_getCurrentRawStream(dev.index))
+        if st != LDPC_OK:
+            _check(st, "ldpc_set_stream")
+        st = lib.ldpc_decode_ex(h, llr.data_ptr(), dt, F, max_iter, 1 if early_stop else 0, check_every,
+                                bits.data_ptr(), iters.data_ptr(), None if ok is None else ok.data_ptr(),
+                                None if soft is None else soft.data_ptr())
         _check(st, "ldpc_decode_ex")
         return bits, iters, ok, soft
 
