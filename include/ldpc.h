@@ -423,13 +423,14 @@ int ldpc_set_stream_staging(ldpc_t *h, int32_t warps_per_cta, int32_t stages, in
 
 /*
  * ldpc_set_stream_messages: how the streaming variant keeps the check-to-bit messages of
- * FP32 codes whose rows have at most 16 edges. compressed = 1 (default): per row and frame
+ * FP32 codes whose rows have at most 27 edges. compressed = 1 (default): per row and frame
  * only the two smallest magnitudes min0 <= min1 of Observation 1, the first location of
  * min0 and the signs of Observation 2 (12 bytes per row; every message eta_ij of eq.
  * (eta_update) is rebuilt from them exactly), so the per-edge messages never travel
- * through DRAM; it needs the staged check pass (ldpc_set_stream_staging with stages >= 2).
+ * through DRAM; rows of at most 16 edges need the staged check pass for it
+ * (ldpc_set_stream_staging with stages >= 2).
  * compressed = 0: one stored message per edge slot. Results do not depend on the choice.
- * Fixed-point mode and rows longer than 16 edges always keep per-edge messages.
+ * Fixed-point mode, rows longer than 27 edges and small batches always keep per-edge messages.
  * ldpc_autotune also chooses this for FP32 codes. LDPC_ERR_INVALID_ARG for other values.
  * ldpc_get_stream_messages: 1 when the next streaming decode keeps compressed messages.
  */

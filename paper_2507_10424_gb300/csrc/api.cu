@@ -114,7 +114,7 @@ static void free_graph(DevGraph& g) {
     void* ptrs[] = {g.row_ptr, g.col_idx, g.col_ptr, g.col_edge, g.packed, g.r_base,
                     g.r_deg, g.r_slot_pos, g.c_base, g.c_deg, g.c_slot, g.col_pos,
                     g.col_class, g.r_slot_cls, g.ell_col, g.ell_deg, g.ell_cslot, g.ell_cls,
-                    g.col_row, g.col_k, g.idx_blob};
+                    g.col_row, g.col_k, g.row_slot, g.idx_blob};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     g = DevGraph();
@@ -170,9 +170,12 @@ static void apply_staging(const ldpc_t* h, StreamWork& w) {
     w.msg_compressed = h->st_msg;
 }
 
-static int ensure_stream_work(ldpc_t* h, int32_t frames, int32_t L, int32_t granule = 256) {
+// The workspace of a decode of `frames` frames: a frame stride of whole blocks of `granule`
+// frames, room for whole blocks of `room` frames.
+static int ensure_stream_work(ldpc_t* h, int32_t frames, int32_t L, int32_t granule = 256, int32_t room = 1) {
     if (frames > kMaxStreamFrames) return fail(LDPC_ERR_INVALID_ARG);
-    const int32_t Fp = (frames + granule - 1) / granule * granule;
+    const int32_t stride = (frames + granule - 1) / granule * granule;
+    const int32_t Fp = (stride + room - 1) / room * room;
     if (Fp > h->sw_cap) {
         if (h->sw_big) {
             cudaStreamSynchronize(h->stream);
@@ -224,7 +227,7 @@ static int ensure_stream_work(ldpc_t* h, int32_t frames, int32_t L, int32_t gran
         }
         h->sw_cap_L = L;
     }
-    h->sw.Fp = Fp;
+    h->sw.Fp = stride;
     h->sw.unsat = h->sw_unsat;
     h->sw.n_done = h->counters + 1;
     apply_staging(h, h->sw);
@@ -390,14 +393,24 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
             std::vector<uint8_t> col_k((size_t)hg.E);
             for (int32_t i = 0; i < hg.M; i++)
                 for (int32_t e2 = hg.row_ptr[i]; e2 < hg.row_ptr[i + 1]; e2++) row_of[e2] = i;
-            for (int64_t q = 0; q < hg.E; q++) {
-                const int32_t e2 = hg.col_edge[q];
-                col_row[q] = row_of[e2];
-                col_k[q] = (uint8_t)(e2 - hg.row_ptr[row_of[e2]]);
+            // (12 bytes a row of state in the place of 4 an edge; slots in 31 bits)
+            if (hg.max_dc <= kCmsgMaxRow && hg.E >= 3 * (int64_t)hg.M && hg.M < (1 << 26)) {
+                std::vector<int32_t> row_slot((size_t)hg.E);
+                for (int64_t q = 0; q < hg.E; q++) {
+                    const int32_t e2 = hg.col_edge[q], i = row_of[e2];
+                    row_slot[q] = i << kRowSlotShift | (e2 - hg.row_ptr[i]);
+                }
+                if ((rc = upload(&h->dg.row_slot, row_slot.data(), row_slot.size()))) return bail(rc);
+            } else {
+                for (int64_t q = 0; q < hg.E; q++) {
+                    const int32_t e2 = hg.col_edge[q];
+                    col_row[q] = row_of[e2];
+                    col_k[q] = (uint8_t)(e2 - hg.row_ptr[row_of[e2]]);
+                }
+                if ((rc = upload(&h->dg.col_row, col_row.data(), col_row.size())) ||
+                    (rc = upload(&h->dg.col_k, col_k.data(), col_k.size())))
+                    return bail(rc);
             }
-            if ((rc = upload(&h->dg.col_row, col_row.data(), col_row.size())) ||
-                (rc = upload(&h->dg.col_k, col_k.data(), col_k.size())))
-                return bail(rc);
         }
     }
     // edge classes (learned weights)
@@ -621,7 +634,9 @@ int ldpc_decode_ex(ldpc_t* h, const void* llr, int32_t llr_dtype, int32_t frames
         } else {
             apply_staging(h, h->sw);
             const int vw = stream_lane_frames(frames, h->sw);
-            int rc = ensure_stream_work(h, frames, max_iter, vw ? 32 * vw : 256);
+            // (room for 256 frames in any case: a captured decode after one of fewer frames
+            // must not allocate)
+            int rc = ensure_stream_work(h, frames, max_iter, vw ? 32 * vw : 256, 256);
             if (rc != LDPC_OK) return rc;
             int32_t used_cmp = 0;
             StreamWork w = h->sw;
@@ -1070,7 +1085,12 @@ int ldpc_set_stream_messages(ldpc_t* h, int32_t compressed) {
 int ldpc_get_stream_messages(const ldpc_t* h, int32_t* compressed) {
     if (!h || !compressed) return fail(LDPC_ERR_BAD_POINTER);
     *compressed = 0;
-    if (!h->st_msg || h->mode != kModeFP32 || h->dg.ell_D == 0 || h->st_stages < 0) return LDPC_OK;
+    if (!h->st_msg || h->mode != kModeFP32) return LDPC_OK;
+    if (h->dg.row_slot) {  // rows of 17 to 27 edges need no staging
+        *compressed = 1;
+        return LDPC_OK;
+    }
+    if (h->dg.ell_D == 0 || h->st_stages < 0) return LDPC_OK;
     if (h->w_rows > 0 && h->dg.n_classes > 256) return LDPC_OK;
     // the staged kernel must fit (else the decode keeps per-edge messages)
     StreamWork w;

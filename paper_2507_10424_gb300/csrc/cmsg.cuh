@@ -1,20 +1,21 @@
-// Compressed check messages of the streaming variant (padded row layout, FP32 mode).
+// Compressed check messages of the streaming variant (FP32 mode, rows of at most 27 edges).
 //
 // Every message a check sends in one iteration follows from four things (Section III,
 // Observations 1 and 2): the two smallest magnitudes min0 <= min1 of the row's lambdas,
 // the first location of min0, and per edge the sign (the row's sign parity XOR the sign
-// of that edge's lambda). So a row of d <= 16 edges keeps, per frame,
+// of that edge's lambda). So a row of d <= 27 edges keeps, per frame,
 //   m0 = min0, m1 = min1 (binary32), and
-//   w  = bit t set for the edge holding min0 (t < 16) | sign of the message to edge t at
-//        bit 16 + t,
-// and the message to edge t is +-(bit t of w ? m1 : m0), with the magnitude weighted in the
+//   w  = the edge holding min0 (bits 0 .. 4) | sign of the message to edge t at bit 31 - t,
+// and the message to edge t is +-(t = w mod 32 ? m1 : m0), with the magnitude weighted in the
 // learned decoder (max(fma(alpha, m, -beta), 0), alpha and beta of the class of edge t's
-// bit). Twelve bytes per row and frame replace four bytes per message slot (8 or 16 per
-// row); the arrays are frame-interleaved like every streaming array, element (row i,
+// bit). Twelve bytes per row and frame replace four bytes per message slot (8, 16 or the row's
+// edges); the arrays are frame-interleaved like every streaming array, element (row i,
 // position p) at i Fp + p.
 #pragma once
 
 #include <stdint.h>
+
+#include "ldpc_internal.h"  // kCmsgMaxRow
 
 namespace ldpc_impl {
 
@@ -32,12 +33,19 @@ __host__ __device__ inline CState cstate_at(void* base, int64_t M, int64_t Fp) {
 
 // Magnitude of the message to edge t (before any weighting).
 __device__ __forceinline__ float cmsg_mag(float m0, float m1, uint32_t w, int t) {
-    return ((w >> t) & 1u) ? m1 : m0;
+    return (w & 31u) == (uint32_t)t ? m1 : m0;
 }
 
-// The message to edge t: magnitude m (>= 0) with the sign kept at bit 16 + t of w.
+// The message to edge t: magnitude m (>= 0) with the sign kept at bit 31 - t of w.
 __device__ __forceinline__ float cmsg_signed(float m, uint32_t w, int t) {
-    return __uint_as_float(__float_as_uint(m) | ((w << (15 - t)) & 0x80000000u));
+    return __uint_as_float(__float_as_uint(m) | ((w << t) & 0x80000000u));
+}
+
+// The word of a row of d edges: sg: lambda's signs, edge t at bit d - 1 - t. The message signs are the row's parity XOR each
+// edge's own.
+__device__ __forceinline__ uint32_t cmsg_word(uint32_t sg, int d, uint32_t loc) {
+    const uint32_t p = (__popc(sg) & 1) ? 0xffffffffu : 0u;
+    return (d ? (sg ^ p) << (32 - d) : 0u) | loc;
 }
 
 // Learned weighting of a magnitude: max(fma(alpha, m, -beta), 0) in binary32.

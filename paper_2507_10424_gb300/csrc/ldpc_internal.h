@@ -149,6 +149,9 @@ struct DevCluster {
 };
 
 // Device copies of the graph.
+constexpr int kRowSlotShift = 5;
+constexpr int kCmsgMaxRow = 27;  // longest row of compressed messages (cmsg.cuh)
+
 struct DevGraph {
     // CSR/CSC (streaming kernels)
     int32_t* row_ptr = nullptr;
@@ -183,6 +186,9 @@ struct DevGraph {
     // codes without the padded row layout: row of each CSC edge and its position in the row
     // (rows of at most 255 edges)
     int32_t* col_row = nullptr;  // E
+    // rows of 17 to 27 edges: both in one word, row << kRowSlotShift | position, in place of
+    // the two arrays (null where the row states would not fit the message slots)
+    int32_t* row_slot = nullptr;
     uint8_t* col_k = nullptr;    // E
 };
 
@@ -248,7 +254,8 @@ struct StreamWork {
     uint32_t wait_limit = 1u << 16;
     int32_t num_sms = 0;
     // FP32 codes on the padded row layout: keep each row's messages compressed (min0,
-    // min1, location and signs; cmsg.cuh) when the staged check pass runs (1), or keep one
+    // min1, location and signs; cmsg.cuh) when the staged check pass runs, and for rows of 17
+    // to 27 edges (1), or keep one
     // message per edge slot (0); used_compressed (host, nullable) receives the choice made
     int32_t msg_compressed = 1;
     int32_t* used_compressed = nullptr;

@@ -99,8 +99,8 @@ __global__ void k_lw_in(const float* src, int F, int N, float* dst, int Fp) {
 struct LwArgs {
     const int32_t *row_ptr, *col_idx, *col_ptr, *col_edge;
     const uint8_t* col_class;
-    // row and position in the row of each CSC edge: ell_cslot on the padded row layout (rows
-    // of at most 16 edges), else the two arrays
+    // row and position in the row of each CSC edge: one word on the padded row layout (rows of
+    // at most 16 edges) and for rows of at most 27, else the two arrays
     const int32_t *ell_cslot, *col_row;
     const uint8_t* col_k;
     int32_t dshift;
@@ -140,7 +140,7 @@ __device__ __forceinline__ uint32_t info_par(uint32_t info) {
 // Row and position in the row of CSC edge q.
 template <bool PK>
 __device__ __forceinline__ void edge_at(const LwArgs& a, int q, int& i, int& k) {
-    if (PK) {
+    if (PK || a.ell_cslot) {
         const int slot = __ldg(a.ell_cslot + q);
         i = slot >> a.dshift;
         k = slot & ((1 << a.dshift) - 1);
@@ -592,10 +592,10 @@ LwArgs make_args(const HandleView& v, int32_t Fp, const float* alpha, const floa
     a.col_ptr = v.dg->col_ptr;
     a.col_edge = v.dg->col_edge;
     a.col_class = v.dg->col_class;
-    a.ell_cslot = v.dg->ell_cslot;
+    a.ell_cslot = v.dg->ell_D ? v.dg->ell_cslot : v.dg->row_slot;
     a.col_row = v.dg->col_row;
     a.col_k = v.dg->col_k;
-    a.dshift = v.dg->ell_D == 16 ? 4 : 3;
+    a.dshift = v.dg->ell_D == 16 ? 4 : v.dg->ell_D == 8 ? 3 : kRowSlotShift;
     a.vrow = v.M > v.E;
     a.M = v.M;
     a.N = v.N;

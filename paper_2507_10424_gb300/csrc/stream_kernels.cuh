@@ -753,7 +753,7 @@ __device__ __forceinline__ uint32_t dec_sign(float s, float pm) { return __float
 __device__ __forceinline__ uint32_t dec_sign(int32_t s, int32_t pm) { return (uint32_t)(s * pm); }
 
 template <int MODE, bool FIRST, bool W, int V>
-__global__ void __launch_bounds__(128, 8)
+__global__ void __launch_bounds__(128, V <= 2 ? 8 : 4)
     k_check_few(const int32_t* __restrict__ col, const uint8_t* __restrict__ ell_deg,
                 const int32_t* __restrict__ row_ptr, int D, int M,
                 const typename Tr<MODE>::T* __restrict__ s, typename Tr<MODE>::T* eta, int Fp,
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(128, 8)
         loc[v] = 0;
         sg[v] = zx[v] = 0;
     }
-    constexpr int U = 8;
+    constexpr int U = V <= 2 ? 8 : 4;
     for (int k0 = 0; k0 < d; k0 += U) {
         VT sv[U], ev[U];
         const T* ep = er + (size_t)k0 * Fp;
@@ -841,7 +841,105 @@ __global__ void __launch_bounds__(128, 8)
     }
 }
 
-// The final syndrome of few frames.
+// The check pass on compressed messages of rows without the padded layout (17 to 27 edges), a
+// warp per row of 32 V frames: the row's columns (and, learned, the previous iteration's
+// weights of their classes) come in one load a warp and go to the lanes by shuffles, the
+// posteriors of U edges are requested together, and the row's state is all that is kept of the
+// messages. Bound by the gathers of s, 4 bytes an edge mostly from L2. The pass it replaces
+// (k_check: one dependent gather after another, 8 bytes an edge of messages) and its bit pass
+// took 343 us an iteration of N=16200 (rows of 20-21 edges, 2001 frames), the two now 260 us.
+template <bool FIRST, bool W, int V>
+__global__ void __launch_bounds__(128, 5)
+    k_check_cmp(const int32_t* __restrict__ col_idx, const int32_t* __restrict__ row_ptr, int M,
+                const float* __restrict__ s, CState cs, int Fp, const uint8_t* __restrict__ state,
+                uint32_t* unsat, int do_syn, int paper, IterWeights wt) {
+    using VF = Vec<float, V>;
+    using VU = Vec<uint32_t, V>;
+    FewRow<V> row;
+    row.lane = threadIdx.x & 31;
+    row.i = blockIdx.x * 4 + (threadIdx.x >> 5);
+    row.f0 = (blockIdx.y * 32 + row.lane) * V;
+    if (row.i >= M) return;
+    VF om0, om1;
+    VU ow;
+    if (!FIRST) {
+        const size_t o = (size_t)row.i * Fp + row.f0;
+        om0 = *reinterpret_cast<const VF*>(cs.m0 + o);
+        om1 = *reinterpret_cast<const VF*>(cs.m1 + o);
+        ow = *reinterpret_cast<const VU*>(cs.w + o);
+    }
+    if (!row.load(col_idx, nullptr, row_ptr, 0, state, unsat, do_syn)) return;
+    float mywa = 1.0f, mywb = 0.0f;
+    if constexpr (W && !FIRST) {
+        const int c = __ldg(wt.col_class + row.mycol);
+        mywa = __ldg(wt.alpha + c);
+        mywb = __ldg(wt.beta + c);
+    }
+    const int d = row.d;
+    const float* const sp = s + row.fo;
+    const float pm = paper ? -1.0f : 1.0f;
+    float min0[V], min1[V];
+    uint32_t loc[V], sg[V], zx[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        min0[v] = min1[v] = big(0.0f);
+        loc[v] = sg[v] = zx[v] = 0;
+    }
+    constexpr int U = 8;
+    for (int k0 = 0; k0 < d; k0 += U) {
+        VF sv[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int c = __shfl_sync(0xffffffffu, row.mycol, (k0 + u) & 31);
+            if (k0 + u < d) sv[u] = ld_nc(reinterpret_cast<const VF*>(sp + (size_t)c * Fp));
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int k = k0 + u;
+            if (k >= d) break;  // the same for the whole warp
+            float wa = 1.0f, wb = 0.0f;
+            if constexpr (W && !FIRST) {
+                wa = __shfl_sync(0xffffffffu, mywa, k);
+                wb = __shfl_sync(0xffffffffu, mywb, k);
+            }
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                const float sa = sv[u].x[v];
+                zx[v] ^= dec_sign(sa, pm);
+                float l = sa;
+                if constexpr (!FIRST) {
+                    float m = cmsg_mag(om0.x[v], om1.x[v], ow.x[v], k);
+                    if constexpr (W) m = cmsg_weight(m, wa, wb);
+                    l = sa - cmsg_signed(m, ow.x[v], k);
+                }
+                const float a = fabsf(l);
+                const bool lt = a < min0[v];  // strict: the first location of min0 stays
+                min1[v] = lt ? min0[v] : fminf(min1[v], a);
+                min0[v] = lt ? a : min0[v];
+                loc[v] = lt ? (uint32_t)k : loc[v];
+                sg[v] = __funnelshift_l(sbits(l), sg[v], 1);  // (sg << 1) | sign of lambda
+            }
+        }
+    }
+    uint32_t z = 0;
+    VF n0, n1;
+    VU nw;
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        z |= (zx[v] >> 31) << v;
+        n0.x[v] = min0[v];
+        n1.x[v] = min1[v];
+        nw.x[v] = cmsg_word(sg[v], d, loc[v]);
+    }
+    if (do_syn) flag_unsat<V>(unsat, row.f0, z & row.act, row.have);
+    if (!row.on) return;
+    const size_t o = (size_t)row.i * Fp + row.f0;
+    *reinterpret_cast<VF*>(cs.m0 + o) = n0;
+    *reinterpret_cast<VF*>(cs.m1 + o) = n1;
+    *reinterpret_cast<VU*>(cs.w + o) = nw;
+}
+
+// The final syndrome of few frames, and of any number on rows of 17 to 32 edges.
 template <int MODE, int V>
 __global__ void __launch_bounds__(128) k_syn_few(const int32_t* __restrict__ col,
                                                  const uint8_t* __restrict__ ell_deg,
@@ -970,7 +1068,7 @@ template <bool FIRST, bool SYN, bool PAPER, bool W, int VW, int D>
 __device__ __forceinline__ uint32_t row_update_cmp(const unsigned char* st, int chunk, int lane, int d,
                                                    const int* cls, const float* walpha,
                                                    const float* wbeta, const CState& cs, size_t off) {
-    static_assert(D <= 16, "signs and locations of at most 16 edges fit the word");
+    static_assert(D <= kCmsgMaxRow, "the signs and the location fit the word");
     using VF = Vec<float, VW>;
     using VU = Vec<uint32_t, VW>;
     auto at = [&](int c) { return st + (size_t)c * chunk + (size_t)lane * sizeof(VF); };
@@ -982,12 +1080,12 @@ __device__ __forceinline__ uint32_t row_update_cmp(const unsigned char* st, int 
         ow = *reinterpret_cast<const VU*>(at(D + 2));
     }
     float min0[VW], min1[VW];
-    uint32_t oh[VW], sg[VW], zx[VW];  // sg: lambda's sign bits, the first edge's highest
+    uint32_t loc[VW], sg[VW], zx[VW];  // sg: lambda's sign bits, the first edge's highest
 #pragma unroll
     for (int v = 0; v < VW; v++) {
         min0[v] = big(0.0f);
         min1[v] = big(0.0f);
-        oh[v] = 0;
+        loc[v] = 0;
         sg[v] = 0;
         zx[v] = 0;
     }
@@ -1015,7 +1113,7 @@ __device__ __forceinline__ uint32_t row_update_cmp(const unsigned char* st, int 
                 const bool lt = a < min0[v];  // strict: the first location of min0 stays
                 min1[v] = lt ? min0[v] : fminf(min1[v], a);
                 min0[v] = lt ? a : min0[v];
-                oh[v] = lt ? (1u << t) : oh[v];
+                loc[v] = lt ? (uint32_t)t : loc[v];
                 sg[v] = __funnelshift_l(sbits(l), sg[v], 1);  // (sg << 1) | sign of l
             }
         }
@@ -1024,17 +1122,13 @@ __device__ __forceinline__ uint32_t row_update_cmp(const unsigned char* st, int 
 #pragma unroll
         for (int v = 0; v < VW; v++) z |= (zx[v] >> 31) << v;
     }
-    const uint32_t dmask = (1u << d) - 1u;  // d <= 16
     VF n0, n1;
     VU nw;
 #pragma unroll
     for (int v = 0; v < VW; v++) {
         n0.x[v] = min0[v];
         n1.x[v] = min1[v];
-        // message signs: the row's sign parity XOR each edge's own sign; edge t's sign sits
-        // at bit d - 1 - t of sg, at bit 16 + t of the word (bit reversal, shift)
-        const uint32_t sgt = __brev(sg[v]) >> (16 - d);
-        nw.x[v] = oh[v] | ((sgt ^ ((__popc(sg[v]) & 1u) ? dmask << 16 : 0u)));
+        nw.x[v] = cmsg_word(sg[v], d, loc[v]);
     }
     *reinterpret_cast<VF*>(cs.m0 + off) = n0;
     *reinterpret_cast<VF*>(cs.m1 + off) = n1;
@@ -1310,8 +1404,8 @@ __global__ void __launch_bounds__(kStagedMaxThreads) k_check_staged(const Staged
 // ------------------------------------------------------------------------------------
 // Variable-node pass. Block = 4 warps = 4 columns; lane = one frame vector.
 // test_prev: the previous decision's syndrome (in unsat) decides whether a frame stops.
-// CMP (FP32): the messages are compressed (cmsg.cuh): col_edge holds padded-row slots
-// i 2^dshift + t, and the message of each edge is rebuilt from row i's state cs, weighted
+// CMP (FP32): the messages are compressed (cmsg.cuh): col_edge holds the slots i 2^dshift + t
+// of the padded rows (or row_slot), and the message of each edge is rebuilt from row i's state cs, weighted
 // (W) with this iteration's weights of the column's class.
 // HD (the last iteration, 4 or 8 frames per lane): each lane also writes the decisions of
 // its frames as one byte, bit v = frame f0 + v, to hd[j][Fp / VW] (byte f0 / VW), for the
@@ -1751,14 +1845,20 @@ bool staged(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
     return launch_staged<MODE, V, FIRST, W, D, false, CMP>(g, a, w, s, eta, un, test_prev, wt, st);
 }
 
-// One check pass on compressed messages (FP32, padded row layout, staged kernel only);
-// false when the staged kernel cannot run (the caller then keeps per-edge messages; this
+// One check pass on compressed messages (FP32): the staged kernel on the padded row layout,
+// k_check_cmp on rows of 17 to 27 edges (which need no staging); false when the staged kernel cannot run (the caller then keeps per-edge messages; this
 // can only happen on the first iteration, before any state exists).
 template <int V, bool FIRST, bool W>
 bool check_pass_cmp(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, const float* s,
                     float* state, uint32_t* un, int test_prev, const IterWeights& wt_prev, cudaStream_t st) {
     if (g.ell_D == 8) return staged<kModeFP32, V, FIRST, W, 8, true>(g, a, w, s, state, un, test_prev, wt_prev, st);
     if (g.ell_D == 16) return staged<kModeFP32, V, FIRST, W, 16, true>(g, a, w, s, state, un, test_prev, wt_prev, st);
+    if constexpr (V == 4) {
+        k_check_cmp<FIRST, W, V><<<dim3((a.M + 3) / 4, w.Fp / (32 * V)), 128, 0, st>>>(
+            g.col_idx, g.row_ptr, a.M, s, cstate_at(state, a.M, w.Fp), w.Fp, w.state, un, test_prev,
+            a.paper_slicer, wt_prev);
+        return true;
+    }
     return false;
 }
 
@@ -1771,14 +1871,14 @@ void check_pass_t(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, d
     const int Fp = w.Fp;
     if (g.ell_D == 8 && staged<MODE, V, FIRST, W, 8>(g, a, w, s, eta, un, test_prev, wt, st)) return;
     if (g.ell_D == 16 && staged<MODE, V, FIRST, W, 16>(g, a, w, s, eta, un, test_prev, wt, st)) return;
-    if constexpr (V <= 2) {
+    if (V <= 2 || g.ell_D == 0) {
         if (g.max_dc <= 32) {
             k_check_few<MODE, FIRST, W, V><<<gc, 128, 0, st>>>(
                 g.ell_D ? g.ell_col : g.col_idx, g.ell_D ? g.ell_deg : nullptr, g.row_ptr, g.ell_D, a.M, s, eta,
                 Fp, w.state, un, test_prev, a.paper_slicer, wt);
             return;
         }
-    } else {
+    } else if constexpr (V > 2) {
         if (g.ell_D == 8) {
             k_check_ell<MODE, FIRST, W, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, eta, Fp, w.state,
                                                                   un, test_prev, a.paper_slicer, wt);
@@ -1895,11 +1995,12 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
                         : dim3((unsigned)std::max(1ll, std::min(var_tasks, 16ll * (w.num_sms > 0 ? w.num_sms : 148))));
     // message slot of each edge in column order: padded-row slots or CSR edge ids
     const int32_t* cslot = g.ell_D ? g.ell_cslot : g.col_edge;
+    const int32_t* cslot_cmp = g.ell_D ? g.ell_cslot : g.row_slot;
     // compressed messages (cmsg.cuh) where the mode, the layout and the staging allow
     // (the staged kernel holds at most 256 classes of learned weights)
-    bool cmp = MODE == kModeFP32 && w.msg_compressed && g.ell_D > 0 && w.stages > 0 &&
-               (a.w_rows == 0 || a.n_classes <= 256);
-    const int dshift = g.ell_D == 16 ? 4 : 3;
+    bool cmp = MODE == kModeFP32 && w.msg_compressed &&
+               (g.ell_D > 0 ? w.stages > 0 && (a.w_rows == 0 || a.n_classes <= 256) : V == 4 && g.row_slot);
+    const int dshift = g.ell_D == 16 ? 4 : g.ell_D == 8 ? 3 : kRowSlotShift;
     // decisions of the last bit pass packed into w.hd (4 or 8 frames per lane): for the final
     // syndrome on the padded row layout, and for the output bits when no frame stops early
     // and no soft output is asked for (every position in use is then updated by that pass)
@@ -1932,10 +2033,10 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
                 if (ok) {
                     const CState cs = cstate_at(eta, a.M, Fp);
                     if (W)
-                        var_pass<MODE, V, true, true>(g, a, w, gv, g.ell_cslot, un, test_prev, k, hd && k == a.L,
+                        var_pass<MODE, V, true, true>(g, a, w, gv, cslot_cmp, un, test_prev, k, hd && k == a.L,
                                                       cs, dshift, wt, st);
                     else
-                        var_pass<MODE, V, true, false>(g, a, w, gv, g.ell_cslot, un, test_prev, k, hd && k == a.L,
+                        var_pass<MODE, V, true, false>(g, a, w, gv, cslot_cmp, un, test_prev, k, hd && k == a.L,
                                                        cs, dshift, wt, st);
                     launches += 2;
                     if (may_compact && k < a.L && k % kCompactEvery == 0)
@@ -1970,18 +2071,20 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
     if (!syn_done) {
         bool done = (g.ell_D == 8 && launch_staged<MODE, V, true, false, 8, true>(g, a, w, s, eta, unf, 1, IterWeights(), st)) ||
                     (g.ell_D == 16 && launch_staged<MODE, V, true, false, 16, true>(g, a, w, s, eta, unf, 1, IterWeights(), st));
-        if constexpr (V <= 2) {
+        if (V <= 2 || g.ell_D == 0) {
             if (!done && g.max_dc <= 32) {
                 k_syn_few<MODE, V><<<gc, 128, 0, st>>>(g.ell_D ? g.ell_col : g.col_idx, g.ell_D ? g.ell_deg : nullptr,
                                                        g.row_ptr, g.ell_D, a.M, s, Fp, state, unf, a.paper_slicer);
                 done = true;
             }
-        } else if (!done && g.ell_D == 8) {
-            k_syn_ell<MODE, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf, a.paper_slicer);
-            done = true;
-        } else if (!done && g.ell_D == 16) {
-            k_syn_ell<MODE, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf, a.paper_slicer);
-            done = true;
+        } else if constexpr (V > 2) {
+            if (!done && g.ell_D == 8) {
+                k_syn_ell<MODE, V, 8><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf, a.paper_slicer);
+                done = true;
+            } else if (!done && g.ell_D == 16) {
+                k_syn_ell<MODE, V, 16><<<gc, 128, 0, st>>>(g.ell_col, g.ell_deg, a.M, s, Fp, state, unf, a.paper_slicer);
+                done = true;
+            }
         }
         if (!done)
             k_check<MODE, false, true, false, V><<<gc, 128, 0, st>>>(g.row_ptr, g.col_idx, a.M, s, eta, Fp,
