@@ -101,7 +101,7 @@ __global__ void k_read_messages(const T* __restrict__ eta, int32_t Fp, const int
 // rebuilt from the row's state, weighted by the class of the edge's bit when w_alpha is set.
 __global__ void k_read_cmessages(CState cs, int32_t Fp, const int32_t* __restrict__ row_ptr,
                                  const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ col_class,
-                                 int32_t M, int32_t frames, int64_t E, const float* w_alpha,
+                                 int32_t M, int32_t half, int32_t frames, int64_t E, const float* w_alpha,
                                  const float* w_beta, float* __restrict__ out) {
     const int64_t total = (int64_t)frames * E;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total;
@@ -116,12 +116,13 @@ __global__ void k_read_cmessages(CState cs, int32_t Fp, const int32_t* __restric
         }
         const int t = e - row_ptr[lo];
         const size_t o = (size_t)lo * Fp + f;
-        float m = cmsg_mag(cs.m0[o], cs.m1[o], cs.w[o], t);
+        const uint32_t w = half ? cmsg_whole(static_cast<const uint16_t*>(cs.w)[o]) : static_cast<const uint32_t*>(cs.w)[o];
+        float m = cmsg_mag(cs.m0[o], cs.m1[o], w, t);
         if (w_alpha) {
             const int c = col_class[col_idx[e]];
             m = cmsg_weight(m, w_alpha[c], w_beta[c]);
         }
-        out[k] = cmsg_signed(m, cs.w[o], t);
+        out[k] = cmsg_signed(m, w, t);
     }
 }
 
@@ -132,7 +133,7 @@ int stream_read_messages(int mode, const DevGraph& g, int32_t M, int64_t E, cons
     const int grid = (int)std::min<int64_t>((total + 255) / 256, 65535);
     if (cmp)
         k_read_cmessages<<<grid, 256, 0, st>>>(cstate_at(w.eta, M, w.Fp), w.Fp, g.row_ptr, g.col_idx,
-                                               g.col_class, M, frames, E, w_alpha, w_beta, out);
+                                               g.col_class, M, g.ell_D == 8, frames, E, w_alpha, w_beta, out);
     else if (mode == kModeFP32)
         k_read_messages<float><<<grid, 256, 0, st>>>((const float*)w.eta, w.Fp, g.row_ptr, M, g.ell_D,
                                                      frames, E, 1.0f, out);

@@ -90,6 +90,34 @@ __device__ __forceinline__ uint32_t unsat_now(const uint32_t* unsat, int f0) {
     return __ldcg(unsat + (f0 >> 5));
 }
 
+// The same for a CTA whose warps take rows of the same 32 VW positions: the bits meet in shared
+// memory (one word per 32 positions) and one read and at most one atomic per word leave the
+// CTA. Reading the words warp by warp, every SM at once from the same L2 lines, made the
+// register check passes a third slower (N=64800, 1024 frames: 217 us with the syndrome, 136 us
+// without). begin: before the rows, all threads; end: after them, all threads.
+template <int VW>
+struct CtaFlags {
+    uint32_t have, *sh, *un;
+    __device__ __forceinline__ void begin(uint32_t* shared, uint32_t* unsat, int block_f0) {
+        sh = shared;
+        un = unsat + (block_f0 >> 5);
+        if (threadIdx.x < VW) {
+            have = __ldcg(un + threadIdx.x);
+            sh[threadIdx.x] = 0;
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void end(uint32_t z) {
+        const int lane = threadIdx.x & 31;
+        uint32_t x = z << ((lane * VW) & 31);
+#pragma unroll
+        for (int o = 1; o < 32 / VW; o <<= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
+        if (x && (lane & (32 / VW - 1)) == 0) atomicOr(sh + (lane * VW >> 5), x);
+        __syncthreads();
+        if (threadIdx.x < VW && (sh[threadIdx.x] & ~have)) atomicOr(un + threadIdx.x, sh[threadIdx.x]);
+    }
+};
+
 // ------------------------------------------------------------------------------------
 // Per-frame state
 // ------------------------------------------------------------------------------------
@@ -633,17 +661,19 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
     using VS = Vec<uint8_t, VW>;
     static_assert(sizeof(VT) == sizeof(T) * VW, "one vector = VW frames");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = blockIdx.x * 4 + warp;
+    const int i = min((int)blockIdx.x * 4 + warp, M - 1);
     const int f0 = (blockIdx.y * 32 + lane) * VW;
-    if (i >= M) return;
+    __shared__ uint32_t fail[VW];
+    CtaFlags<VW> flags;
+    if (do_syn) flags.begin(fail, unsat, blockIdx.y * 32 * VW);
     const VS st = *reinterpret_cast<const VS*>(state + f0);
     const int d = __ldg(ell_deg + i);
     int c[D];
     load_cols<D>(ell_col + (size_t)i * D, c);
-    const uint32_t have = do_syn ? unsat_now(unsat, f0) : 0u;
     uint32_t act = 0;
 #pragma unroll
     for (int v = 0; v < VW; v++) act |= (uint32_t)(st.x[v] != 0) << v;
+    if ((int)blockIdx.x * 4 + warp != i) act = 0;  // past the last row
     uint32_t z = 0;
     if (act) {  // lanes whose frames have all stopped touch nothing
         T* const erow = eta + (size_t)i * D * Fp + f0;
@@ -660,7 +690,7 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
         else z = row_update<MODE, FIRST, true, true, W, VW, D>(row, d, erow, Fp, wt);
     }
     __syncwarp();
-    if (do_syn) flag_unsat<VW>(unsat, f0, z & act, have);
+    if (do_syn) flags.end(z & act);
 }
 
 // ------------------------------------------------------------------------------------
@@ -841,102 +871,138 @@ __global__ void __launch_bounds__(128, V <= 2 ? 8 : 4)
     }
 }
 
-// The check pass on compressed messages of rows without the padded layout (17 to 27 edges), a
-// warp per row of 32 V frames: the row's columns (and, learned, the previous iteration's
-// weights of their classes) come in one load a warp and go to the lanes by shuffles, the
-// posteriors of U edges are requested together, and the row's state is all that is kept of the
-// messages. Bound by the gathers of s, 4 bytes an edge mostly from L2. The pass it replaces
-// (k_check: one dependent gather after another, 8 bytes an edge of messages) and its bit pass
-// took 343 us an iteration of N=16200 (rows of 20-21 edges, 2001 frames), the two now 260 us.
-template <bool FIRST, bool W, int V>
+// The check pass on compressed messages (cmsg.cuh), a warp per row of 32 V frames: D = 8 or 16,
+// the padded rows; D = 0, CSR rows of at most kCmsgMaxRow edges. State, degree and columns come
+// in one round trip, the posteriors of eight edges in the next; the row's state is all that is
+// kept of the messages. The edges are unrolled, so an edge's position is a constant in every
+// pick and shift: the pass is bound by the ALU (about ten instructions an edge and frame) and
+// by DRAM. The staged kernel, which serves staging shapes that were asked for, spends another
+// six an edge and frame on its copies and barriers. A launch, 1024 frames of N=64800: 182 us
+// (5.1 TB/s) against 236 staged, with learned weights and the syndrome 260 us; N=16200 (rows of
+// 20-21 edges), 2001 frames: 79 us. (k_check on per-edge messages with its bit pass took 343
+// us an iteration there, this pass with its bit pass 185.)
+struct CheckRegArgs {
+    const int32_t* col;      // ell_col, or col_idx
+    const uint8_t* ell_deg;  // D > 0
+    const uint8_t* ell_cls;
+    const int32_t* row_ptr;  // D = 0
+    int M, Fp, paper;
+    const uint8_t* state;
+    uint32_t* unsat;
+};
+template <bool FIRST, bool SYN, bool W, int V, int D>
 __global__ void __launch_bounds__(128, 5)
-    k_check_cmp(const int32_t* __restrict__ col_idx, const int32_t* __restrict__ row_ptr, int M,
-                const float* __restrict__ s, CState cs, int Fp, const uint8_t* __restrict__ state,
-                uint32_t* unsat, int do_syn, int paper, IterWeights wt) {
+    k_check_reg(const CheckRegArgs a, const float* __restrict__ s, CState cs, IterWeights wt) {
     using VF = Vec<float, V>;
-    using VU = Vec<uint32_t, V>;
-    FewRow<V> row;
-    row.lane = threadIdx.x & 31;
-    row.i = blockIdx.x * 4 + (threadIdx.x >> 5);
-    row.f0 = (blockIdx.y * 32 + row.lane) * V;
-    if (row.i >= M) return;
+    using VU = CWords<V, D == 8>;
+    using VS = Vec<uint8_t, V>;
+    constexpr int E = D ? D : kCmsgMaxRow, U = 8;
+    const int lane = threadIdx.x & 31, row = blockIdx.x * 4 + (threadIdx.x >> 5), i = min(row, a.M - 1);
+    const int f0 = (blockIdx.y * 32 + lane) * V;
+    __shared__ uint32_t fail[V];
+    CtaFlags<V> flags;
+    if (SYN) flags.begin(fail, a.unsat, blockIdx.y * 32 * V);
+    const VS st = *reinterpret_cast<const VS*>(a.state + f0);
+    int c[U], d;
+    const int32_t* col;
+    uint32_t cls4[D ? D / 4 : 1];  // learned-weight classes of the padded row, a byte an edge
+    if constexpr (D > 0 && W && !FIRST) {
+#pragma unroll
+        for (int q = 0; q < D / 4; q++) cls4[q] = __ldg(reinterpret_cast<const uint32_t*>(a.ell_cls + (size_t)i * D) + q);
+    }
+    if constexpr (D > 0) {
+        col = a.col + (size_t)i * D;
+        d = __ldg(a.ell_deg + i);
+    } else {
+        const int e0 = __ldg(a.row_ptr + i);
+        d = __ldg(a.row_ptr + i + 1) - e0;
+        col = a.col + e0;
+    }
+    auto load_c = [&](int k0) {  // the columns of edges k0 .. k0 + U - 1
+        if constexpr (D > 0) {
+            load_cols<U>(col + k0, c);
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (k0 + u < d) c[u] = __ldg(col + k0 + u);
+        }
+    };
+    load_c(0);
+    const size_t o = (size_t)i * a.Fp + f0;
+    VU* const wp = reinterpret_cast<VU*>(static_cast<unsigned char*>(cs.w) + o * (D == 8 ? 2 : 4));
     VF om0, om1;
     VU ow;
     if (!FIRST) {
-        const size_t o = (size_t)row.i * Fp + row.f0;
         om0 = *reinterpret_cast<const VF*>(cs.m0 + o);
         om1 = *reinterpret_cast<const VF*>(cs.m1 + o);
-        ow = *reinterpret_cast<const VU*>(cs.w + o);
+        ow = *wp;
     }
-    if (!row.load(col_idx, nullptr, row_ptr, 0, state, unsat, do_syn)) return;
-    float mywa = 1.0f, mywb = 0.0f;
-    if constexpr (W && !FIRST) {
-        const int c = __ldg(wt.col_class + row.mycol);
-        mywa = __ldg(wt.alpha + c);
-        mywb = __ldg(wt.beta + c);
-    }
-    const int d = row.d;
-    const float* const sp = s + row.fo;
-    const float pm = paper ? -1.0f : 1.0f;
-    float min0[V], min1[V];
-    uint32_t loc[V], sg[V], zx[V];
+    uint32_t act = 0, z = 0;
 #pragma unroll
-    for (int v = 0; v < V; v++) {
-        min0[v] = min1[v] = big(0.0f);
-        loc[v] = sg[v] = zx[v] = 0;
-    }
-    constexpr int U = 8;
-    for (int k0 = 0; k0 < d; k0 += U) {
-        VF sv[U];
+    for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
+    if (row != i) act = 0;  // past the last row
+    if (act) {  // lanes whose frames have all stopped touch nothing
+        const float pm = a.paper ? -1.0f : 1.0f;
+        VF n0, n1;
+        uint32_t loc[V], sg[V], zx[V];
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int c = __shfl_sync(0xffffffffu, row.mycol, (k0 + u) & 31);
-            if (k0 + u < d) sv[u] = ld_nc(reinterpret_cast<const VF*>(sp + (size_t)c * Fp));
+        for (int v = 0; v < V; v++) {
+            n0.x[v] = n1.x[v] = big(0.0f);
+            loc[v] = sg[v] = zx[v] = 0;
         }
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int k = k0 + u;
-            if (k >= d) break;  // the same for the whole warp
-            float wa = 1.0f, wb = 0.0f;
-            if constexpr (W && !FIRST) {
-                wa = __shfl_sync(0xffffffffu, mywa, k);
-                wb = __shfl_sync(0xffffffffu, mywb, k);
-            }
+        for (int k0 = 0; k0 < E; k0 += U) {
+            if (k0 >= d) break;  // d is the same for the whole warp
+            VF sv[U];
+            float wa[U], wb[U];
 #pragma unroll
-            for (int v = 0; v < V; v++) {
-                const float sa = sv[u].x[v];
-                zx[v] ^= dec_sign(sa, pm);
-                float l = sa;
-                if constexpr (!FIRST) {
-                    float m = cmsg_mag(om0.x[v], om1.x[v], ow.x[v], k);
-                    if constexpr (W) m = cmsg_weight(m, wa, wb);
-                    l = sa - cmsg_signed(m, ow.x[v], k);
+            for (int u = 0; u < U; u++)
+                if (k0 + u < d) {
+                    sv[u] = ld_nc(reinterpret_cast<const VF*>(s + (size_t)c[u] * a.Fp + f0));
+                    if constexpr (W && !FIRST) {
+                        const int cl = D > 0 ? (int)(cls4[(k0 + u) / 4 % (D ? D / 4 : 1)] >> ((k0 + u) % 4 * 8) & 255u)
+                                             : (int)__ldg(wt.col_class + c[u]);
+                        wa[u] = __ldg(wt.alpha + cl);
+                        wb[u] = __ldg(wt.beta + cl);
+                    }
                 }
-                const float a = fabsf(l);
-                const bool lt = a < min0[v];  // strict: the first location of min0 stays
-                min1[v] = lt ? min0[v] : fminf(min1[v], a);
-                min0[v] = lt ? a : min0[v];
-                loc[v] = lt ? (uint32_t)k : loc[v];
-                sg[v] = __funnelshift_l(sbits(l), sg[v], 1);  // (sg << 1) | sign of lambda
+            if (k0 + U < E) load_c(k0 + U);
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int t = k0 + u;
+                if (t >= E || t >= d) break;
+#pragma unroll
+                for (int v = 0; v < V; v++) {
+                    const float sa = sv[u].x[v];
+                    if (SYN) zx[v] ^= dec_sign(sa, pm);
+                    float l = sa;
+                    if constexpr (!FIRST) {
+                        float m = ow.mag(om0.x[v], om1.x[v], v, t);
+                        if constexpr (W) m = cmsg_weight(m, wa[u], wb[u]);
+                        l = sa - ow.signed_mag(m, v, t);
+                    }
+                    const float x = fabsf(l);
+                    const bool lt = x < n0.x[v];  // strict: the first location of min0 stays
+                    n1.x[v] = lt ? n0.x[v] : fminf(n1.x[v], x);
+                    n0.x[v] = lt ? x : n0.x[v];
+                    loc[v] = lt ? (uint32_t)t : loc[v];
+                    sg[v] = __funnelshift_l(sbits(l), sg[v], 1);  // (sg << 1) | sign of lambda
+                }
             }
         }
-    }
-    uint32_t z = 0;
-    VF n0, n1;
-    VU nw;
 #pragma unroll
-    for (int v = 0; v < V; v++) {
-        z |= (zx[v] >> 31) << v;
-        n0.x[v] = min0[v];
-        n1.x[v] = min1[v];
-        nw.x[v] = cmsg_word(sg[v], d, loc[v]);
+        for (int v = 0; v < V; v++) {
+            z |= (zx[v] >> 31) << v;
+            sg[v] = cmsg_word(sg[v], d, loc[v]);
+        }
+        VU nw;
+        nw.set(sg);
+        *reinterpret_cast<VF*>(cs.m0 + o) = n0;
+        *reinterpret_cast<VF*>(cs.m1 + o) = n1;
+        *wp = nw;
     }
-    if (do_syn) flag_unsat<V>(unsat, row.f0, z & row.act, row.have);
-    if (!row.on) return;
-    const size_t o = (size_t)row.i * Fp + row.f0;
-    *reinterpret_cast<VF*>(cs.m0 + o) = n0;
-    *reinterpret_cast<VF*>(cs.m1 + o) = n1;
-    *reinterpret_cast<VU*>(cs.w + o) = nw;
+    __syncwarp();
+    if (SYN) flags.end(z & act);
 }
 
 // The final syndrome of few frames, and of any number on rows of 17 to 32 edges.
@@ -1070,14 +1136,15 @@ __device__ __forceinline__ uint32_t row_update_cmp(const unsigned char* st, int 
                                                    const float* wbeta, const CState& cs, size_t off) {
     static_assert(D <= kCmsgMaxRow, "the signs and the location fit the word");
     using VF = Vec<float, VW>;
-    using VU = Vec<uint32_t, VW>;
+    using VU = CWords<VW, D == 8>;
     auto at = [&](int c) { return st + (size_t)c * chunk + (size_t)lane * sizeof(VF); };
+    static_assert(sizeof(VU) == VW * (D == 8 ? 2 : 4), "the words of a lane");
     VF om0, om1;
     VU ow;
     if (!FIRST) {
         om0 = *reinterpret_cast<const VF*>(at(D));
         om1 = *reinterpret_cast<const VF*>(at(D + 1));
-        ow = *reinterpret_cast<const VU*>(at(D + 2));
+        ow = *reinterpret_cast<const VU*>(st + (size_t)(D + 2) * chunk + (size_t)lane * sizeof(VU));
     }
     float min0[VW], min1[VW];
     uint32_t loc[VW], sg[VW], zx[VW];  // sg: lambda's sign bits, the first edge's highest
@@ -1105,9 +1172,9 @@ __device__ __forceinline__ uint32_t row_update_cmp(const unsigned char* st, int 
                 if (SYN) zx[v] ^= PAPER ? sbits(0.0f - sa) : sbits(sa);
                 float l = sa;
                 if constexpr (!FIRST) {
-                    float m = cmsg_mag(om0.x[v], om1.x[v], ow.x[v], t);
+                    float m = ow.mag(om0.x[v], om1.x[v], v, t);
                     if constexpr (W) m = cmsg_weight(m, wa, wb);
-                    l = sa - cmsg_signed(m, ow.x[v], t);
+                    l = sa - ow.signed_mag(m, v, t);
                 }
                 const float a = fabsf(l);
                 const bool lt = a < min0[v];  // strict: the first location of min0 stays
@@ -1128,11 +1195,12 @@ __device__ __forceinline__ uint32_t row_update_cmp(const unsigned char* st, int 
     for (int v = 0; v < VW; v++) {
         n0.x[v] = min0[v];
         n1.x[v] = min1[v];
-        nw.x[v] = cmsg_word(sg[v], d, loc[v]);
+        sg[v] = cmsg_word(sg[v], d, loc[v]);
     }
+    nw.set(sg);
     *reinterpret_cast<VF*>(cs.m0 + off) = n0;
     *reinterpret_cast<VF*>(cs.m1 + off) = n1;
-    *reinterpret_cast<VU*>(cs.w + off) = nw;
+    *reinterpret_cast<VU*>(static_cast<unsigned char*>(cs.w) + off * (sizeof(VU) / VW)) = nw;
     return z;
 }
 
@@ -1267,7 +1335,9 @@ __global__ void __launch_bounds__(kStagedMaxThreads) k_check_staged(const Staged
     const int FB = 32 * VW;  // frames per block
     static_assert(!CMP || MODE == kModeFP32, "compressed messages are FP32");
     const uint32_t tx = (FIRST || CMP ? 1u : 2u) * (uint32_t)LY::kChunk;  // per edge
-    const uint32_t tx_row = (CMP && !FIRST) ? 3u * (uint32_t)LY::kChunk : 0u;  // per row
+    // per row: m0, m1 and the words (half as many bytes on rows of 8 slots)
+    constexpr uint32_t w_bytes = D == 8 ? LY::kChunk / 2 : LY::kChunk;
+    const uint32_t tx_row = (CMP && !FIRST) ? 2u * (uint32_t)LY::kChunk + w_bytes : 0u;
     const CState cs = CMP ? cstate_at(eta, M, a.Fp) : CState{};
     int ci = first % M, cy = first / M;  // the task being computed
     int ni = ci, ny = cy;                // the next task to issue
@@ -1314,9 +1384,9 @@ __global__ void __launch_bounds__(kStagedMaxThreads) k_check_staged(const Staged
         if (CMP && !FIRST && any && lane >= D && lane < D + 3) {  // the row's old state
             unsigned char* st = buf + (size_t)q * LY::kStage;
             const int c = lane - D;
-            const float* src = c == 0 ? cs.m0 : c == 1 ? cs.m1 : reinterpret_cast<const float*>(cs.w);
-            bulk_g2s(st + (size_t)lane * LY::kChunk, src + (size_t)ni * a.Fp + (size_t)ny * FB, LY::kChunk,
-                     &bar[q], drop_eta);
+            const size_t o = (size_t)ni * a.Fp + (size_t)ny * FB;
+            const void* src = c == 0 ? cs.m0 + o : c == 1 ? cs.m1 + o : static_cast<const void*>(static_cast<const unsigned char*>(cs.w) + o * (D == 8 ? 2 : 4));
+            bulk_g2s(st + (size_t)lane * LY::kChunk, src, c < 2 ? (uint32_t)LY::kChunk : w_bytes, &bar[q], drop_eta);
         }
         pend |= 1u << q;
         ni += di;
@@ -1417,7 +1487,7 @@ __global__ void __launch_bounds__(kStagedMaxThreads) k_check_staged(const Staged
 // registers), which measured faster than fewer, larger-register warps (N=64800 FP32 with
 // compressed messages: 102 -> 96.5 ms per 4096-frame, 50-iteration decode).
 // One task: column j for the V frames at positions f0 .. f0 + V - 1.
-template <int MODE, int VW, bool CMP, bool W, bool HD>
+template <int MODE, int VW, bool CMP, bool W, bool HD, bool H>
 __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restrict__ col_ptr,
                                          const int32_t* __restrict__ col_edge,
                                          const typename Tr<MODE>::R* __restrict__ r,
@@ -1463,7 +1533,7 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
     if constexpr (CMP) {
         static_assert(MODE == kModeFP32, "compressed messages are FP32");
         using VF = Vec<float, V>;
-        using VU = Vec<uint32_t, V>;
+        using VU = CWords<V, H>;
         float wa = 1.0f, wb = 0.0f;
         if constexpr (W) {
             const int c = __ldg(wt.col_class + j);
@@ -1480,12 +1550,12 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
             const int tp = slot & tmask;
             const VF m0 = ld_nc(reinterpret_cast<const VF*>(cs.m0 + o));
             const VF m1 = ld_nc(reinterpret_cast<const VF*>(cs.m1 + o));
-            const VU w = ld_nc(reinterpret_cast<const VU*>(cs.w + o));
+            const VU w = ld_nc(reinterpret_cast<const VU*>(static_cast<const unsigned char*>(cs.w) + o * (H ? 2 : 4)));
 #pragma unroll
             for (int v = 0; v < V; v++) {
-                float m = cmsg_mag(m0.x[v], m1.x[v], w.x[v], tp);
+                float m = w.mag(m0.x[v], m1.x[v], v, tp);
                 if constexpr (W) m = cmsg_weight(m, wa, wb);
-                acc[v] = acc[v] + (A)cmsg_signed(m, w.x[v], tp);
+                acc[v] = acc[v] + (A)w.signed_mag(m, v, tp);
             }
         }
     } else if constexpr (MODE == kModeFixed && V % 2 == 0) {
@@ -1538,6 +1608,9 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
     }
 }
 
+// The frame blocks go in the opposite order of the check pass, so that each pass begins with the
+// blocks the other has just left in L2 (N=64800 in fixed point with early stop, 1000 frames:
+// 15.4 -> 15.0 ms).
 // The bit pass over the positions in use (comp[1]: after a frame compaction the running
 // frames sit at the front): tasks t = y G + c, column group c (4 columns, one per warp) of
 // frame block y (32 lanes x V frames).
@@ -1549,7 +1622,7 @@ __device__ __forceinline__ void var_task(int j, int f0, const int32_t* __restric
 // gathered row states of a frame block are then reused in L2 by the CTAs running together
 // (CTAs that loop over strided tasks drift apart: 20 % slower on the N=64800 code); with
 // per-edge messages the looping form measured 1.7 % slower on the QC N=2304 code.
-template <int MODE, int VW = Tr<MODE>::V, bool CMP = false, bool W = false, bool HD = false>
+template <int MODE, int VW = Tr<MODE>::V, bool CMP = false, bool W = false, bool HD = false, bool H = false>
 __global__ void __launch_bounds__(128, 16) k_var(const int32_t* __restrict__ col_ptr,
                                              const int32_t* __restrict__ col_edge, int N,
                                              const typename Tr<MODE>::R* __restrict__ r,
@@ -1565,12 +1638,12 @@ __global__ void __launch_bounds__(128, 16) k_var(const int32_t* __restrict__ col
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int FB = 32 * VW;
     if constexpr (MODE == kModeFP32) {
-        const int j = blockIdx.x * 4 + warp, y = blockIdx.y;
+        const int j = blockIdx.x * 4 + warp, y = gridDim.y - 1 - blockIdx.y;
         const int cur = __ldcg(comp + 1), done = *(volatile const int*)n_done;  // one round trip
         if (j >= N || y * FB >= cur || done >= frames) return;
-        var_task<MODE, VW, CMP, W, HD>(j, (y * 32 + lane) * VW, col_ptr, col_edge, r, s, eta, Fp, state,
-                                       done_iter, pos2frame, unsat, test_prev, k, n_done, cs, dshift, wt,
-                                       hd, paper);
+        var_task<MODE, VW, CMP, W, HD, H>(j, (y * 32 + lane) * VW, col_ptr, col_edge, r, s, eta, Fp, state,
+                                          done_iter, pos2frame, unsat, test_prev, k, n_done, cs, dshift, wt,
+                                          hd, paper);
         return;
     }
     if (*(volatile const int*)n_done >= frames) return;
@@ -1581,8 +1654,8 @@ __global__ void __launch_bounds__(128, 16) k_var(const int32_t* __restrict__ col
     for (; y < nb;) {
         const int j = c * 4 + warp;
         if (j < N)
-            var_task<MODE, VW, CMP, W, HD>(j, (y * 32 + lane) * VW, col_ptr, col_edge, r, s, eta, Fp, state,
-                                           done_iter, pos2frame, unsat, test_prev, k, n_done, cs, dshift,
+            var_task<MODE, VW, CMP, W, HD, H>(j, ((nb - 1 - y) * 32 + lane) * VW, col_ptr, col_edge, r, s, eta, Fp,
+                                              state, done_iter, pos2frame, unsat, test_prev, k, n_done, cs, dshift,
                                            wt, hd, paper);
         y += step_y;
         c += step_c;
@@ -1851,14 +1924,19 @@ bool staged(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
 template <int V, bool FIRST, bool W>
 bool check_pass_cmp(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, const float* s,
                     float* state, uint32_t* un, int test_prev, const IterWeights& wt_prev, cudaStream_t st) {
+    if constexpr (V == 4) {
+        if (w.auto_staging || g.ell_D == 0) {
+            auto kern = g.ell_D == 8    ? (test_prev ? k_check_reg<FIRST, true, W, V, 8> : k_check_reg<FIRST, false, W, V, 8>)
+                        : g.ell_D == 16 ? (test_prev ? k_check_reg<FIRST, true, W, V, 16> : k_check_reg<FIRST, false, W, V, 16>)
+                                        : (test_prev ? k_check_reg<FIRST, true, W, V, 0> : k_check_reg<FIRST, false, W, V, 0>);
+            const CheckRegArgs ra{g.ell_D ? g.ell_col : g.col_idx, g.ell_deg, g.ell_cls, g.row_ptr, a.M, w.Fp,
+                                  a.paper_slicer, w.state, un};
+            kern<<<dim3((a.M + 3) / 4, w.Fp / (32 * V)), 128, 0, st>>>(ra, s, cstate_at(state, a.M, w.Fp), wt_prev);
+            return true;
+        }
+    }
     if (g.ell_D == 8) return staged<kModeFP32, V, FIRST, W, 8, true>(g, a, w, s, state, un, test_prev, wt_prev, st);
     if (g.ell_D == 16) return staged<kModeFP32, V, FIRST, W, 16, true>(g, a, w, s, state, un, test_prev, wt_prev, st);
-    if constexpr (V == 4) {
-        k_check_cmp<FIRST, W, V><<<dim3((a.M + 3) / 4, w.Fp / (32 * V)), 128, 0, st>>>(
-            g.col_idx, g.row_ptr, a.M, s, cstate_at(state, a.M, w.Fp), w.Fp, w.state, un, test_prev,
-            a.paper_slicer, wt_prev);
-        return true;
-    }
     return false;
 }
 
@@ -1926,7 +2004,10 @@ int compact(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStr
     if (cmp) {  // the rows' compressed messages: m0 and m1 (binary32), then the words
         const CState cs = cstate_at(w.eta, a.M, Fp);
         k_cmp_rows<float><<<blocks, 256, 0, st>>>(cs.m0, 2ll * a.M, Fp, w.new_pos, w.comp);
-        k_cmp_rows<uint32_t><<<blocks, 256, 0, st>>>(cs.w, (long long)a.M, Fp, w.new_pos, w.comp);
+        if (g.ell_D == 8)
+            k_cmp_rows<uint16_t><<<blocks, 256, 0, st>>>((uint16_t*)cs.w, (long long)a.M, Fp, w.new_pos, w.comp);
+        else
+            k_cmp_rows<uint32_t><<<blocks, 256, 0, st>>>((uint32_t*)cs.w, (long long)a.M, Fp, w.new_pos, w.comp);
     } else {
         k_cmp_rows<T><<<blocks, 256, 0, st>>>((T*)w.eta, (long long)g.eta_slots, Fp, w.new_pos, w.comp,
                                               g.ell_D ? g.ell_deg : nullptr, g.ell_D ? g.ell_D : 1);
@@ -1939,7 +2020,7 @@ int compact(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStr
 }
 
 // One bit pass of iteration k; hd: the HD variant (the last iteration, decisions packed).
-template <int MODE, int V, bool CMP, bool W>
+template <int MODE, int V, bool CMP, bool W, bool H = false>
 void var_pass(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, dim3 gv, const int32_t* cslot,
               uint32_t* un, int test_prev, int k, bool hd, const CState& cs, int dshift,
               const IterWeights& wt, cudaStream_t st) {
@@ -1954,13 +2035,13 @@ void var_pass(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, dim3 
     } else {
         if constexpr (V == 4 || V == 8) {
             if (hd) {
-                k_var<MODE, V, CMP, W, true><<<gv, 128, 0, st>>>(
+                k_var<MODE, V, CMP, W, true, H><<<gv, 128, 0, st>>>(
                     g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state, w.done_iter, w.pos2frame, un, test_prev, k,
                     w.n_done, a.frames, w.comp, cs, dshift, wt, w.hd, a.paper_slicer);
                 return;
             }
         }
-        k_var<MODE, V, CMP, W><<<gv, 128, 0, st>>>(g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state, w.done_iter,
+        k_var<MODE, V, CMP, W, false, H><<<gv, 128, 0, st>>>(g.col_ptr, cslot, a.N, r, s, eta, w.Fp, w.state, w.done_iter,
                                                    w.pos2frame, un, test_prev, k, w.n_done, a.frames, w.comp, cs,
                                                    dshift, wt);
     }
@@ -2032,12 +2113,9 @@ int run(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, cudaStream_
                                             : check_pass_cmp<V, false, false>(g, a, w, s, (float*)eta, un, test_prev, wp, st));
                 if (ok) {
                     const CState cs = cstate_at(eta, a.M, Fp);
-                    if (W)
-                        var_pass<MODE, V, true, true>(g, a, w, gv, cslot_cmp, un, test_prev, k, hd && k == a.L,
-                                                      cs, dshift, wt, st);
-                    else
-                        var_pass<MODE, V, true, false>(g, a, w, gv, cslot_cmp, un, test_prev, k, hd && k == a.L,
-                                                       cs, dshift, wt, st);
+                    auto pass = g.ell_D == 8 ? (W ? var_pass<MODE, V, true, true, true> : var_pass<MODE, V, true, false, true>)
+                                             : (W ? var_pass<MODE, V, true, true> : var_pass<MODE, V, true, false>);
+                    pass(g, a, w, gv, cslot_cmp, un, test_prev, k, hd && k == a.L, cs, dshift, wt, st);
                     launches += 2;
                     if (may_compact && k < a.L && k % kCompactEvery == 0)
                         launches += compact<MODE>(g, a, w, st, true);
