@@ -43,9 +43,6 @@ struct TrainWork {
     uint32_t* info;  // [T][M][Fp]: the check's word (see above)
 };
 
-// Rows of at most 16 edges keep their sign bits in the check's word.
-constexpr int kPackedSignsMaxRow = 16;
-
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Carve the workspace; returns the bytes needed (and fills w when base != nullptr).
@@ -99,6 +96,9 @@ __global__ void k_lw_in(const float* src, int F, int N, float* dst, int Fp) {
 struct LwArgs {
     const int32_t *row_ptr, *col_idx, *col_ptr, *col_edge;
     const uint8_t* col_class;
+    // padded rows of D slots (rows of at most 16 edges)
+    const int32_t* ell_col;
+    const uint8_t *ell_deg, *ell_cls;
     // row and position in the row of each CSC edge: one word on the padded row layout (rows of
     // at most 16 edges) and for rows of at most 27, else the two arrays
     const int32_t *ell_cslot, *col_row;
@@ -150,6 +150,22 @@ __device__ __forceinline__ void edge_at(const LwArgs& a, int q, int& i, int& k) 
     }
 }
 
+// Eight columns of a padded row from edge k0 on, and the class of an edge from the row's bytes.
+__device__ __forceinline__ void load_cols8(const int32_t* p, int (&c)[8]) {
+    const int4 x = __ldg(reinterpret_cast<const int4*>(p)), y = __ldg(reinterpret_cast<const int4*>(p) + 1);
+    c[0] = x.x, c[1] = x.y, c[2] = x.z, c[3] = x.w;
+    c[4] = y.x, c[5] = y.y, c[6] = y.z, c[7] = y.w;
+}
+template <int D>
+struct RowClasses {
+    uint32_t x[D ? D / 4 : 1];
+    __device__ __forceinline__ void load(const uint8_t* p) {
+#pragma unroll
+        for (int q = 0; q < D / 4; q++) x[q] = __ldg(reinterpret_cast<const uint32_t*>(p) + q);
+    }
+    __device__ __forceinline__ int at(int k) const { return (int)(x[D ? k / 4 : 0] >> (k % 4 * 8) & 255u); }
+};
+
 // max(fma(alpha, m, -beta), 0) with the sign bit of `flip`.
 __device__ __forceinline__ float lw_message(float m, float alpha, float beta, uint32_t flip) {
     const float g = __fmaf_rn(alpha, m, -beta);
@@ -161,23 +177,37 @@ __device__ __forceinline__ float lw_message(float m, float alpha, float beta, ui
 // messages of iteration t - 1 are rebuilt from its saved state (12 bytes a row instead of 4
 // an edge, and no message is ever written), so the pass reads each edge's s, gathered, and
 // the row's state twice 12 bytes. PK: the row's sign bits go to its word (rows of at most 16
-// edges). Bound by the latency of its gathers (index, then s). With the posteriors written
+// edges), the padded rows are unrolled (D = 8 or 16; D = 0: longer rows), so that an edge's
+// position is a constant in every pick, shift and location, and eight gathers are in flight.
+// A launch on N=64800, 256 frames: 112 -> 67 us (with three classes of weights), the adjoint's
+// row pass, unrolled likewise, 146 -> 82 us; whole training steps 8.5 -> 6.55 ms, and on N=576,
+// 4096 frames, 10 iterations, 0.61 -> 0.52 ms. With the posteriors written
 // by the bit pass itself, a training step went from 0.87 to 0.61 ms (N=576, 4096 frames, 10
 // iterations) and from 12.7 to 8.5 ms (N=64800, 256 frames, 20 iterations: this pass 167 ->
 // 108 us, the bit pass with its output 176 -> 84 us a launch).
-template <int V, bool FIRST, bool PK>
-__global__ void __launch_bounds__(128) k_lw_check(LwArgs a, TrainWork w, int t) {
+template <int V, bool FIRST, int D>
+__global__ void __launch_bounds__(128, 4) k_lw_check(LwArgs a, TrainWork w, int t) {
+    constexpr bool PK = D > 0;
     const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
     const int f0 = (blockIdx.y * 32 + (threadIdx.x & 31)) * V;
     const int Fp = a.Fp;
     if (i >= a.M || f0 >= Fp) return;
-    const int e0 = __ldg(a.row_ptr + i), d = __ldg(a.row_ptr + i + 1) - e0;
+    const bool one = a.C == 1;
+    int e0 = 0, d, c8[8];
+    RowClasses<D> rc;
+    if constexpr (PK) {
+        d = __ldg(a.ell_deg + i);
+        load_cols8(a.ell_col + (size_t)i * D, c8);
+        if (!FIRST && !one) rc.load(a.ell_cls + (size_t)i * D);
+    } else {
+        e0 = __ldg(a.row_ptr + i);
+        d = __ldg(a.row_ptr + i + 1) - e0;
+    }
     const float* s = FIRST ? w.r : w.s;
     const size_t ri = ((size_t)(t - 1) * a.M + i) * Fp + f0, rp = ri - (size_t)a.M * Fp;
     uint8_t* sg = PK ? nullptr : w.sg + (size_t)(t - 1) * (size_t)a.E * Fp + (size_t)e0 * Fp + f0;
     const float* al = a.alpha + (size_t)(FIRST ? 0 : t - 2) * a.C;
     const float* be = a.beta + (size_t)(FIRST ? 0 : t - 2) * a.C;
-    const bool one = a.C == 1;
     LV<float, V> om0, om1;
     LV<uint32_t, V> oinfo;
     uint32_t osx[V];  // PK: sign of the old message to edge k at bit k
@@ -202,23 +232,12 @@ __global__ void __launch_bounds__(128) k_lw_check(LwArgs a, TrainWork w, int t) 
         loc[v] = loc2[v] = 0;
         par[v] = sgw[v] = 0;
     }
-    constexpr int U = 4;  // gathers in flight together
-    for (int k0 = 0; k0 < d; k0 += U) {
-        int c[U];
-        LV<float, V> sv[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) c[u] = __ldg(a.col_idx + e0 + min(k0 + u, d - 1));
-#pragma unroll
-        for (int u = 0; u < U; u++) sv[u] = ldv<V>(s + (size_t)c[u] * Fp + f0);
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int k = k0 + u;
-            if (k >= d) break;  // the same for the whole warp
+    auto edge = [&](const int k, const int col, const LV<float, V>& sv) {
             float ak = al1, bk = be1;
             LV<uint8_t, V> sb;
             if (!FIRST) {
                 if (!one) {
-                    const int cls = __ldg(a.col_class + c[u]);
+                    const int cls = PK ? rc.at(k) : (int)__ldg(a.col_class + col);
                     ak = __ldg(al + cls);
                     bk = __ldg(be + cls);
                 }
@@ -227,7 +246,7 @@ __global__ void __launch_bounds__(128) k_lw_check(LwArgs a, TrainWork w, int t) 
             LV<uint8_t, V> nb;
 #pragma unroll
             for (int v = 0; v < V; v++) {
-                float lam = sv[u].x[v];
+                float lam = sv.x[v];
                 if (!FIRST) {
                     const float m = k == info_loc<PK>(oinfo.x[v]) ? om1.x[v] : om0.x[v];
                     const uint32_t flip =
@@ -235,10 +254,10 @@ __global__ void __launch_bounds__(128) k_lw_check(LwArgs a, TrainWork w, int t) 
                     lam = lam - lw_message(m, ak, bk, flip);
                 }
                 const float m = fabsf(lam);
-                const uint32_t neg = lam < 0.0f;
-                if (PK) {
-                    sgw[v] |= neg << k;
+                if (PK) {  // (sgw << 1) | [lambda < 0]: "+ 0" leaves no -0 and no negative NaN
+                    sgw[v] = __funnelshift_l(__float_as_uint(lam + 0.0f), sgw[v], 1);
                 } else {
+                    const uint32_t neg = lam < 0.0f;
                     par[v] ^= neg;
                     nb.x[v] = (uint8_t)neg;
                 }
@@ -249,13 +268,45 @@ __global__ void __launch_bounds__(128) k_lw_check(LwArgs a, TrainWork w, int t) 
                 min0.x[v] = lt0 ? m : min0.x[v];
             }
             if (!PK) stv<V>(sg + (size_t)k * Fp, nb);
+    };
+    if constexpr (PK) {
+#pragma unroll
+        for (int k0 = 0; k0 < D; k0 += 8) {
+            if (k0 >= d) break;  // the same for the whole warp
+            LV<float, V> sv[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+                if (k0 + u < d) sv[u] = ldv<V>(s + (size_t)c8[u] * Fp + f0);
+            if (k0 + 8 < D) load_cols8(a.ell_col + (size_t)i * D + k0 + 8, c8);
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (k0 + u >= d) break;
+                edge(k0 + u, 0, sv[u]);
+            }
+        }
+    } else {
+        constexpr int U = 4;  // gathers in flight together
+        for (int k0 = 0; k0 < d; k0 += U) {
+            int c[U];
+            LV<float, V> sv[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) c[u] = __ldg(a.col_idx + e0 + min(k0 + u, d - 1));
+#pragma unroll
+            for (int u = 0; u < U; u++) sv[u] = ldv<V>(s + (size_t)c[u] * Fp + f0);
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (k0 + u >= d) break;
+                edge(k0 + u, c[u], sv[u]);
+            }
         }
     }
     LV<uint32_t, V> info;
 #pragma unroll
-    for (int v = 0; v < V; v++)
+    for (int v = 0; v < V; v++) {
+        if (PK) sgw[v] = d ? __brev(sgw[v]) >> (32 - d) : 0u;  // the sign of lambda_k to bit k
         info.x[v] = PK ? (uint32_t)loc[v] | ((uint32_t)loc2[v] << 4) | ((__popc(sgw[v]) & 1u) << 8) | (sgw[v] << 16)
                        : (uint32_t)loc[v] | ((uint32_t)loc2[v] << 8) | (par[v] << 16);
+    }
     stv<V>(w.mn0 + ri, min0);
     stv<V>(w.mn1 + ri, min1);
     stv<V>(w.info + ri, info);
@@ -345,9 +396,10 @@ __global__ void __launch_bounds__(256) k_lw_var(LwArgs a, TrainWork w, int t, fl
 // whole training steps (forward and backward): N=576, 4096 frames, 10 iterations 3.89 -> 0.87
 // ms; N=64800, 256 frames, 20 iterations 38.4 -> 12.7 ms.
 constexpr int kLwClasses = 16;
-template <int V, bool LAST, bool PK, int GM>
-__global__ void __launch_bounds__(128) k_lw_bwd_row(LwArgs a, TrainWork w, int t, float* grad_alpha,
-                                                    float* grad_beta) {
+template <int V, bool LAST, int D, int GM>
+__global__ void __launch_bounds__(128, 4) k_lw_bwd_row(LwArgs a, TrainWork w, int t, float* grad_alpha,
+                                                       float* grad_beta) {
+    constexpr bool PK = D > 0;
     extern __shared__ float gacc[];  // GM 0, 1: [2 C][128]; GM 2: [2 C]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int q = threadIdx.x; q < 2 * a.C * (GM == 2 ? 1 : 128); q += 128) gacc[q] = 0.0f;
@@ -361,7 +413,17 @@ __global__ void __launch_bounds__(128) k_lw_bwd_row(LwArgs a, TrainWork w, int t
     const uint8_t* sg = PK ? nullptr : w.sg + (size_t)(t - 1) * (size_t)a.E * Fp;
     float ga = 0.0f, gb = 0.0f;
     for (int i = blockIdx.x * 4 + warp; i < a.M; i += gridDim.x * 4) {
-        const int e0 = __ldg(a.row_ptr + i), d = __ldg(a.row_ptr + i + 1) - e0;
+        int e0 = 0, d, c8[8];
+        RowClasses<D> rc;
+        if constexpr (PK) {
+            d = __ldg(a.ell_deg + i);
+            load_cols8(a.ell_col + (size_t)i * D, c8);
+            if (GM != 0) rc.load(a.ell_cls + (size_t)i * D);
+            if (a.vrow) e0 = __ldg(a.row_ptr + i);
+        } else {
+            e0 = __ldg(a.row_ptr + i);
+            d = __ldg(a.row_ptr + i + 1) - e0;
+        }
         if (d == 0) continue;
         const size_t ri = ((size_t)(t - 1) * a.M + i) * Fp + fo;
         const size_t rv = (a.vrow ? (size_t)e0 : 2 * (size_t)i) * Fp + fo;
@@ -388,26 +450,15 @@ __global__ void __launch_bounds__(128) k_lw_bwd_row(LwArgs a, TrainWork w, int t
                 neg2[v] = (x >> (16 + info_loc2<PK>(x))) & 1u;
             }
         }
-        constexpr int U = 4;  // gathers in flight together
-        for (int k0 = 0; k0 < d; k0 += U) {
-            int c[U];
-            LV<float, V> dv[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) c[u] = __ldg(a.col_idx + e0 + min(k0 + u, d - 1));
-#pragma unroll
-            for (int u = 0; u < U; u++) dv[u] = ldv<V>(w.ds + (size_t)c[u] * Fp + fo);
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int k = k0 + u;
-                if (k >= d) break;  // the same for the whole warp
-                const int cls = GM == 0 ? 0 : __ldg(a.col_class + c[u]);
+        auto edge = [&](const int k, const int col, const LV<float, V>& dv) {
+                const int cls = GM == 0 ? 0 : PK ? rc.at(k) : (int)__ldg(a.col_class + col);
                 const float alpha = __ldg(al + cls), beta = __ldg(be + cls);
                 LV<uint8_t, V> sv;
                 if (!PK) sv = ldv<V>(sg + (size_t)(e0 + k) * Fp + fo);
                 float xa = 0.0f, xb = 0.0f;
 #pragma unroll
                 for (int v = 0; v < V; v++) {
-                    float deta = dv[u].x[v];
+                    float deta = dv.x[v];
                     if (!LAST)
                         deta -= k == info_loc<PK>(pinfo.x[v])    ? p1.x[v]
                                 : k == info_loc2<PK>(pinfo.x[v]) ? p2.x[v]
@@ -449,6 +500,36 @@ __global__ void __launch_bounds__(128) k_lw_bwd_row(LwArgs a, TrainWork w, int t
                         atomicAdd(gacc + 2 * cls, xa);
                         atomicAdd(gacc + 2 * cls + 1, xb);
                     }
+                }
+        };
+        if constexpr (PK) {
+#pragma unroll
+            for (int k0 = 0; k0 < D; k0 += 8) {
+                if (k0 >= d) break;  // the same for the whole warp
+                LV<float, V> dv[8];
+#pragma unroll
+                for (int u = 0; u < 8; u++)
+                    if (k0 + u < d) dv[u] = ldv<V>(w.ds + (size_t)c8[u] * Fp + fo);
+                if (k0 + 8 < D) load_cols8(a.ell_col + (size_t)i * D + k0 + 8, c8);
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    if (k0 + u >= d) break;
+                    edge(k0 + u, 0, dv[u]);
+                }
+            }
+        } else {
+            constexpr int U = 4;  // gathers in flight together
+            for (int k0 = 0; k0 < d; k0 += U) {
+                int c[U];
+                LV<float, V> dv[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) c[u] = __ldg(a.col_idx + e0 + min(k0 + u, d - 1));
+#pragma unroll
+                for (int u = 0; u < U; u++) dv[u] = ldv<V>(w.ds + (size_t)c[u] * Fp + fo);
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (k0 + u >= d) break;
+                    edge(k0 + u, c[u], dv[u]);
                 }
             }
         }
@@ -541,18 +622,19 @@ int lane_frames(int32_t rows, int32_t Fp, int num_sms, const void* work) {
     return V;
 }
 
-template <int V, bool PK>
+// D: slots of a padded row (0: rows of more than 16 edges).
+template <int V, int D>
 void launch_fwd(const LwArgs& a, const TrainWork& w, int t, float* soft, int frames, bool keep,
                 cudaStream_t st) {
     const int fb = (a.Fp + 32 * V - 1) / (32 * V);
     const dim3 gc((a.M + 3) / 4, fb);
-    if (t == 1) k_lw_check<V, true, PK><<<gc, 128, 0, st>>>(a, w, t);
-    else k_lw_check<V, false, PK><<<gc, 128, 0, st>>>(a, w, t);
-    k_lw_var<V, PK><<<dim3((a.N + 31) / 32, fb), 256, 0, st>>>(a, w, t, soft, frames, keep);
+    if (t == 1) k_lw_check<V, true, D><<<gc, 128, 0, st>>>(a, w, t);
+    else k_lw_check<V, false, D><<<gc, 128, 0, st>>>(a, w, t);
+    k_lw_var<V, (D > 0)><<<dim3((a.N + 31) / 32, fb), 256, 0, st>>>(a, w, t, soft, frames, keep);
 }
 
 // grad_prev (nullable): the loss gradient of the posteriors of iteration t - 1.
-template <int V, bool PK>
+template <int V, int D>
 void launch_bwd(const LwArgs& a, const TrainWork& w, int t, bool last, int num_sms, const float* grad_prev,
                 int frames, float* grad_alpha, float* grad_beta, cudaStream_t st) {
     const int fb = (a.Fp + 32 * V - 1) / (32 * V);
@@ -562,18 +644,19 @@ void launch_bwd(const LwArgs& a, const TrainWork& w, int t, bool last, int num_s
     const size_t sm = (size_t)2 * a.C * (gm == 2 ? 1 : 128) * sizeof(float);
     auto go = [&](auto row) { row<<<dim3(gx, fb), 128, sm, st>>>(a, w, t, grad_alpha, grad_beta); };
     if (last) {
-        if (gm == 0) go(k_lw_bwd_row<V, true, PK, 0>);
-        else if (gm == 1) go(k_lw_bwd_row<V, true, PK, 1>);
-        else go(k_lw_bwd_row<V, true, PK, 2>);
+        if (gm == 0) go(k_lw_bwd_row<V, true, D, 0>);
+        else if (gm == 1) go(k_lw_bwd_row<V, true, D, 1>);
+        else go(k_lw_bwd_row<V, true, D, 2>);
     } else {
-        if (gm == 0) go(k_lw_bwd_row<V, false, PK, 0>);
-        else if (gm == 1) go(k_lw_bwd_row<V, false, PK, 1>);
-        else go(k_lw_bwd_row<V, false, PK, 2>);
+        if (gm == 0) go(k_lw_bwd_row<V, false, D, 0>);
+        else if (gm == 1) go(k_lw_bwd_row<V, false, D, 1>);
+        else go(k_lw_bwd_row<V, false, D, 2>);
     }
-    if (t > 1) k_lw_bwd_col<V, PK><<<dim3((a.N + 31) / 32, fb), 256, 0, st>>>(a, w, t, grad_prev, frames);
+    if (t > 1) k_lw_bwd_col<V, (D > 0)><<<dim3((a.N + 31) / 32, fb), 256, 0, st>>>(a, w, t, grad_prev, frames);
 }
 
-bool packed_signs(const HandleView& v) { return v.dg->max_dc <= kPackedSignsMaxRow; }
+// Rows of at most 16 edges (the padded layout) keep their sign bits in the check's word.
+bool packed_signs(const HandleView& v) { return v.dg->ell_D > 0; }
 
 int check_common(const HandleView& v, int32_t frames, int32_t iters, const void* alpha,
                  const void* beta, const void* work, uint64_t work_bytes) {
@@ -592,6 +675,9 @@ LwArgs make_args(const HandleView& v, int32_t Fp, const float* alpha, const floa
     a.col_ptr = v.dg->col_ptr;
     a.col_edge = v.dg->col_edge;
     a.col_class = v.dg->col_class;
+    a.ell_col = v.dg->ell_col;
+    a.ell_deg = v.dg->ell_deg;
+    a.ell_cls = v.dg->ell_cls;
     a.ell_cslot = v.dg->ell_D ? v.dg->ell_cslot : v.dg->row_slot;
     a.col_row = v.dg->col_row;
     a.col_k = v.dg->col_k;
@@ -633,9 +719,10 @@ int ldpc_train_forward(ldpc_t* h, const float* llr, int32_t frames, int32_t iter
     cudaStream_t st = v.stream;
     k_lw_in<<<dim3((v.N + 31) / 32, w.Fp / 32), dim3(32, 8), 0, st>>>(llr, frames, v.N, w.r, w.Fp);
     const int V = lane_frames(v.M, w.Fp, v.num_sms, work);
-    auto step = V == 4   ? (pk ? launch_fwd<4, true> : launch_fwd<4, false>)
-                : V == 2 ? (pk ? launch_fwd<2, true> : launch_fwd<2, false>)
-                         : (pk ? launch_fwd<1, true> : launch_fwd<1, false>);
+    const int D = v.dg->ell_D;  // (set exactly where the signs are packed)
+    auto step = V == 4   ? (D == 8 ? launch_fwd<4, 8> : D == 16 ? launch_fwd<4, 16> : launch_fwd<4, 0>)
+                : V == 2 ? (D == 8 ? launch_fwd<2, 8> : D == 16 ? launch_fwd<2, 16> : launch_fwd<2, 0>)
+                         : (D == 8 ? launch_fwd<1, 8> : D == 16 ? launch_fwd<1, 16> : launch_fwd<1, 0>);
     int launches = 1;
     for (int t = 1; t <= iters; t++) {
         float* out = soft_every ? soft + (size_t)(t - 1) * frames * v.N : t == iters ? soft : nullptr;
@@ -668,12 +755,12 @@ int ldpc_train_backward(ldpc_t* h, int32_t frames, int32_t iters, const float* a
     // ds^T = the loss gradient of the last posteriors
     k_lw_in<<<gi, bi, 0, st>>>(grad_soft + (soft_every ? (size_t)(iters - 1) * plane : 0), frames,
                                v.N, w.ds, w.Fp);
-    const int V = lane_frames(v.M, w.Fp, v.num_sms, work);
+    const int V = lane_frames(v.M, w.Fp, v.num_sms, work), D = v.dg->ell_D;
     int launches = 1;
     for (int t = iters; t >= 1; t--) {
-        auto step = V == 4   ? (pk ? launch_bwd<4, true> : launch_bwd<4, false>)
-                    : V == 2 ? (pk ? launch_bwd<2, true> : launch_bwd<2, false>)
-                             : (pk ? launch_bwd<1, true> : launch_bwd<1, false>);
+        auto step = V == 4   ? (D == 8 ? launch_bwd<4, 8> : D == 16 ? launch_bwd<4, 16> : launch_bwd<4, 0>)
+                    : V == 2 ? (D == 8 ? launch_bwd<2, 8> : D == 16 ? launch_bwd<2, 16> : launch_bwd<2, 0>)
+                             : (D == 8 ? launch_bwd<1, 8> : D == 16 ? launch_bwd<1, 16> : launch_bwd<1, 0>);
         step(a, w, t, t == iters, v.num_sms, soft_every && t > 1 ? grad_soft + (size_t)(t - 2) * plane : nullptr,
              frames, grad_alpha, grad_beta, st);
         launches += t > 1 ? 2 : 1;
