@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/ldpc.h"
@@ -50,6 +51,29 @@ int upload(T** dst, const T* src, size_t n) {
     }
     return LDPC_OK;
 }
+
+// The index arrays of a code in one allocation and one copy, each on a 256-byte boundary (an
+// allocation and a copy of its own cost each of the twenty arrays about 25 us of a handle's
+// creation).
+struct Arena {
+    std::vector<uint8_t> bytes;
+    std::vector<std::pair<void**, size_t>> at;
+    template <typename T>
+    void add(T** dst, const std::vector<T>& v) {
+        const size_t o = (bytes.size() + 255) & ~(size_t)255;
+        bytes.resize(o + std::max<size_t>(1, v.size()) * sizeof(T));  // never a null array
+        if (!v.empty()) std::memcpy(bytes.data() + o, v.data(), v.size() * sizeof(T));
+        at.emplace_back((void**)dst, o);
+    }
+    int upload(void** base) {
+        uint8_t* p;
+        const int rc = ::upload(&p, bytes.data(), bytes.size());
+        *base = p;
+        if (rc != LDPC_OK) return rc;
+        for (auto& x : at) *x.first = p + x.second;
+        return LDPC_OK;
+    }
+};
 }  // namespace
 
 struct ldpc {
@@ -111,11 +135,7 @@ struct ldpc {
 };
 
 static void free_graph(DevGraph& g) {
-    void* ptrs[] = {g.row_ptr, g.col_idx, g.col_ptr, g.col_edge, g.packed, g.r_base,
-                    g.r_deg, g.r_slot_pos, g.c_base, g.c_deg, g.c_slot, g.col_pos,
-                    g.col_class, g.r_slot_cls, g.ell_col, g.ell_deg, g.ell_cslot, g.ell_cls,
-                    g.col_row, g.col_k, g.row_slot, g.idx_blob};
-    for (void* p : ptrs)
+    for (void* p : {g.arena, (void*)g.packed})
         if (p) cudaFree(p);
     g = DevGraph();
 }
@@ -370,27 +390,25 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
     // point never maps or allocates anything itself
     if ((rc = noalloc_setup(h->device)) != LDPC_OK) return bail(fail(rc));
     // CSR / CSC
-    if ((rc = upload(&h->dg.row_ptr, hg.row_ptr.data(), hg.row_ptr.size())) ||
-        (rc = upload(&h->dg.col_idx, hg.col_idx.data(), hg.col_idx.size())) ||
-        (rc = upload(&h->dg.col_ptr, hg.col_ptr.data(), hg.col_ptr.size())) ||
-        (rc = upload(&h->dg.col_edge, hg.col_edge.data(), hg.col_edge.size())))
-        return bail(rc);
+    Arena arena;
+    arena.add(&h->dg.row_ptr, hg.row_ptr);
+    arena.add(&h->dg.col_idx, hg.col_idx);
+    arena.add(&h->dg.col_ptr, hg.col_ptr);
+    arena.add(&h->dg.col_edge, hg.col_edge);
     h->dg.max_dc = hg.max_dc;
     h->dg.eta_slots = hg.E;
     // padded row layout of the streaming kernels (rows of at most 16 edges)
     {
         EllGraph eg;
         if (build_ell(hg, eg)) {
-            if ((rc = upload(&h->dg.ell_col, eg.ell_col.data(), eg.ell_col.size())) ||
-                (rc = upload(&h->dg.ell_deg, eg.ell_deg.data(), eg.ell_deg.size())) ||
-                (rc = upload(&h->dg.ell_cslot, eg.ell_cslot.data(), eg.ell_cslot.size())) ||
-                (rc = upload(&h->dg.ell_cls, eg.ell_cls.data(), eg.ell_cls.size())))
-                return bail(rc);
+            arena.add(&h->dg.ell_col, eg.ell_col);
+            arena.add(&h->dg.ell_deg, eg.ell_deg);
+            arena.add(&h->dg.ell_cslot, eg.ell_cslot);
+            arena.add(&h->dg.ell_cls, eg.ell_cls);
             h->dg.ell_D = eg.D;
             h->dg.eta_slots = (int64_t)hg.M * eg.D;
         } else if (hg.max_dc <= 255) {
-            std::vector<int32_t> col_row((size_t)hg.E), row_of((size_t)hg.E);
-            std::vector<uint8_t> col_k((size_t)hg.E);
+            std::vector<int32_t> row_of((size_t)hg.E);
             for (int32_t i = 0; i < hg.M; i++)
                 for (int32_t e2 = hg.row_ptr[i]; e2 < hg.row_ptr[i + 1]; e2++) row_of[e2] = i;
             // (12 bytes a row of state in the place of 4 an edge; slots in 31 bits)
@@ -400,16 +418,17 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
                     const int32_t e2 = hg.col_edge[q], i = row_of[e2];
                     row_slot[q] = i << kRowSlotShift | (e2 - hg.row_ptr[i]);
                 }
-                if ((rc = upload(&h->dg.row_slot, row_slot.data(), row_slot.size()))) return bail(rc);
+                arena.add(&h->dg.row_slot, row_slot);
             } else {
+                std::vector<int32_t> col_row((size_t)hg.E);
+                std::vector<uint8_t> col_k((size_t)hg.E);
                 for (int64_t q = 0; q < hg.E; q++) {
                     const int32_t e2 = hg.col_edge[q];
                     col_row[q] = row_of[e2];
                     col_k[q] = (uint8_t)(e2 - hg.row_ptr[row_of[e2]]);
                 }
-                if ((rc = upload(&h->dg.col_row, col_row.data(), col_row.size())) ||
-                    (rc = upload(&h->dg.col_k, col_k.data(), col_k.size())))
-                    return bail(rc);
+                arena.add(&h->dg.col_row, col_row);
+                arena.add(&h->dg.col_k, col_k);
             }
         }
     }
@@ -417,7 +436,7 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
     h->class_degree = hg.class_degree;
     h->dg.n_classes = (int32_t)hg.class_degree.size();
     if (h->dg.n_classes > 255) h->dg.n_classes = 0;  // weights unsupported for such codes
-    if ((rc = upload(&h->dg.col_class, hg.col_class.data(), hg.col_class.size()))) return bail(rc);
+    arena.add(&h->dg.col_class, hg.col_class);
     // bit-packed rows
     {
         const int64_t W = (hg.N + 31) / 32;
@@ -435,15 +454,7 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
         d.n_cslices = sg.n_cslices;
         d.E_pad = sg.E_pad;
         d.Ec_pad = sg.Ec_pad;
-        if ((rc = upload(&d.r_base, sg.r_base.data(), sg.r_base.size())) ||
-            (rc = upload(&d.r_deg, sg.r_deg.data(), sg.r_deg.size())) ||
-            (rc = upload(&d.r_slot_pos, sg.r_slot_pos.data(), sg.r_slot_pos.size())) ||
-            (rc = upload(&d.c_base, sg.c_base.data(), sg.c_base.size())) ||
-            (rc = upload(&d.c_deg, sg.c_deg.data(), sg.c_deg.size())) ||
-            (rc = upload(&d.c_slot, sg.c_slot.data(), sg.c_slot.size())) ||
-            (rc = upload(&d.col_pos, sg.col_pos.data(), sg.col_pos.size())) ||
-            (rc = upload(&d.r_slot_cls, sg.r_slot_cls.data(), sg.r_slot_cls.size())))
-            return bail(rc);
+        arena.add(&d.r_slot_cls, sg.r_slot_cls);
         const IdxLayout I = idx_layout(sg.E_pad, sg.Ec_pad, sg.n_rslices, sg.n_cslices, hg.N);
         std::vector<uint8_t> blob(I.total, 0);
         auto put = [&](uint32_t at, const auto& v) { std::memcpy(blob.data() + at, v.data(), v.size() * sizeof(v[0])); };
@@ -454,9 +465,21 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
         put(I.cdeg, sg.c_deg);
         put(I.rbase, sg.r_base);
         put(I.cbase, sg.c_base);
-        if ((rc = upload(&d.idx_blob, blob.data(), blob.size()))) return bail(rc);
+        arena.add(&d.idx_blob, blob);
         d.sliced = 1;
         replan(h);
+    }
+    if ((rc = arena.upload(&h->dg.arena))) return bail(rc);
+    if (h->dg.sliced) {  // the index arrays of the resident kernels are parts of the one array
+        DevGraph& d = h->dg;
+        const IdxLayout I = idx_layout(d.E_pad, d.Ec_pad, d.n_rslices, d.n_cslices, hg.N);
+        d.r_slot_pos = (uint16_t*)(d.idx_blob + I.rpos);
+        d.c_slot = (uint16_t*)(d.idx_blob + I.cslot);
+        d.col_pos = (uint16_t*)(d.idx_blob + I.cpos);
+        d.r_deg = d.idx_blob + I.rdeg;
+        d.c_deg = d.idx_blob + I.cdeg;
+        d.r_base = (int32_t*)(d.idx_blob + I.rbase);
+        d.c_base = (int32_t*)(d.idx_blob + I.cbase);
     }
     e = cudaMalloc((void**)&h->counters, 8 * sizeof(int32_t));
     if (e != cudaSuccess) return bail(alloc_fail(e));

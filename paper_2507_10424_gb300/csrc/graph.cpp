@@ -170,6 +170,22 @@ static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of
         for (int32_t e = g.row_ptr[i]; e < g.row_ptr[i + 1]; e++) row_of[e] = i;
     for (int64_t q = 0; q < g.E; q++) lane[q] = (uint8_t)(lane_of_row[row_of[g.col_edge[q]]] % group);
     uint8_t cnt[kMaxDeg][32], most[kMaxDeg];
+    {  // an order with little to gain (up to 32 groups looked at) stays as it is
+        int sum = 0, least = 0;
+        for (int32_t p = 0; p + group <= N; p += group * std::max(1, N / group / 32)) {
+            std::memset(cnt, 0, sizeof(cnt));
+            std::memset(most, 0, sizeof(most));
+            for (int32_t x = p; x < p + group; x++) {
+                const int32_t q = g.col_ptr[order[x]], d = std::min<int32_t>(g.col_ptr[order[x] + 1] - q, kMaxDeg);
+                for (int t = 0; t < d; t++) most[t] = std::max(most[t], ++cnt[t][lane[q + t]]);
+            }
+            for (int t = 0; t < kMaxDeg; t++) {
+                sum += most[t];
+                least += most[t] > 0;
+            }
+        }
+        if (4 * sum <= 5 * least) return;
+    }
     std::vector<int32_t> out;
     out.reserve(N);
     std::vector<int32_t> win;  // the columns to choose from, in order

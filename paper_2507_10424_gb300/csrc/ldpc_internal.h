@@ -173,6 +173,7 @@ struct DevGraph {
     uint8_t* r_slot_cls = nullptr;
     int32_t n_rslices = 0, n_cslices = 0, E_pad = 0, Ec_pad = 0;
     uint8_t* idx_blob = nullptr;  // the arrays above but r_slot_cls, laid out by idx_layout
+    void* arena = nullptr;        // the allocation that holds every array but `packed`
     int32_t sliced = 0;  // the sliced layout exists
     int32_t max_dc = 0;  // longest row (set for every code)
     // padded row layout (streaming kernels); ell_D = 0 when absent
