@@ -154,8 +154,9 @@ static int32_t make_slices(const std::vector<int32_t>& ptr, const std::vector<in
 // 32 / V. Each place takes, from the next columns in order, one that adds the fewest
 // wavefronts to its group (over the column's edges: those whose bank already has the most
 // lanes of the group). Random codes went from 2.6 wavefronts a group of 8 lanes to 1.6 (a
-// window of 64), of 16 from 3.1 to 2.0, of 32 from 3.5 to 2.6; a quasi-cyclic code has none to
-// save and keeps its order. The window shrinks with N so that the search stays under half a
+// window of 64), of 16 from 3.1 to 2.0, of 32 from 3.5 to 2.6; quasi-cyclic codes start below
+// 1.5 (2112: 1.24), which the search makes worse (1.40, and a decode 3 % slower): they keep
+// theirs. The window shrinks with N so that the search stays under half a
 // millisecond. A decode of 4096 frames, (3,6) code, before and after: N=576, 10 iterations 89
 // -> 76 us, N=1500 254 -> 216 us; N=576 with early stop, 65536 frames, 1420 -> 1214 us.
 static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of_row, int group,
@@ -170,13 +171,14 @@ static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of
         for (int32_t e = g.row_ptr[i]; e < g.row_ptr[i + 1]; e++) row_of[e] = i;
     for (int64_t q = 0; q < g.E; q++) lane[q] = (uint8_t)(lane_of_row[row_of[g.col_edge[q]]] % group);
     uint8_t cnt[kMaxDeg][32], most[kMaxDeg];
-    {  // an order with little to gain (up to 32 groups looked at) stays as it is
-        int sum = 0, least = 0;
-        for (int32_t p = 0; p + group <= N; p += group * std::max(1, N / group / 32)) {
+    // wavefronts of an order over the wavefronts of one without conflicts
+    auto cost = [&](const std::vector<int32_t>& ord) {
+        int64_t sum = 0, least = 0;
+        for (int32_t p = 0; p < N; p += group) {
             std::memset(cnt, 0, sizeof(cnt));
             std::memset(most, 0, sizeof(most));
-            for (int32_t x = p; x < p + group; x++) {
-                const int32_t q = g.col_ptr[order[x]], d = std::min<int32_t>(g.col_ptr[order[x] + 1] - q, kMaxDeg);
+            for (int32_t x = p; x < std::min(N, p + group); x++) {
+                const int32_t q = g.col_ptr[ord[x]], d = std::min<int32_t>(g.col_ptr[ord[x] + 1] - q, kMaxDeg);
                 for (int t = 0; t < d; t++) most[t] = std::max(most[t], ++cnt[t][lane[q + t]]);
             }
             for (int t = 0; t < kMaxDeg; t++) {
@@ -184,8 +186,10 @@ static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of
                 least += most[t] > 0;
             }
         }
-        if (4 * sum <= 5 * least) return;
-    }
+        return least ? (double)sum / least : 1.0;
+    };
+    const double before = cost(order);
+    if (before <= 1.6) return;  // quasi-cyclic codes: the search would not better their order
     std::vector<int32_t> out;
     out.reserve(N);
     std::vector<int32_t> win;  // the columns to choose from, in order
@@ -197,14 +201,14 @@ static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of
         }
         while (next < N && (int32_t)win.size() < window) win.push_back(order[next++]);
         const int32_t d = g.col_ptr[win[0] + 1] - g.col_ptr[win[0]], dd = std::min(d, kMaxDeg);
-        int best = 0, cost = dd + 1;
-        for (int c = 0; c < (int)win.size() && cost > 0; c++) {
+        int best = 0, least = dd + 1;
+        for (int c = 0; c < (int)win.size() && least > 0; c++) {
             const int32_t q = g.col_ptr[win[c]];
             if (g.col_ptr[win[c] + 1] - q != d) break;  // the degrees stay sorted
             int x = 0;
             for (int t = 0; t < dd; t++) x += cnt[t][lane[q + t]] >= most[t];
-            if (x < cost) {
-                cost = x;
+            if (x < least) {
+                least = x;
                 best = c;
             }
         }
@@ -213,7 +217,7 @@ static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of
         out.push_back(j);
         for (int t = 0; t < dd; t++) most[t] = std::max(most[t], ++cnt[t][lane[q + t]]);
     }
-    order.swap(out);
+    if (cost(out) < before) order.swap(out);
 }
 
 bool build_sliced(const HostGraph& g, SlicedGraph& sg) {
