@@ -41,6 +41,10 @@ struct TrainWork {
     float* mn0;      // [T][M][Fp]
     float* mn1;      // [T][M][Fp]
     uint32_t* info;  // [T][M][Fp]: the check's word (see above)
+    // backward: sums of the weight gradients [C][2] of iterations g0 + 1 .. (0-based rows from
+    // g0 on), in the place of r and s, which only the forward pass uses
+    double* gsum;
+    int32_t g0;
 };
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -397,8 +401,7 @@ __global__ void __launch_bounds__(256) k_lw_var(LwArgs a, TrainWork w, int t, fl
 // ms; N=64800, 256 frames, 20 iterations 38.4 -> 12.7 ms.
 constexpr int kLwClasses = 16;
 template <int V, bool LAST, int D, int GM>
-__global__ void __launch_bounds__(128, 4) k_lw_bwd_row(LwArgs a, TrainWork w, int t, float* grad_alpha,
-                                                       float* grad_beta) {
+__global__ void __launch_bounds__(128, 4) k_lw_bwd_row(LwArgs a, TrainWork w, int t) {
     constexpr bool PK = D > 0;
     extern __shared__ float gacc[];  // GM 0, 1: [2 C][128]; GM 2: [2 C]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -552,18 +555,27 @@ __global__ void __launch_bounds__(128, 4) k_lw_bwd_row(LwArgs a, TrainWork w, in
         for (int q = 0; q < 2 * a.C; q++) gacc[q * 128 + threadIdx.x] = 0.0f;
     __syncthreads();
     for (int q = GM == 2 ? (int)threadIdx.x : warp; q < 2 * a.C; q += GM == 2 ? 128 : 4) {
-        float x;
+        // the lanes' and the blocks' sums meet in 64 bits: up to 128 times some thousand of them
+        double x;
         if constexpr (GM == 2) {
             x = gacc[q];
         } else {
             const float* g = gacc + q * 128 + lane;
-            x = (g[0] + g[32]) + (g[64] + g[96]);
+            x = ((double)g[0] + g[32]) + ((double)g[64] + g[96]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         }
-        if (x != 0.0f && (GM == 2 || lane == 0))
-            atomicAdd((q & 1 ? grad_beta : grad_alpha) + (size_t)(t - 1) * a.C + q / 2, x);
+        if (x != 0.0 && (GM == 2 || lane == 0))
+            atomicAdd(w.gsum + ((size_t)(t - 1 - w.g0) * a.C + q / 2) * 2 + (q & 1), x);
     }
+}
+
+// The summed weight gradients, rounded once.
+__global__ void k_lw_grad(const double* __restrict__ gsum, float* grad_alpha, float* grad_beta, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    grad_alpha[i] = (float)gsum[2 * i];
+    grad_beta[i] = (float)gsum[2 * i + 1];
 }
 
 // ds^(t-1)_j = sum over the edges of bit j of dlambda^t, ascending rows (the pair of each
@@ -636,13 +648,13 @@ void launch_fwd(const LwArgs& a, const TrainWork& w, int t, float* soft, int fra
 // grad_prev (nullable): the loss gradient of the posteriors of iteration t - 1.
 template <int V, int D>
 void launch_bwd(const LwArgs& a, const TrainWork& w, int t, bool last, int num_sms, const float* grad_prev,
-                int frames, float* grad_alpha, float* grad_beta, cudaStream_t st) {
+                int frames, cudaStream_t st) {
     const int fb = (a.Fp + 32 * V - 1) / (32 * V);
     // about 16 blocks an SM (their warps take several rows each)
     const int gx = std::max(1, std::min((a.M + 3) / 4, (16 * num_sms + fb - 1) / fb));
     const int gm = a.C == 1 ? 0 : a.C <= kLwClasses ? 1 : 2;
     const size_t sm = (size_t)2 * a.C * (gm == 2 ? 1 : 128) * sizeof(float);
-    auto go = [&](auto row) { row<<<dim3(gx, fb), 128, sm, st>>>(a, w, t, grad_alpha, grad_beta); };
+    auto go = [&](auto row) { row<<<dim3(gx, fb), 128, sm, st>>>(a, w, t); };
     if (last) {
         if (gm == 0) go(k_lw_bwd_row<V, true, D, 0>);
         else if (gm == 1) go(k_lw_bwd_row<V, true, D, 1>);
@@ -746,24 +758,36 @@ int ldpc_train_backward(ldpc_t* h, int32_t frames, int32_t iters, const float* a
     carve(v.M, v.N, v.E, frames, iters, pk, (char*)work, &w);
     const LwArgs a = make_args(v, w.Fp, alpha, beta);
     cudaStream_t st = v.stream;
-    const size_t gbytes = (size_t)iters * a.C * sizeof(float);
-    if (cudaMemsetAsync(grad_alpha, 0, gbytes, st) != cudaSuccess ||
-        cudaMemsetAsync(grad_beta, 0, gbytes, st) != cudaSuccess)
-        return LDPC_ERR_CUDA;
+    // r and s hold the sums of this many iterations at least (of one in any case: there are no
+    // more classes than bits)
+    w.gsum = (double*)(((uintptr_t)w.r + 7) & ~(uintptr_t)7);
+    const int64_t per = (2 * (int64_t)v.N * w.Fp * 4 - 8) / (16 * a.C);
+    w.g0 = iters;
     const dim3 gi((v.N + 31) / 32, w.Fp / 32), bi(32, 8);
     const size_t plane = (size_t)frames * v.N;
     // ds^T = the loss gradient of the last posteriors
     k_lw_in<<<gi, bi, 0, st>>>(grad_soft + (soft_every ? (size_t)(iters - 1) * plane : 0), frames,
                                v.N, w.ds, w.Fp);
     const int V = lane_frames(v.M, w.Fp, v.num_sms, work), D = v.dg->ell_D;
-    int launches = 1;
+    int launches = 1, g_top = iters;
     for (int t = iters; t >= 1; t--) {
         auto step = V == 4   ? (D == 8 ? launch_bwd<4, 8> : D == 16 ? launch_bwd<4, 16> : launch_bwd<4, 0>)
                     : V == 2 ? (D == 8 ? launch_bwd<2, 8> : D == 16 ? launch_bwd<2, 16> : launch_bwd<2, 0>)
                              : (D == 8 ? launch_bwd<1, 8> : D == 16 ? launch_bwd<1, 16> : launch_bwd<1, 0>);
+        if (t == w.g0) {  // the sums of the next iterations
+            w.g0 = (int32_t)std::max<int64_t>(0, t - per);
+            if (cudaMemsetAsync(w.gsum, 0, (size_t)(t - w.g0) * a.C * 16, st) != cudaSuccess) return LDPC_ERR_CUDA;
+            g_top = t;
+        }
         step(a, w, t, t == iters, v.num_sms, soft_every && t > 1 ? grad_soft + (size_t)(t - 2) * plane : nullptr,
-             frames, grad_alpha, grad_beta, st);
+             frames, st);
         launches += t > 1 ? 2 : 1;
+        if (t - 1 == w.g0) {
+            const int n = (g_top - w.g0) * a.C;
+            const size_t o = (size_t)w.g0 * a.C;
+            k_lw_grad<<<(n + 127) / 128, 128, 0, st>>>(w.gsum, grad_alpha + o, grad_beta + o, n);
+            launches++;
+        }
     }
     *v.last_launches = launches;
     return cudaGetLastError() == cudaSuccess ? LDPC_OK : LDPC_ERR_CUDA;
