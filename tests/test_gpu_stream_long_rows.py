@@ -1,6 +1,7 @@
-"""GPU tests of the streaming variant on rows of 17 to 32 edges and full frame blocks: compressed
-messages (FP32, rows of at most 27 edges) and the register kernels beyond, around the longest
-row and the frame counts of a block, in both modes, against the oracle; learned weights; the
+"""GPU tests of the streaming variant on full frame blocks with automatic staging: compressed
+messages in the register check pass (FP32, padded rows of 8 and 16 slots and rows of up to 27
+edges) and the register kernels beyond, around the longest row of each and the frame counts of
+a block, in both modes, against the oracle; learned weights; the
 messages read back; frame compaction; infinite channel values, whatever the message format."""
 import numpy as np
 import pytest
@@ -18,7 +19,7 @@ def code_of(rows):
         r = np.repeat(np.arange(len(deg)), deg)
         c = 7 * np.arange(deg.sum()) % 180
         return inputs._make_code(len(deg), 180, r, c, "rows of 2 to 27 edges")
-    N, M = {"17": (500, 100), "21": (601, 100), "27": (540, 70), "28": (560, 69), "32": (640, 70)}[rows]
+    N, M = {"8": (480, 204), "9": (480, 190), "16": (480, 102), "17": (500, 100), "21": (601, 100), "27": (540, 70), "28": (560, 69), "32": (640, 70)}[rows]
     return inputs.irregular_code(N, M, [2, 3, 4, 8], [0.3, 0.4, 0.2, 0.1], 9)
 
 
@@ -33,7 +34,7 @@ def decoder(code, mode, compressed=True):
 
 
 @pytest.mark.parametrize("mode", ["fp32", "fixed"])
-@pytest.mark.parametrize("rows", ["mixed", "17", "21", "27", "28", "32"])
+@pytest.mark.parametrize("rows", ["mixed", "8", "9", "16", "17", "21", "27", "28", "32"])
 def test_long_rows_match_oracle(mode, rows):
     import torch
     code = code_of(rows)
@@ -58,7 +59,7 @@ def test_long_rows_match_oracle(mode, rows):
     dec.close()
 
 
-@pytest.mark.parametrize("rows", ["mixed", "21", "32"])
+@pytest.mark.parametrize("rows", ["mixed", "8", "16", "21", "32"])
 def test_long_rows_with_learned_weights(rows):
     import torch
     code = code_of(rows)
@@ -78,9 +79,10 @@ def test_long_rows_with_learned_weights(rows):
         dec.close()
 
 
-def test_long_rows_messages_read_back():
+@pytest.mark.parametrize("rows", ["8", "16", "27"])
+def test_long_rows_messages_read_back(rows):
     import torch
-    code = code_of("27")
+    code = code_of(rows)
     llr = inputs.all_zero_awgn_llr(130, code.N, 4.0, code.design_rate, 2)
     g = oracle.Graph.from_code(code)
     dec = decoder(code, "fp32")
@@ -93,10 +95,11 @@ def test_long_rows_messages_read_back():
 
 
 @pytest.mark.parametrize("conflicts", [False, True])
-@pytest.mark.parametrize("rows", ["mixed", "21"])
+@pytest.mark.parametrize("rows", ["mixed", "8", "16", "21"])
 def test_infinite_channel_values(rows, conflicts):
     """Known bits, down to rows whose second minimum is infinite; with conflicts infinities of
-    both signs meet in a sum (NaN). Both message formats give the same."""
+    both signs meet in a sum (NaN). The register check pass gives what the staged one gives on
+    padded rows, and what per-edge messages give on longer ones."""
     import torch
     code = code_of(rows)
     llr = inputs.all_zero_awgn_llr(140, code.N, 2.0, code.design_rate, 3)
@@ -106,8 +109,12 @@ def test_infinite_channel_values(rows, conflicts):
         if conflicts:
             llr[f, rng.random(code.N) < 0.1] *= -1.0
     got = []
-    for compressed in (False, True):
-        dec = decoder(code, "fp32", compressed)
+    padded = rows in ("8", "16")
+    for reference in (True, False):
+        dec = decoder(code, "fp32", compressed=padded or not reference)
+        if padded and reference:
+            dec.set_stream_staging(8, 2)
+        assert dec.stream_messages_compressed() == (padded or not reference)
         got.append(dec.decode(torch.from_numpy(llr).cuda(), 6, early_stop=False, want_ok=True, want_soft=True))
         torch.cuda.synchronize()
         dec.close()
