@@ -185,7 +185,7 @@ __device__ __forceinline__ float lw_message(float m, float alpha, float beta, ui
 // position is a constant in every pick, shift and location, and eight gathers are in flight.
 // A launch on N=64800, 256 frames: 112 -> 67 us (with three classes of weights), the adjoint's
 // row pass, unrolled likewise, 146 -> 82 us; whole training steps 8.5 -> 6.55 ms, and on N=576,
-// 4096 frames, 10 iterations, 0.61 -> 0.52 ms. With the posteriors written
+// 4096 frames, 10 iterations, 0.61 -> 0.52 ms (0.53 with the gradients summed in 64 bits). With the posteriors written
 // by the bit pass itself, a training step went from 0.87 to 0.61 ms (N=576, 4096 frames, 10
 // iterations) and from 12.7 to 8.5 ms (N=64800, 256 frames, 20 iterations: this pass 167 ->
 // 108 us, the bit pass with its output 176 -> 84 us a launch).
@@ -555,18 +555,18 @@ __global__ void __launch_bounds__(128, 4) k_lw_bwd_row(LwArgs a, TrainWork w, in
         for (int q = 0; q < 2 * a.C; q++) gacc[q * 128 + threadIdx.x] = 0.0f;
     __syncthreads();
     for (int q = GM == 2 ? (int)threadIdx.x : warp; q < 2 * a.C; q += GM == 2 ? 128 : 4) {
-        // the lanes' and the blocks' sums meet in 64 bits: up to 128 times some thousand of them
-        double x;
+        // the blocks' sums, some thousand of them, meet in 64 bits
+        float x;
         if constexpr (GM == 2) {
             x = gacc[q];
         } else {
             const float* g = gacc + q * 128 + lane;
-            x = ((double)g[0] + g[32]) + ((double)g[64] + g[96]);
+            x = (g[0] + g[32]) + (g[64] + g[96]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         }
-        if (x != 0.0 && (GM == 2 || lane == 0))
-            atomicAdd(w.gsum + ((size_t)(t - 1 - w.g0) * a.C + q / 2) * 2 + (q & 1), x);
+        if (x != 0.0f && (GM == 2 || lane == 0))
+            atomicAdd(w.gsum + ((size_t)(t - 1 - w.g0) * a.C + q / 2) * 2 + (q & 1), (double)x);
     }
 }
 
