@@ -447,7 +447,8 @@ int ldpc_get_stream_staging(const ldpc_t *h, int32_t *warps_per_cta, int32_t *st
  * iteration of the handle's last decode, for tests and diagnosis. They are available when
  * that decode (ldpc_decode_ex or a function built on it) ran the streaming variant without
  * early stop and without frame groups, since its messages then remain in the handle's
- * workspace; the resident, cluster and dense variants keep them on chip and discard them.
+ * workspace; the resident, cluster and dense variants keep them on chip and discard them, and
+ * an ldpc_reserve that allocates a larger workspace does too.
  *   frames  how many frames to read (the first ones of that decode), 0 .. its frame count;
  *   out     device float [frames][E], frame-major; edge e in CSR order (rows ascending, the
  *           columns of a row ascending); values in LLR units (fixed mode: eta / 4, exact).

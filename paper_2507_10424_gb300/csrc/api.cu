@@ -125,6 +125,7 @@ struct ldpc {
     // streaming decode without early stop or frame groups), and that decode's mode; 0 when
     // the last decode left none (ldpc_read_messages)
     int32_t msg_frames = 0, msg_mode = kModeFP32;
+    int32_t msg_Fp = 0;              // its frame stride (sw.Fp is the last call's, ldpc_reserve's too)
     int32_t msg_cmp = 0, msg_L = 0;  // that decode kept compressed messages; its iterations
     int32_t st_msg = 1;              // ldpc_set_stream_messages
     // host pipeline staging (2 slots)
@@ -197,6 +198,7 @@ static int ensure_stream_work(ldpc_t* h, int32_t frames, int32_t L, int32_t gran
     const int32_t stride = (frames + granule - 1) / granule * granule;
     const int32_t Fp = (stride + room - 1) / room * room;
     if (Fp > h->sw_cap) {
+        h->msg_frames = 0;  // the messages of the last decode go with the old workspace
         if (h->sw_big) {
             cudaStreamSynchronize(h->stream);
             cudaFree(h->sw_big);
@@ -668,6 +670,7 @@ int ldpc_decode_ex(ldpc_t* h, const void* llr, int32_t llr_dtype, int32_t frames
             n = stream_decode(h->mode, h->dg, a, w, h->stream, vw);
             if (n >= 0 && !a.early_stop) {  // no compaction: position = frame
                 h->msg_frames = frames;
+                h->msg_Fp = w.Fp;
                 h->msg_mode = h->mode;
                 h->msg_cmp = used_cmp;
                 h->msg_L = max_iter;
@@ -1151,7 +1154,9 @@ int ldpc_read_messages(ldpc_t* h, int32_t frames, float* out) {
         wa = h->w_alpha + (size_t)row * h->dg.n_classes;
         wb = h->w_alpha + (size_t)h->w_rows * h->dg.n_classes + (size_t)row * h->dg.n_classes;
     }
-    const int n = stream_read_messages(h->msg_mode, h->dg, h->M, h->E, h->sw, frames, out, h->stream,
+    StreamWork w = h->sw;
+    w.Fp = h->msg_Fp;
+    const int n = stream_read_messages(h->msg_mode, h->dg, h->M, h->E, w, frames, out, h->stream,
                                        h->msg_cmp, wa, wb);
     if (n < 0) {
         cudaError_t e = cudaGetLastError();
