@@ -127,6 +127,9 @@ struct ldpc {
     int32_t msg_frames = 0, msg_mode = kModeFP32;
     int32_t msg_Fp = 0;              // its frame stride (sw.Fp is the last call's, ldpc_reserve's too)
     int32_t msg_cmp = 0, msg_L = 0;  // that decode kept compressed messages; its iterations
+    const float* msg_w = nullptr;    // its weights (device; nullptr: none), which the messages
+    int32_t msg_w_rows = 0;          // are rebuilt with, and their rows
+    float* kept_w = nullptr;         // msg_w's allocation once the handle has other weights
     int32_t st_msg = 1;              // ldpc_set_stream_messages
     // host pipeline staging (2 slots)
     cudaStream_t h2d = nullptr, d2h = nullptr;
@@ -156,6 +159,20 @@ static void free_stream_work(ldpc_t* h) {
     h->sw = StreamWork();
     h->sw_cap = 0;
     h->sw_cap_L = -1;
+}
+
+// Give up the weights in force: freed, or kept for ldpc_read_messages while the last decode's
+// compressed messages are rebuilt with them.
+static void drop_weights(ldpc_t* h) {
+    const float* used = h->msg_frames > 0 && h->msg_cmp ? h->msg_w : nullptr;
+    if (h->kept_w && h->kept_w != used) {
+        cudaFree(h->kept_w);
+        h->kept_w = nullptr;
+    }
+    if (h->w_alpha && h->w_alpha == used) h->kept_w = h->w_alpha;
+    else if (h->w_alpha) cudaFree(h->w_alpha);
+    h->w_alpha = nullptr;
+    h->w_rows = 0;
 }
 
 // Largest batch of one streaming decode (its grids put frame blocks on the y dimension).
@@ -674,6 +691,8 @@ int ldpc_decode_ex(ldpc_t* h, const void* llr, int32_t llr_dtype, int32_t frames
                 h->msg_mode = h->mode;
                 h->msg_cmp = used_cmp;
                 h->msg_L = max_iter;
+                h->msg_w = a.w_alpha;
+                h->msg_w_rows = a.w_rows;
             }
         }
     }
@@ -1062,9 +1081,7 @@ int ldpc_set_weights(ldpc_t* h, int32_t n_rows, const float* alpha, const float*
     if (n_rows > 0 && (!alpha || !beta)) return fail(LDPC_ERR_BAD_POINTER);
     if (n_rows > 0 && h->dg.n_classes == 0) return fail(LDPC_ERR_UNSUPPORTED);
     cudaStreamSynchronize(h->stream);
-    if (h->w_alpha) cudaFree(h->w_alpha);
-    h->w_alpha = nullptr;
-    h->w_rows = 0;
+    drop_weights(h);
     if (n_rows == 0) {
         replan(h);
         return LDPC_OK;
@@ -1149,10 +1166,10 @@ int ldpc_read_messages(ldpc_t* h, int32_t frames, float* out) {
     if (frames > h->msg_frames) return fail(LDPC_ERR_INVALID_ARG);
     if (!is_device_ptr(out)) return fail(LDPC_ERR_BAD_POINTER);
     const float *wa = nullptr, *wb = nullptr;  // weights of the decode's last iteration
-    if (h->msg_cmp && h->w_rows > 0 && h->msg_L > 0) {
-        const int row = std::min(h->msg_L, h->w_rows) - 1;
-        wa = h->w_alpha + (size_t)row * h->dg.n_classes;
-        wb = h->w_alpha + (size_t)h->w_rows * h->dg.n_classes + (size_t)row * h->dg.n_classes;
+    if (h->msg_cmp && h->msg_w && h->msg_L > 0) {
+        const int row = std::min(h->msg_L, h->msg_w_rows) - 1;
+        wa = h->msg_w + (size_t)row * h->dg.n_classes;
+        wb = wa + (size_t)h->msg_w_rows * h->dg.n_classes;
     }
     StreamWork w = h->sw;
     w.Fp = h->msg_Fp;
@@ -1305,6 +1322,7 @@ void ldpc_destroy(ldpc_t* h) {
     for (auto& c : h->dcl) free_cluster(c);
     if (h->counters) cudaFree(h->counters);
     if (h->w_alpha) cudaFree(h->w_alpha);
+    if (h->kept_w) cudaFree(h->kept_w);
     if (h->dense_work) cudaFree(h->dense_work);
     delete h;
 }

@@ -1,6 +1,7 @@
 """GPU tests of ldpc_read_messages after calls that touch the handle between the decode and the
 read: ldpc_reserve, which sets a frame stride of its own, and allocates a workspace of more
-frames, against the oracle's messages."""
+frames, against the oracle's messages; and ldpc_set_weights, which leaves the messages of the
+decode as they were, in either format."""
 import numpy as np
 import pytest
 
@@ -51,4 +52,33 @@ def test_messages_after_reserve(rows, mode, frames):
     assert e.value.status == ldpc.LDPC_ERR_UNSUPPORTED
     dec.decode(x, 3, early_stop=False)
     assert torch.equal(dec.read_messages(frames).cpu(), torch.from_numpy(eta))
+    dec.close()
+
+
+@pytest.mark.parametrize("compressed", [True, False])
+@pytest.mark.parametrize("rows", ["6", "20"])
+def test_messages_after_set_weights(rows, compressed):
+    import torch
+    code = code_of(rows)
+    C = len(oracle.column_classes(code)[1])
+    rng = np.random.default_rng(4)
+    tables = [(rng.uniform(0.6, 1.0, (3, C)).astype(np.float32), rng.uniform(0.0, 0.3, (3, C)).astype(np.float32))
+              for _ in range(3)]
+    x = torch.from_numpy(inputs.all_zero_awgn_llr(130, code.N, 2.0, code.design_rate, 3)).cuda()
+    dec = decoder(code)
+    dec.set_stream_messages(compressed)
+    dec.decode(x, 2, early_stop=False)  # no weights
+    plain = dec.read_messages(130).clone()
+    dec.set_weights(*tables[0])
+    assert torch.equal(dec.read_messages(130), plain)
+    dec.decode(x, 2, early_stop=False)
+    want = dec.read_messages(130).clone()
+    assert not torch.equal(want, plain)
+    for t in tables[1:]:
+        dec.set_weights(*t)
+        assert torch.equal(dec.read_messages(130), want)
+    dec.set_weights(None, None)
+    assert torch.equal(dec.read_messages(130), want)
+    dec.decode(x, 2, early_stop=False)
+    assert torch.equal(dec.read_messages(130), plain)
     dec.close()
