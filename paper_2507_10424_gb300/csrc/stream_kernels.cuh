@@ -15,7 +15,8 @@
 //            (eq. lambda_j); frames whose previous syndrome was zero are frozen there.
 // A final syndrome-only pass gives the status of frames that never stopped early. With
 // early stop the running frames are compacted to the front now and then, and both passes
-// then skip the frame blocks behind the positions in use (comp[1]).
+// then skip the frame blocks behind the positions in use (comp[1]; the register check passes:
+// k_check_reg where its comment says, the others by the frames' states).
 #pragma once
 
 #include "../../include/ldpc.h"
@@ -94,27 +95,29 @@ __device__ __forceinline__ uint32_t unsat_now(const uint32_t* unsat, int f0) {
 // memory (one word per 32 positions) and one read and at most one atomic per word leave the
 // CTA. Reading the words warp by warp, every SM at once from the same L2 lines, made the
 // register check passes a third slower (N=64800, 1024 frames: 217 us with the syndrome, 136 us
-// without). begin: before the rows, all threads; end: after them, all threads.
+// without). begin: before the rows, all threads; end: after them, all threads; sh: 2 VW words.
 template <int VW>
 struct CtaFlags {
-    uint32_t have, *sh, *un;
-    __device__ __forceinline__ void begin(uint32_t* shared, uint32_t* unsat, int block_f0) {
-        sh = shared;
-        un = unsat + (block_f0 >> 5);
+    // the thread's word of the flags so far (an argument of begin)
+    static __device__ __forceinline__ uint32_t now(const uint32_t* unsat, int block_f0) {
+        return threadIdx.x < VW ? __ldcg(unsat + (block_f0 >> 5) + threadIdx.x) : 0u;
+    }
+    static __device__ __forceinline__ void begin(uint32_t* sh, uint32_t have) {
         if (threadIdx.x < VW) {
-            have = __ldcg(un + threadIdx.x);
+            sh[VW + threadIdx.x] = have;
             sh[threadIdx.x] = 0;
         }
         __syncthreads();
     }
-    __device__ __forceinline__ void end(uint32_t z) {
+    static __device__ __forceinline__ void end(uint32_t* sh, uint32_t* unsat, int block_f0, uint32_t z) {
         const int lane = threadIdx.x & 31;
         uint32_t x = z << ((lane * VW) & 31);
 #pragma unroll
         for (int o = 1; o < 32 / VW; o <<= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
         if (x && (lane & (32 / VW - 1)) == 0) atomicOr(sh + (lane * VW >> 5), x);
         __syncthreads();
-        if (threadIdx.x < VW && (sh[threadIdx.x] & ~have)) atomicOr(un + threadIdx.x, sh[threadIdx.x]);
+        if (threadIdx.x < VW && (sh[threadIdx.x] & ~sh[VW + threadIdx.x]))
+            atomicOr(unsat + (block_f0 >> 5) + threadIdx.x, sh[threadIdx.x]);
     }
 };
 
@@ -663,9 +666,8 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = min((int)blockIdx.x * 4 + warp, M - 1);
     const int f0 = (blockIdx.y * 32 + lane) * VW;
-    __shared__ uint32_t fail[VW];
-    CtaFlags<VW> flags;
-    if (do_syn) flags.begin(fail, unsat, blockIdx.y * 32 * VW);
+    __shared__ uint32_t fail[2 * VW];
+    if (do_syn) CtaFlags<VW>::begin(fail, CtaFlags<VW>::now(unsat, blockIdx.y * 32 * VW));
     const VS st = *reinterpret_cast<const VS*>(state + f0);
     const int d = __ldg(ell_deg + i);
     int c[D];
@@ -690,7 +692,7 @@ __global__ void __launch_bounds__(128, D <= 8 ? 4 : 2)
         else z = row_update<MODE, FIRST, true, true, W, VW, D>(row, d, erow, Fp, wt);
     }
     __syncwarp();
-    if (do_syn) flags.end(z & act);
+    if (do_syn) CtaFlags<VW>::end(fail, unsat, blockIdx.y * 32 * VW, z & act);
 }
 
 // ------------------------------------------------------------------------------------
@@ -877,10 +879,23 @@ __global__ void __launch_bounds__(128, V <= 2 ? 8 : 4)
 // kept of the messages. The edges are unrolled, so an edge's position is a constant in every
 // pick and shift: the pass is bound by the ALU (about ten instructions an edge and frame) and
 // by DRAM. The staged kernel, which serves staging shapes that were asked for, spends another
-// six an edge and frame on its copies and barriers. A launch, 1024 frames of N=64800: 182 us
-// (5.1 TB/s) against 236 staged, with learned weights and the syndrome 260 us; N=16200 (rows of
-// 20-21 edges), 2001 frames: 79 us. (k_check on per-edge messages with its bit pass took 343
-// us an iteration there, this pass with its bit pass 185.)
+// six an edge and frame on its copies and barriers. A launch, 1024 frames of N=64800: 183 us
+// (4.9 TB/s) against 224 staged (236 on the 16-bit words); N=16200 (rows of 20-21 edges), 2001
+// frames: 79 us. (k_check on per-edge messages with its bit pass took 343 us an iteration there,
+// this pass with its bit pass 185.)
+// ROWS, the tested passes of padded rows once there are 128 warps of rows an SM: a warp takes
+// four rows, so that the flags cost a quarter, and the CTA first looks whether its frame block
+// lies behind the positions in use or every frame has stopped (in the round trip of its state
+// and flags, and with a quarter of the CTAs to look). One row a warp without the look, which
+// read the row states of such blocks in every iteration, against this, decodes of 50 iterations:
+// N=64800, 4096 frames that all stop early (7 iterations on average) 46.5 -> 40.9 ms (the staged
+// pass, which is bounded too: 42.2), 1024 frames of which none stops 23.4 -> 21.1 ms, with
+// learned weights 24.8 -> 23.4 ms; N=12288 (rows of 13-14 edges), 4096 frames, all stop 7.58 ->
+// 6.92 ms (staged 7.0), 2001 of which none stops (25 iterations) 4.17 -> 4.20 ms. Fewer warps
+// (700 frames there) lose 3 % to the loop. Rows of 17 to 27 edges (no staged pass before it;
+// all 4096 frames stop: 9.3 ms against 10.5) and the passes that test nothing gain nothing from
+// the look and would pay 1 to 2 % for it.
+constexpr int kCheckRegRows = 4;  // rows a warp takes (ROWS)
 struct CheckRegArgs {
     const int32_t* col;      // ell_col, or col_idx
     const uint8_t* ell_deg;  // D > 0
@@ -889,59 +904,72 @@ struct CheckRegArgs {
     int M, Fp, paper;
     const uint8_t* state;
     uint32_t* unsat;
+    const int32_t *comp, *n_done;  // ROWS: positions in use (comp[1]), stopped frames of `frames`
+    int frames;
 };
-template <bool FIRST, bool SYN, bool W, int V, int D>
-__global__ void __launch_bounds__(128, 5)
+template <bool FIRST, bool SYN, bool W, int V, int D, bool ROWS = false>
+__global__ void __launch_bounds__(128, ROWS && W && D == 16 ? 4 : 5)
     k_check_reg(const CheckRegArgs a, const float* __restrict__ s, CState cs, IterWeights wt) {
     using VF = Vec<float, V>;
     using VU = CWords<V, D == 8>;
     using VS = Vec<uint8_t, V>;
     constexpr int E = D ? D : kCmsgMaxRow, U = 8;
-    const int lane = threadIdx.x & 31, row = blockIdx.x * 4 + (threadIdx.x >> 5), i = min(row, a.M - 1);
+    const int lane = threadIdx.x & 31;
     const int f0 = (blockIdx.y * 32 + lane) * V;
-    __shared__ uint32_t fail[V];
-    CtaFlags<V> flags;
-    if (SYN) flags.begin(fail, a.unsat, blockIdx.y * 32 * V);
+    static_assert(!ROWS || (SYN && D > 0), "several rows a warp: the tested passes of padded rows");
     const VS st = *reinterpret_cast<const VS*>(a.state + f0);
-    int c[U], d;
-    const int32_t* col;
-    uint32_t cls4[D ? D / 4 : 1];  // learned-weight classes of the padded row, a byte an edge
-    if constexpr (D > 0 && W && !FIRST) {
-#pragma unroll
-        for (int q = 0; q < D / 4; q++) cls4[q] = __ldg(reinterpret_cast<const uint32_t*>(a.ell_cls + (size_t)i * D) + q);
-    }
-    if constexpr (D > 0) {
-        col = a.col + (size_t)i * D;
-        d = __ldg(a.ell_deg + i);
-    } else {
-        const int e0 = __ldg(a.row_ptr + i);
-        d = __ldg(a.row_ptr + i + 1) - e0;
-        col = a.col + e0;
-    }
-    auto load_c = [&](int k0) {  // the columns of edges k0 .. k0 + U - 1
-        if constexpr (D > 0) {
-            load_cols<U>(col + k0, c);
-        } else {
-#pragma unroll
-            for (int u = 0; u < U; u++)
-                if (k0 + u < d) c[u] = __ldg(col + k0 + u);
+    __shared__ uint32_t fail[2 * V];
+    if constexpr (SYN) {
+        const uint32_t have = CtaFlags<V>::now(a.unsat, blockIdx.y * 32 * V);
+        if constexpr (ROWS) {  // the same for the whole CTA; all four loads in one round trip
+            const int cur = __ldcg(a.comp + 1), done = __ldcg(a.n_done);
+            if ((int)blockIdx.y * 32 * V >= cur || done >= a.frames) return;
         }
-    };
-    load_c(0);
-    const size_t o = (size_t)i * a.Fp + f0;
-    VU* const wp = reinterpret_cast<VU*>(static_cast<unsigned char*>(cs.w) + o * (D == 8 ? 2 : 4));
-    VF om0, om1;
-    VU ow;
-    if (!FIRST) {
-        om0 = *reinterpret_cast<const VF*>(cs.m0 + o);
-        om1 = *reinterpret_cast<const VF*>(cs.m1 + o);
-        ow = *wp;
+        CtaFlags<V>::begin(fail, have);
     }
     uint32_t act = 0, z = 0;
+    auto running = [&] {
 #pragma unroll
-    for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
-    if (row != i) act = 0;  // past the last row
-    if (act) {  // lanes whose frames have all stopped touch nothing
+        for (int v = 0; v < V; v++) act |= (uint32_t)(st.x[v] != 0) << v;
+    };
+    auto one_row = [&](const int row, const int i) {  // row > i: past the last row
+        int c[U], d;
+        const int32_t* col;
+        uint32_t cls4[D ? D / 4 : 1];  // learned-weight classes of the padded row, a byte an edge
+        if constexpr (D > 0 && W && !FIRST) {
+#pragma unroll
+            for (int q = 0; q < D / 4; q++) cls4[q] = __ldg(reinterpret_cast<const uint32_t*>(a.ell_cls + (size_t)i * D) + q);
+        }
+        if constexpr (D > 0) {
+            col = a.col + (size_t)i * D;
+            d = __ldg(a.ell_deg + i);
+        } else {
+            const int e0 = __ldg(a.row_ptr + i);
+            d = __ldg(a.row_ptr + i + 1) - e0;
+            col = a.col + e0;
+        }
+        auto load_c = [&](int k0) {  // the columns of edges k0 .. k0 + U - 1
+            if constexpr (D > 0) {
+                load_cols<U>(col + k0, c);
+            } else {
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    if (k0 + u < d) c[u] = __ldg(col + k0 + u);
+            }
+        };
+        load_c(0);
+        const size_t o = (size_t)i * a.Fp + f0;
+        VU* const wp = reinterpret_cast<VU*>(static_cast<unsigned char*>(cs.w) + o * (D == 8 ? 2 : 4));
+        VF om0, om1;
+        VU ow;
+        if (!FIRST) {
+            om0 = *reinterpret_cast<const VF*>(cs.m0 + o);
+            om1 = *reinterpret_cast<const VF*>(cs.m1 + o);
+            ow = *wp;
+        }
+        running();
+        if (row != i) act = 0;
+        if (!act) return;  // lanes whose frames have all stopped change nothing
         const float pm = a.paper ? -1.0f : 1.0f;
         VF n0, n1;
         uint32_t loc[V], sg[V], zx[V];
@@ -1000,9 +1028,22 @@ __global__ void __launch_bounds__(128, 5)
         *reinterpret_cast<VF*>(cs.m0 + o) = n0;
         *reinterpret_cast<VF*>(cs.m1 + o) = n1;
         *wp = nw;
+    };
+    const int warp = threadIdx.x >> 5;
+    if constexpr (ROWS) {
+        running();
+#pragma unroll 1
+        for (int n = 0; n < kCheckRegRows; n++) {
+            const int i = ((int)blockIdx.x * kCheckRegRows + n) * 4 + warp;
+            if (i >= a.M || !act) break;
+            one_row(i, i);
+        }
+    } else {
+        const int row = blockIdx.x * 4 + warp;
+        one_row(row, min(row, a.M - 1));
     }
     __syncwarp();
-    if (SYN) flags.end(z & act);
+    if (SYN) CtaFlags<V>::end(fail, a.unsat, blockIdx.y * 32 * V, z & act);
 }
 
 // The final syndrome of few frames, and of any number on rows of 17 to 32 edges.
@@ -1918,20 +1959,30 @@ bool staged(const DevGraph& g, const DecodeArgs& a, const StreamWork& w,
     return launch_staged<MODE, V, FIRST, W, D, false, CMP>(g, a, w, s, eta, un, test_prev, wt, st);
 }
 
-// One check pass on compressed messages (FP32): the staged kernel on the padded row layout,
-// k_check_cmp on rows of 17 to 27 edges (which need no staging); false when the staged kernel cannot run (the caller then keeps per-edge messages; this
+// One check pass on compressed messages (FP32): k_check_reg on full lanes (V = 4) where no
+// staging shape was asked for, and on rows of 17 to 27 edges always; else the staged kernel.
+// false when the staged kernel cannot run (the caller then keeps per-edge messages; this
 // can only happen on the first iteration, before any state exists).
 template <int V, bool FIRST, bool W>
 bool check_pass_cmp(const DevGraph& g, const DecodeArgs& a, const StreamWork& w, const float* s,
                     float* state, uint32_t* un, int test_prev, const IterWeights& wt_prev, cudaStream_t st) {
     if constexpr (V == 4) {
         if (w.auto_staging || g.ell_D == 0) {
-            auto kern = g.ell_D == 8    ? (test_prev ? k_check_reg<FIRST, true, W, V, 8> : k_check_reg<FIRST, false, W, V, 8>)
-                        : g.ell_D == 16 ? (test_prev ? k_check_reg<FIRST, true, W, V, 16> : k_check_reg<FIRST, false, W, V, 16>)
-                                        : (test_prev ? k_check_reg<FIRST, true, W, V, 0> : k_check_reg<FIRST, false, W, V, 0>);
+            const int fb = (a.frames + 32 * V - 1) / (32 * V);  // (the blocks behind them hold no frame)
+            const bool rows = test_prev && g.ell_D > 0 && (int64_t)a.M * fb >= 128ll * w.num_sms;
+            auto pick = [&](auto d) {
+                constexpr int D = decltype(d)::value;
+                if constexpr (D > 0)
+                    if (rows) return k_check_reg<FIRST, true, W, V, D, true>;
+                return test_prev ? k_check_reg<FIRST, true, W, V, D> : k_check_reg<FIRST, false, W, V, D>;
+            };
+            auto kern = g.ell_D == 8    ? pick(std::integral_constant<int, 8>())
+                        : g.ell_D == 16 ? pick(std::integral_constant<int, 16>())
+                                        : pick(std::integral_constant<int, 0>());
+            const int per_cta = rows ? 4 * kCheckRegRows : 4;
             const CheckRegArgs ra{g.ell_D ? g.ell_col : g.col_idx, g.ell_deg, g.ell_cls, g.row_ptr, a.M, w.Fp,
-                                  a.paper_slicer, w.state, un};
-            kern<<<dim3((a.M + 3) / 4, w.Fp / (32 * V)), 128, 0, st>>>(ra, s, cstate_at(state, a.M, w.Fp), wt_prev);
+                                  a.paper_slicer, w.state, un, w.comp, w.n_done, a.frames};
+            kern<<<dim3((a.M + per_cta - 1) / per_cta, fb), 128, 0, st>>>(ra, s, cstate_at(state, a.M, w.Fp), wt_prev);
             return true;
         }
     }
