@@ -19,9 +19,10 @@
 //     (eq. 1-2);
 //   phase B, one thread per column lane: s = r + the column's eta in ascending row order
 //     (eq. lambda_j).
-// A frame whose syndrome is zero is written out at once (iterations = k); it keeps being
-// computed with its tile (no per-frame branches in the inner loops) but is never written
-// again. The tile ends when all its frames are out or after max_iter iterations.
+// A frame whose syndrome is zero is written out at once (iterations = k). In early-stop decodes
+// (decode_refill) its slot then goes to the next frame of the batch, where that pays; else it
+// keeps being computed with its tile (no per-frame branches in the inner loops) but is never
+// written again, and the tile ends when all its frames are out or after max_iter iterations.
 #pragma once
 
 #include <algorithm>
@@ -1065,6 +1066,9 @@ struct Slots {
     int32_t next;      // first of the frames taken from the counter for the slots that ended
     uint32_t due;      // slots to be tested after the next column pass, if they go on
     uint32_t last;     // those of them that reach the iteration limit there
+    // RULE: iterations of the frame that ended last; mean difference of two such counts, in
+    // 1/1024, over about 64 frames
+    int32_t k_prev, spread;
 };
 
 // Frame fr into slot f of the tile, between the row and the column pass: its channel values in
@@ -1097,6 +1101,15 @@ __device__ __forceinline__ void refill_slot(const ResArgs& a, const Idx& ix, VT*
     }
 }
 
+// RULE: mean difference of the iterations of two frames, in 1/1024, from which on a CTA refills
+// its slots. Tiles of 4 frames against whole tiles: at 0.2 to 0.7 iterations 4 to 15 % slower,
+// at 0.9 one per cent slower, at 1.1 five, at 1.3 four and at 2.2 15 % faster (fixed point
+// QC N=2304, both modes N=576 and N=2048, 3 to 7 dB). The rule is for batches of at least
+// kSpreadTiles tiles a CTA: it takes that many to learn, and costs 1 to 3 % where it refills
+// anyway (fixed point QC N=2304, 8191 frames, 978 against 998 us).
+constexpr int kSpread = 832;
+constexpr int kSpreadTiles = 16;
+
 // Early-stop decode of the CTA's share of the frames (plain Min-Sum, standard slicer): a tile
 // of FT frames, in which a frame that stops gives its slot to the next frame of the batch
 // while the others go on, so that a tile does not run idle slots until its slowest frame
@@ -1108,19 +1121,29 @@ __device__ __forceinline__ void refill_slot(const ResArgs& a, const Idx& ix, VT*
 // tiles spent 20 iterations on the slowest of four frames where the mean is 7. Measured
 // against them: QC N=2304, 8191 frames (int8, Eb/N0 3.5-4.5 dB, at most 20 iterations) 1337
 // -> 962 us; 16384 frames FP32 2628 -> 2135 us; N=576, 65536 frames FP32 at 2.5 dB 1948 ->
-// 1420 us. Where all frames of a tile stop within an iteration or two of each other it gains
-// nothing (QC at 4.5 dB, 16384 frames: FP32 1300 -> 1273, fixed point 1025 -> 1053 us).
+// 1217 us (with the reordered columns). Where all frames of a tile stop within an iteration of
+// each other refilling loses on tiles of 4 frames; large batches look (RULE, kSpread): N=576,
+// 65536 frames at 7 dB whole tiles 374, always refilled 391, with the rule 338 us (FP32), fixed
+// point 420, 463, 413 us; fixed point QC, 16384 frames at 4.5 dB 1102, 1124, 1086 us.
 // Measured and not kept: frames taken from the counter ahead of their use, prefetched channel
 // values, and waiting for a quiet iteration before the first refill of a tile (all slower).
-template <int MODE, int FT, typename VT, bool DEC>
+template <int MODE, int FT, typename VT, bool DEC, bool RULE>
 __device__ __forceinline__ void decode_refill(const ResArgs& a, const Idx& ix, VT* eta, VT* s, VT* r,
                                               uint32_t* unsat_w, Slots* sl, int n_rtasks, uint8_t* dec) {
     using T = typename RT<MODE>::T;
     using A = typename RT<MODE>::A;
     constexpr bool kPacked = MODE == kModeFixed && FT % 2 == 0;
     constexpr uint32_t kAll = (1u << FT) - 1u;
+    // (without the rule every empty slot has just ended, or no frames are left)
+    constexpr bool kRefillAll = RULE || FT <= 2;
     const int N = a.N;
-    if (threadIdx.x == 0) sl->next = (int)blockIdx.x * FT;
+    if (threadIdx.x == 0) {
+        sl->next = (int)blockIdx.x * FT;
+        if (RULE) {
+            sl->k_prev = 0;
+            sl->spread = 9 * kSpread / 8;
+        }
+    }
     for (;;) {  // fresh tiles
         __syncthreads();
         const int fbase = sl->next;
@@ -1174,10 +1197,16 @@ __device__ __forceinline__ void decode_refill(const ResArgs& a, const Idx& ix, V
                     active &= ~fin;
                     // the counter's answer comes while the frames are written out
                     if (threadIdx.x == 0) {
-                        if (a.tile_counter)
-                            sl->next = (int)gridDim.x * FT + atomicAdd(a.tile_counter, active ? __popc(fin) : FT);
+                        if (a.tile_counter && (!RULE || !active || sl->spread >= kSpread))
+                            sl->next = (int)gridDim.x * FT + atomicAdd(a.tile_counter, kRefillAll ? __popc(kAll & ~active) : active ? __popc(fin) : FT);
                         else
-                            sl->next = a.frames;  // every frame was in a first tile
+                            sl->next = a.frames;  // no counter: every frame was in a first tile
+                        if constexpr (RULE) {  // the others of `fin` are taken to have ended with the first
+                            const int k = sl->k[__ffs(fin) - 1];
+                            const int sp = sl->spread + ((min(abs(k - sl->k_prev), 64) * 1024 - sl->spread) >> 6);
+                            sl->spread = sp - ((__popc(fin) - 1) * sp >> 6);
+                            sl->k_prev = k;
+                        }
                     }
                     for (int j = threadIdx.x; j < N; j += blockDim.x) {
                         const auto v = s[ix.col_pos[j]];
@@ -1196,10 +1225,11 @@ __device__ __forceinline__ void decode_refill(const ResArgs& a, const Idx& ix, V
                     }
                     if (!active) break;  // (the fresh tile begins with a barrier)
                     __syncthreads();  // (also orders the reads of s before the column pass)
-                    // the ended slots take the frames next, next + 1, ... in order
+                    // the empty slots take the frames next, next + 1, ... in order
                     const int next = sl->next;
-                    for (uint32_t m = fin; m; m &= m - 1) {
-                        const int f = __ffs(m) - 1, fr = next + __popc(fin & ((1u << f) - 1u));
+                    const uint32_t empty = kRefillAll ? kAll & ~active : fin;
+                    for (uint32_t m = empty; m; m &= m - 1) {
+                        const int f = __ffs(m) - 1, fr = next + __popc(empty & ((1u << f) - 1u));
                         if (fr >= a.frames) break;
                         fresh |= 1u << f;
                         refill_slot<MODE, FT>(a, ix, eta, r, f, fr);
@@ -1237,7 +1267,8 @@ __device__ __forceinline__ void decode_refill(const ResArgs& a, const Idx& ix, V
 // stop): no work counter, and the index arrays arrive in one copy. The kernels of full batches
 // keep the loop over the counter and the copies array by array, which the compiler turned into
 // a faster iteration (QC N=2304, 65536 frames: 8350 us against 8420).
-template <int MODE, int FT, bool IDX_SMEM, bool PAPER, bool W, bool ES, bool ONE = false>
+// RULE: early-stop decodes of many tiles a CTA (kSpreadTiles).
+template <int MODE, int FT, bool IDX_SMEM, bool PAPER, bool W, bool ES, bool ONE = false, bool RULE = false>
 __global__ void __launch_bounds__(kMaxThreads, 1) k_resident(const ResArgs a) {
     using T = typename RT<MODE>::T;
     using VT = VecR<T, FT>;
@@ -1306,7 +1337,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_resident(const ResArgs a) {
     if constexpr (ES && !W) {
         __shared__ Slots slots;
         __syncthreads();  // the index arrays are in shared memory
-        decode_refill<MODE, FT, VT, kDec>(a, ix, eta, s, r, unsat_w, &slots, n_rtasks, dec);
+        decode_refill<MODE, FT, VT, kDec, RULE>(a, ix, eta, s, r, unsat_w, &slots, n_rtasks, dec);
     } else if constexpr (ONE) {
         const int fbase = blockIdx.x * FT;
         if (threadIdx.x < 2) unsat_w[threadIdx.x] = 0;
@@ -1348,6 +1379,12 @@ int launch(const ResArgs& ra, const ResidentPlan& p, int num_sms, cudaStream_t s
         return LDPC_ERR_CUDA;
     if (per_sm < 1) return LDPC_ERR_UNSUPPORTED;
     const int grid = std::max(1, std::min(ra.n_tiles, num_sms * per_sm));
+    if constexpr (ES && !W && FT == 4)
+        if (ra.n_tiles >= (int64_t)kSpreadTiles * grid) {
+            kern = k_resident<MODE, FT, IDX, PAPER, W, ES, false, true>;
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess)
+                return LDPC_ERR_CUDA;
+        }
     ResArgs r = ra;
     // early stop: the first tile of CTA b is tile b, and without more there is no counter
     if (one || (ES && !W && ra.n_tiles <= grid)) r.tile_counter = nullptr;
