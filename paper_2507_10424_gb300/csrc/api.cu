@@ -61,8 +61,10 @@ struct Arena {
     template <typename T>
     void add(T** dst, const std::vector<T>& v) {
         const size_t o = (bytes.size() + 255) & ~(size_t)255;
-        bytes.resize(o + std::max<size_t>(1, v.size()) * sizeof(T));  // never a null array
-        if (!v.empty()) std::memcpy(bytes.data() + o, v.data(), v.size() * sizeof(T));
+        bytes.resize(o);
+        const uint8_t* src = reinterpret_cast<const uint8_t*>(v.data());
+        if (v.empty()) bytes.resize(o + sizeof(T));  // never a null array
+        else bytes.insert(bytes.end(), src, src + v.size() * sizeof(T));
         at.emplace_back((void**)dst, o);
     }
     int upload(void** base) {
@@ -139,7 +141,7 @@ struct ldpc {
 };
 
 static void free_graph(DevGraph& g) {
-    for (void* p : {g.arena, (void*)g.packed})
+    for (void* p : {g.arena, g.packed_mem})
         if (p) cudaFree(p);
     g = DevGraph();
 }
@@ -410,6 +412,7 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
     if ((rc = noalloc_setup(h->device)) != LDPC_OK) return bail(fail(rc));
     // CSR / CSC
     Arena arena;
+    arena.bytes.reserve((size_t)hg.E * 24 + (size_t)hg.M * 90 + (size_t)hg.N * 32 + (1 << 16));  // about all
     arena.add(&h->dg.row_ptr, hg.row_ptr);
     arena.add(&h->dg.col_idx, hg.col_idx);
     arena.add(&h->dg.col_ptr, hg.col_ptr);
@@ -427,26 +430,18 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
             h->dg.ell_D = eg.D;
             h->dg.eta_slots = (int64_t)hg.M * eg.D;
         } else if (hg.max_dc <= 255) {
-            std::vector<int32_t> row_of((size_t)hg.E);
-            for (int32_t i = 0; i < hg.M; i++)
-                for (int32_t e2 = hg.row_ptr[i]; e2 < hg.row_ptr[i + 1]; e2++) row_of[e2] = i;
             // (12 bytes a row of state in the place of 4 an edge; slots in 31 bits)
             if (hg.max_dc <= kCmsgMaxRow && hg.E >= 3 * (int64_t)hg.M && hg.M < (1 << 26)) {
                 std::vector<int32_t> row_slot((size_t)hg.E);
                 for (int64_t q = 0; q < hg.E; q++) {
-                    const int32_t e2 = hg.col_edge[q], i = row_of[e2];
-                    row_slot[q] = i << kRowSlotShift | (e2 - hg.row_ptr[i]);
+                    const int32_t i = hg.col_row[q];
+                    row_slot[q] = i << kRowSlotShift | (hg.col_edge[q] - hg.row_ptr[i]);
                 }
                 arena.add(&h->dg.row_slot, row_slot);
             } else {
-                std::vector<int32_t> col_row((size_t)hg.E);
                 std::vector<uint8_t> col_k((size_t)hg.E);
-                for (int64_t q = 0; q < hg.E; q++) {
-                    const int32_t e2 = hg.col_edge[q];
-                    col_row[q] = row_of[e2];
-                    col_k[q] = (uint8_t)(e2 - hg.row_ptr[row_of[e2]]);
-                }
-                arena.add(&h->dg.col_row, col_row);
+                for (int64_t q = 0; q < hg.E; q++) col_k[q] = (uint8_t)(hg.col_edge[q] - hg.row_ptr[hg.col_row[q]]);
+                arena.add(&h->dg.col_row, hg.col_row);
                 arena.add(&h->dg.col_k, col_k);
             }
         }
@@ -463,11 +458,17 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
         for (int32_t i = 0; i < hg.M; i++)
             for (int32_t e2 = hg.row_ptr[i]; e2 < hg.row_ptr[i + 1]; e2++)
                 packed[(size_t)i * W + hg.col_idx[e2] / 32] |= 1u << (hg.col_idx[e2] % 32);
-        if ((rc = upload(&h->dg.packed, packed.data(), packed.size()))) return bail(rc);
+        if (packed.size() < (1u << 16)) {
+            arena.add(&h->dg.packed, packed);
+        } else {  // (the copy on the host would cost more than the allocation: N=8176 722 -> 803 us a handle)
+            rc = upload(&h->dg.packed, packed.data(), packed.size());
+            h->dg.packed_mem = h->dg.packed;
+            if (rc) return bail(rc);
+        }
     }
     // sliced layouts for the resident kernel (codes small enough to be resident)
     SlicedGraph sg;
-    if (build_sliced(hg, sg)) {
+    if (build_sliced(hg, sg, mode == kModeFP32 ? 4 : 2, h->smem_optin)) {
         DevGraph& d = h->dg;
         d.n_rslices = sg.n_rslices;
         d.n_cslices = sg.n_cslices;
@@ -504,6 +505,7 @@ static ldpc_t* create_from_graph(HostGraph& hg, int32_t mode, int32_t flags) {
     if (e != cudaSuccess) return bail(alloc_fail(e));
     e = cudaMemset(h->counters, 0, 8 * sizeof(int32_t));
     if (e != cudaSuccess) return bail(cuda_fail(e));
+    hg.col_row = std::vector<int32_t>();  // (not needed any more)
     h->hg = std::move(hg);
     g_last_error = LDPC_OK;
     return h;

@@ -23,9 +23,14 @@ static int finish_graph(HostGraph& g) {
     for (int64_t e = 0; e < g.E; e++) g.col_ptr[g.col_idx[e] + 1]++;
     for (int32_t j = 0; j < N; j++) g.col_ptr[j + 1] += g.col_ptr[j];
     g.col_edge.resize(g.E);
+    g.col_row.resize(g.E);
     std::vector<int32_t> fill(g.col_ptr.begin(), g.col_ptr.end() - 1);
     for (int32_t i = 0; i < M; i++)  // rows in ascending order -> ascending rows per column
-        for (int32_t e = g.row_ptr[i]; e < g.row_ptr[i + 1]; e++) g.col_edge[fill[g.col_idx[e]]++] = e;
+        for (int32_t e = g.row_ptr[i]; e < g.row_ptr[i + 1]; e++) {
+            const int32_t q = fill[g.col_idx[e]]++;
+            g.col_edge[q] = e;
+            g.col_row[q] = i;
+        }
     g.max_dv = 0;
     for (int32_t j = 0; j < N; j++) g.max_dv = std::max(g.max_dv, g.col_ptr[j + 1] - g.col_ptr[j]);
     assign_classes(g);
@@ -122,11 +127,17 @@ int graph_from_csr(int32_t M, int32_t N, const int64_t* row_ptr, const int32_t* 
 // Degree-sorted order of n items (descending degree, stable).
 static std::vector<int32_t> sorted_by_degree(const std::vector<int32_t>& ptr) {
     const int32_t n = (int32_t)ptr.size() - 1;
+    int32_t most = 0;
+    for (int32_t x = 0; x < n; x++) most = std::max(most, ptr[x + 1] - ptr[x]);
+    std::vector<int32_t> at(most + 2, 0);  // at[d]: place of the next item of degree d
+    for (int32_t x = 0; x < n; x++) at[ptr[x + 1] - ptr[x]]++;
+    for (int32_t d = most, p = 0; d >= 0; d--) {
+        const int32_t c = at[d];
+        at[d] = p;
+        p += c;
+    }
     std::vector<int32_t> order(n);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-        return (ptr[a + 1] - ptr[a]) > (ptr[b + 1] - ptr[b]);
-    });
+    for (int32_t x = 0; x < n; x++) order[at[ptr[x + 1] - ptr[x]]++] = x;
     return order;
 }
 
@@ -156,25 +167,26 @@ static int32_t make_slices(const std::vector<int32_t>& ptr, const std::vector<in
 // lanes of the group). Random codes went from 2.6 wavefronts a group of 8 lanes to 1.6 (a
 // window of 64), of 16 from 3.1 to 2.0, of 32 from 3.5 to 2.6; quasi-cyclic codes start below
 // 1.5 (2112: 1.24), which the search makes worse (1.40, and a decode 3 % slower): they keep
-// theirs. The window shrinks with N so that the search stays under half a
-// millisecond. A decode of 4096 frames, (3,6) code, before and after: N=576, 10 iterations 89
+// theirs. The window shrinks with N so that the search stays under half a millisecond (creating
+// a handle: N=2048 0.41 ms, N=8192 1.29 ms, N=16200 in fixed point 2.35 ms, and 1.65 ms in FP32,
+// where that code streams and nothing is searched). A decode of 4096 frames, (3,6) code, before and after: N=576, 10 iterations 89
 // -> 76 us, N=1500 254 -> 216 us; N=576 with early stop, 65536 frames, 1420 -> 1214 us.
 static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of_row, int group,
                          std::vector<int32_t>& order) {
     constexpr int kMaxDeg = 16;  // edges looked at
     const int32_t N = (int32_t)order.size();
     const int32_t window = std::min(64, std::max(8, 65536 / std::max(1, N)));
-    // the lane, modulo the group, of each column's edges
+    // the lane, modulo the group (a power of two), of each column's edges
     std::vector<uint8_t> lane((size_t)g.E);
-    std::vector<int32_t> row_of((size_t)g.E);
-    for (int32_t i = 0; i < g.M; i++)
-        for (int32_t e = g.row_ptr[i]; e < g.row_ptr[i + 1]; e++) row_of[e] = i;
-    for (int64_t q = 0; q < g.E; q++) lane[q] = (uint8_t)(lane_of_row[row_of[g.col_edge[q]]] % group);
+    for (int64_t q = 0; q < g.E; q++) lane[q] = (uint8_t)(lane_of_row[g.col_row[q]] & (group - 1));
     uint8_t cnt[kMaxDeg][32], most[kMaxDeg];
-    // wavefronts of an order over the wavefronts of one without conflicts
+    uint32_t full[kMaxDeg];  // the lanes whose next edge adds a wavefront
+    // wavefronts of an order over the wavefronts of one without conflicts, on about 1024 of its
+    // columns
+    const int32_t step = group * std::max(1, N / 1024);
     auto cost = [&](const std::vector<int32_t>& ord) {
         int64_t sum = 0, least = 0;
-        for (int32_t p = 0; p < N; p += group) {
+        for (int32_t p = 0; p < N; p += step) {
             std::memset(cnt, 0, sizeof(cnt));
             std::memset(most, 0, sizeof(most));
             for (int32_t x = p; x < std::min(N, p + group); x++) {
@@ -190,37 +202,53 @@ static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of
     };
     const double before = cost(order);
     if (before <= 1.6) return;  // quasi-cyclic codes: the search would not better their order
-    std::vector<int32_t> out;
-    out.reserve(N);
-    std::vector<int32_t> win;  // the columns to choose from, in order
-    int32_t next = 0;
-    while ((int32_t)out.size() < N) {
-        if (out.size() % group == 0) {
+    std::vector<int32_t> out(N);
+    // the columns to choose from, in order: win[0 .. n), their edges in at[], their degrees in
+    // deg[]
+    int32_t win[64], at[64], deg[64], n = 0, next = 0;
+    for (int32_t p = 0; p < N; p++) {
+        if (p % group == 0) {
             std::memset(cnt, 0, sizeof(cnt));
             std::memset(most, 1, sizeof(most));
+            std::memset(full, 0, sizeof(full));
         }
-        while (next < N && (int32_t)win.size() < window) win.push_back(order[next++]);
-        const int32_t d = g.col_ptr[win[0] + 1] - g.col_ptr[win[0]], dd = std::min(d, kMaxDeg);
+        for (; next < N && n < window; next++, n++) {
+            win[n] = order[next];
+            at[n] = g.col_ptr[win[n]];
+            deg[n] = g.col_ptr[win[n] + 1] - at[n];
+        }
+        const int32_t d = deg[0], dd = std::min(d, kMaxDeg);
         int best = 0, least = dd + 1;
-        for (int c = 0; c < (int)win.size() && least > 0; c++) {
-            const int32_t q = g.col_ptr[win[c]];
-            if (g.col_ptr[win[c] + 1] - q != d) break;  // the degrees stay sorted
+        for (int c = 0; c < n && deg[c] == d; c++) {  // (the degrees stay sorted)
+            const uint8_t* l = lane.data() + at[c];
             int x = 0;
-            for (int t = 0; t < dd; t++) x += cnt[t][lane[q + t]] >= most[t];
+            for (int t = 0; t < dd; t++) x += (int)(full[t] >> l[t] & 1u);
             if (x < least) {
                 least = x;
                 best = c;
+                if (x == 0) break;
             }
         }
-        const int32_t j = win[best], q = g.col_ptr[j];
-        win.erase(win.begin() + best);
-        out.push_back(j);
-        for (int t = 0; t < dd; t++) most[t] = std::max(most[t], ++cnt[t][lane[q + t]]);
+        out[p] = win[best];
+        const uint8_t* l = lane.data() + at[best];
+        for (int t = 0; t < dd; t++) {
+            const uint8_t x = ++cnt[t][l[t]];
+            if (x > most[t]) {  // it alone has that many
+                most[t] = x;
+                full[t] = 1u << l[t];
+            } else if (x == most[t]) {
+                full[t] |= 1u << l[t];
+            }
+        }
+        n--;
+        std::memmove(win + best, win + best + 1, (n - best) * sizeof(win[0]));
+        std::memmove(at + best, at + best + 1, (n - best) * sizeof(at[0]));
+        std::memmove(deg + best, deg + best + 1, (n - best) * sizeof(deg[0]));
     }
     if (cost(out) < before) order.swap(out);
 }
 
-bool build_sliced(const HostGraph& g, SlicedGraph& sg) {
+bool build_sliced(const HostGraph& g, SlicedGraph& sg, int value_bytes, int64_t smem) {
     if (g.N > 65535 || g.max_dc > 255 || g.max_dv > 255) return false;
     const std::vector<int32_t> rorder = sorted_by_degree(g.row_ptr);
     std::vector<int32_t> corder = sorted_by_degree(g.col_ptr);
@@ -229,7 +257,8 @@ bool build_sliced(const HostGraph& g, SlicedGraph& sg) {
     sg.E_pad = make_slices(g.row_ptr, rorder, sg.r_base, sg.r_deg);
     sg.Ec_pad = make_slices(g.col_ptr, corder, sg.c_base, sg.c_deg);
     if (sg.E_pad >= 65536 || sg.Ec_pad >= 65536) return false;
-    {
+    // (no search where not even one frame of the mode fits shared memory: such a code streams)
+    if (value_bytes * ((int64_t)sg.E_pad + 64 * sg.n_cslices) <= smem) {
         std::vector<uint8_t> lane_of_row(g.M);
         for (int32_t p = 0; p < g.M; p++) lane_of_row[rorder[p]] = (uint8_t)(p % 32);
         // the widest FP32 tile that fits shared memory: 4, 2 or 1 frames of 4-byte values

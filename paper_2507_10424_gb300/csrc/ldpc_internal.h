@@ -25,6 +25,7 @@ struct HostGraph {
     std::vector<int32_t> col_idx;   // E
     std::vector<int32_t> col_ptr;   // N+1
     std::vector<int32_t> col_edge;  // E: CSR edge ids of column j, ascending row
+    std::vector<int32_t> col_row;   // E: their rows
     int32_t max_dc = 0, max_dv = 0;
     // edge classes for learned weights: class of bit j = index of its column weight among
     // the sorted distinct column weights
@@ -61,7 +62,8 @@ struct SlicedGraph {
     std::vector<uint8_t> r_slot_cls;    // E_pad: class of the edge's bit (0 for padding)
 };
 // Returns false when the code cannot use 16-bit slot ids or 8-bit degrees.
-bool build_sliced(const HostGraph& g, SlicedGraph& sg);
+// value_bytes: of a message in the handle's mode; smem: shared memory of a CTA.
+bool build_sliced(const HostGraph& g, SlicedGraph& sg, int value_bytes, int64_t smem);
 
 // The index arrays of the resident kernel one after the other, each on a 16-byte boundary: the
 // order and offsets they have in shared memory and, as one array, in global memory.
@@ -173,7 +175,8 @@ struct DevGraph {
     uint8_t* r_slot_cls = nullptr;
     int32_t n_rslices = 0, n_cslices = 0, E_pad = 0, Ec_pad = 0;
     uint8_t* idx_blob = nullptr;  // the arrays above but r_slot_cls, laid out by idx_layout
-    void* arena = nullptr;        // the allocation that holds every array but `packed`
+    void* arena = nullptr;        // the allocation that holds every array but a large `packed`
+    void* packed_mem = nullptr;   // the allocation of a large `packed`
     int32_t sliced = 0;  // the sliced layout exists
     int32_t max_dc = 0;  // longest row (set for every code)
     // padded row layout (streaming kernels); ell_D = 0 when absent
