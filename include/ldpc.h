@@ -368,7 +368,7 @@ int ldpc_autotune_data(ldpc_t *h, const float *llr, int32_t frames, int32_t max_
  * ldpc_decode_i8, ldpc_decode_ex and ldpc_decode_host first run checking kernels on the
  * handle's stream over every index array the decode kernels read through (CSR/CSC
  * offsets and indices, the sliced and padded layouts' slot ids, column positions, slice
- * degrees and weight classes: each within the array it indexes) and over the caller's FP32
+ * degrees, the rows of the columns' edges and weight classes: each within the array it indexes) and over the caller's FP32
  * LLRs (no NaN: the decoder does not define it), then synchronise the stream and read the
  * result. A violation returns LDPC_ERR_DEVICE_CHECK and no decode kernel is launched; the
  * outputs are left untouched. Slow (a stream synchronisation per call): for testing and
@@ -383,7 +383,7 @@ int ldpc_autotune_data(ldpc_t *h, const float *llr, int32_t frames, int32_t max_
  * offsets, 8 row slice degree, 9 column slice degree, 10 column position of a row slot,
  * 11 row slot of a column entry, 12 column position of a bit, 13 class of a row slot,
  * 14 column of a padded row slot, 15 padded row degree, 16 padded slot of an edge, 17 class
- * of a padded row slot). what and where are host pointers.
+ * of a padded row slot, 18 row of a CSC entry and its place in it). what and where are host pointers.
  */
 int ldpc_set_debug(ldpc_t *h, int32_t on);
 int ldpc_debug_report(ldpc_t *h, int32_t *what, int64_t *where);

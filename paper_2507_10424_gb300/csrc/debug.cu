@@ -1,7 +1,8 @@
 // Device-side debug checks (ldpc_set_debug): before a decode, one pass over every index
 // array the kernels read through and over the caller's LLRs, recording the first
 // violation. The decode kernels address shared and global memory through these arrays
-// (slot ids, column positions, CSR/CSC indices, the padded row layout, weight classes), so
+// (slot ids, column positions, CSR/CSC indices, the padded row layout, the row and the place in
+// it of a column's edges, weight classes), so
 // an entry out of range there, from a stray write into the handle's memory, would become
 // an out-of-bounds access; the host refuses the decode instead. FP32 LLRs are checked for
 // NaN, which the decoder does not define (its comparisons would be unordered).
@@ -58,6 +59,20 @@ __global__ void k_slice_deg(const int32_t* __restrict__ base, const uint8_t* __r
     }
 }
 
+// Row and position in the row of each edge in column order: packed (row << kRowSlotShift |
+// position) or two arrays. The row exists and the position is below its degree.
+__global__ void k_edge_row(const int32_t* __restrict__ row_slot, const int32_t* __restrict__ col_row,
+                           const uint8_t* __restrict__ col_k, const int32_t* __restrict__ row_ptr, int32_t M,
+                           int64_t E, int id, unsigned long long* rep) {
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < E;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t i = row_slot ? row_slot[q] >> kRowSlotShift : col_row[q];
+        const int32_t k = row_slot ? row_slot[q] & ((1 << kRowSlotShift) - 1) : col_k[q];
+        if (i < 0 || i >= M || k >= row_ptr[i + 1] - row_ptr[i])
+            report(rep, ((unsigned long long)id << 40) | (unsigned long long)q);
+    }
+}
+
 int grid_for(int64_t n) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((n + kCheckThreads - 1) / kCheckThreads, 4096));
 }
@@ -105,6 +120,9 @@ int debug_check_launch(const DevGraph& g, int32_t M, int32_t N, int64_t E, const
         below(g.ell_cslot, E, slots, DebugArray::kEllCslot);
         if (g.n_classes > 0) below(g.ell_cls, slots, g.n_classes, DebugArray::kEllCls);
     }
+    if (g.row_slot || (g.col_row && g.col_k))
+        k_edge_row<<<grid_for(E), kCheckThreads, 0, st>>>(g.row_slot, g.col_row, g.col_k, g.row_ptr, M, E,
+                                                          (int)DebugArray::kEdgeRow, gr);
     return cudaGetLastError() == cudaSuccess ? LDPC_OK : LDPC_ERR_CUDA;
 }
 

@@ -169,8 +169,9 @@ static int32_t make_slices(const std::vector<int32_t>& ptr, const std::vector<in
 // 1.5 (2112: 1.24), which the search makes worse (1.40, and a decode 3 % slower): they keep
 // theirs. The window shrinks with N so that the search stays under half a millisecond (creating
 // a handle: N=2048 0.41 ms, N=8192 1.29 ms, N=16200 in fixed point 2.35 ms, and 1.65 ms in FP32,
-// where that code streams and nothing is searched). A decode of 4096 frames, (3,6) code, before and after: N=576, 10 iterations 89
-// -> 76 us, N=1500 254 -> 216 us; N=576 with early stop, 65536 frames, 1420 -> 1214 us.
+// where that code streams and nothing is searched). A decode of 4096 frames, (3,6) code, before
+// and after: N=576, 10 iterations 89 -> 76 us, N=1500 254 -> 216 us; N=576 with early stop,
+// 65536 frames, 1420 -> 1214 us.
 static void spread_banks(const HostGraph& g, const std::vector<uint8_t>& lane_of_row, int group,
                          std::vector<int32_t>& order) {
     constexpr int kMaxDeg = 16;  // edges looked at

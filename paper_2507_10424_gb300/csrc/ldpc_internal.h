@@ -199,7 +199,7 @@ struct DevGraph {
 // Index arrays the debug checks cover (ids in the report of ldpc_debug_report).
 enum class DebugArray : int {
     kRowPtr = 1, kColPtr, kColIdx, kColEdge, kColClass, kRowBase, kColBase, kRowDeg, kColDeg,
-    kRowSlotPos, kColSlot, kColPos, kRowSlotCls, kEllCol, kEllDeg, kEllCslot, kEllCls
+    kRowSlotPos, kColSlot, kColPos, kRowSlotCls, kEllCol, kEllDeg, kEllCslot, kEllCls, kEdgeRow
 };
 // Enqueue the debug checks of a decode on st (debug.cu): rep[0] receives the smallest flat
 // index of a NaN FP32 LLR, rep[1] the smallest (array id << 40 | entry) of an index out of
