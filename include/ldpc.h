@@ -350,8 +350,8 @@ int ldpc_autotune(ldpc_t *h, int32_t frames, int32_t max_iter, float *best_ms);
 /*
  * ldpc_autotune_data: as ldpc_autotune, but each shape decodes the caller's frames with the
  * caller's early-stop settings, so the choice fits workloads whose frames stop at
- * different iterations (a tile of several frames runs until its last frame stops, which
- * favours narrower tiles than timing without early stop does).
+ * different iterations (an ended frame's slot goes to the next frame, which costs wide tiles more
+ * than narrow ones; with learned weights a tile runs until its last frame stops).
  *   llr         device pointer, FP32 [frames][N], frame-major (as ldpc_decode_ex with
  *               LDPC_LLR_F32); only the first min(frames, 65536) (resident) or
  *               min(frames, 2048) (streaming) frames are decoded; read only.
@@ -388,7 +388,10 @@ int ldpc_autotune_data(ldpc_t *h, const float *llr, int32_t frames, int32_t max_
 int ldpc_set_debug(ldpc_t *h, int32_t on);
 int ldpc_debug_report(ldpc_t *h, int32_t *what, int64_t *where);
 
-/* ldpc_get_tuning: the resident launch shape in force for the current mode. */
+/* ldpc_get_tuning: the resident launch shape of the current mode, asked for (ldpc_set_tuning,
+ * ldpc_autotune) or automatic. An automatic shape is that of large batches: a batch with few
+ * frames per SM runs tiles of one or two frames, and a code of which only one frame fits with its
+ * index arrays may run two frames with the arrays in global memory. */
 int ldpc_get_tuning(const ldpc_t *h, int32_t *frames_per_tile, int32_t *threads,
                     int32_t *index_placement);
 
@@ -402,9 +405,12 @@ int ldpc_get_tuning(const ldpc_t *h, int32_t *frames_per_tile, int32_t *threads,
 int ldpc_set_stream_group(ldpc_t *h, int32_t frames_per_group);
 
 /*
- * ldpc_set_stream_staging: shape of the streaming variant's check pass for codes whose
+ * ldpc_set_stream_staging: shape of the streaming variant's staged check pass for codes whose
  * rows have at most 16 edges. Row i then owns 8 or 16 message slots (a padded row
- * layout). Each warp of a persistent kernel keeps `stages` shared-memory stages in
+ * layout). With 0, 0, 0 (the default) the library chooses by mode and batch: up to 64 frames a
+ * register kernel on 1 or 2 frames per lane, and FP32 codes with compressed messages
+ * (ldpc_set_stream_messages) a register kernel on 4; else the staged pass with the automatic
+ * shape. Any other value asks for the staged pass, whatever the batch. Each warp of a persistent kernel keeps `stages` shared-memory stages in
  * flight. Into each stage, the TMA engine's bulk asynchronous copies (cp.async.bulk)
  * bring one row's gathered posteriors s_j and old messages for 32 x frames_per_lane
  * frames, completing on an mbarrier, while the warp computes an earlier row (Section
@@ -425,20 +431,24 @@ int ldpc_set_stream_staging(ldpc_t *h, int32_t warps_per_cta, int32_t stages, in
  * ldpc_set_stream_messages: how the streaming variant keeps the check-to-bit messages of
  * FP32 codes whose rows have at most 27 edges. compressed = 1 (default): per row and frame
  * only the two smallest magnitudes min0 <= min1 of Observation 1, the first location of
- * min0 and the signs of Observation 2 (12 bytes per row; every message eta_ij of eq.
- * (eta_update) is rebuilt from them exactly), so the per-edge messages never travel
- * through DRAM; rows of at most 16 edges need the staged check pass for it
- * (ldpc_set_stream_staging with stages >= 2).
+ * min0 and the signs of Observation 2 (12 bytes per row, 10 where no row has more than 8
+ * edges; every message eta_ij of eq. (eta_update) is rebuilt from them exactly), so the
+ * per-edge messages never travel through DRAM. On rows of at most 16 edges staging must not be
+ * off (ldpc_set_stream_staging with stages -1).
  * compressed = 0: one stored message per edge slot. Results do not depend on the choice.
- * Fixed-point mode, rows longer than 27 edges and small batches always keep per-edge messages.
+ * Fixed-point mode, rows longer than 27 edges (or of fewer than 3 on average, without the padded
+ * layout) and, with automatic staging, batches of up to 64 frames always keep per-edge messages;
+ * so do frame groups (ldpc_set_stream_group) on rows of 17 to 27 edges that a lane takes fewer
+ * than 4 frames of.
  * ldpc_autotune also chooses this for FP32 codes. LDPC_ERR_INVALID_ARG for other values.
- * ldpc_get_stream_messages: 1 when the next streaming decode keeps compressed messages.
+ * ldpc_get_stream_messages: 1 when the next streaming decode of more than 64 frames keeps
+ * compressed messages.
  */
 int ldpc_set_stream_messages(ldpc_t *h, int32_t compressed);
 int ldpc_get_stream_messages(const ldpc_t *h, int32_t *compressed);
 
-/* ldpc_get_stream_staging: the staging in force (stages 0 when off; frames_per_lane 0 when
- * automatic). */
+/* ldpc_get_stream_staging: the staged pass's shape, asked for or automatic (stages 0 when off;
+ * frames_per_lane 0 when automatic); which decodes run it: ldpc_set_stream_staging. */
 int ldpc_get_stream_staging(const ldpc_t *h, int32_t *warps_per_cta, int32_t *stages,
                             int32_t *frames_per_lane);
 
@@ -470,7 +480,8 @@ int ldpc_read_messages(ldpc_t *h, int32_t frames, float *out);
 int ldpc_check_device(ldpc_t *h);
 
 /*
- * ldpc_set_wait_limit: tries of each bounded wait in the staged kernels. One try waits at
+ * ldpc_set_wait_limit: tries of each bounded wait in the staged kernels (decodes that run register
+ * kernels have none). One try waits at
  * most about 20 microseconds. The default 65536 bounds a wait near 1.3 s, far above any
  * real copy. A limit of 0 makes every wait give up at once, which is how the tests check
  * the timeout path without a fault. tries must be >= 0, else LDPC_ERR_INVALID_ARG.

@@ -1137,9 +1137,13 @@ int ldpc_get_stream_messages(const ldpc_t* h, int32_t* compressed) {
     }
     if (h->dg.ell_D == 0 || h->st_stages < 0) return LDPC_OK;
     if (h->w_rows > 0 && h->dg.n_classes > 256) return LDPC_OK;
-    // the staged kernel must fit (else the decode keeps per-edge messages)
     StreamWork w;
     apply_staging(h, w);
+    if (w.auto_staging) {  // the register kernel, which needs no shared memory
+        *compressed = 1;
+        return LDPC_OK;
+    }
+    // the staged kernel must fit (else the decode keeps per-edge messages)
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) {
         cudaGetLastError();

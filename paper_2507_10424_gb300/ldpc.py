@@ -424,7 +424,7 @@ class Decoder:
                "ldpc_set_stream_staging")
 
     def set_stream_messages(self, compressed: bool):
-        """Streaming variant, FP32, rows of at most 16 edges: keep each row's messages
+        """Streaming variant, FP32, rows of at most 27 edges: keep each row's messages
         compressed (two minima, location, signs) or one message per edge slot."""
         _check(load().ldpc_set_stream_messages(self.h, int(bool(compressed))),
                "ldpc_set_stream_messages")
