@@ -254,12 +254,12 @@ struct StreamWork {
     int32_t* err = nullptr;
     int32_t stage_warps = 0, stages = 0;
     int32_t stage_vw = 0;  // frames per lane of the staged kernel (0: the run's vector width)
-    int32_t auto_staging = 0;  // no shape was asked for: small batches may take narrow lanes
+    int32_t auto_staging = 0;  // no shape was asked for: register kernels where they serve better
     uint32_t wait_limit = 1u << 16;
     int32_t num_sms = 0;
     // FP32 codes on the padded row layout: keep each row's messages compressed (min0,
-    // min1, location and signs; cmsg.cuh) when the staged check pass runs, and for rows of 17
-    // to 27 edges (1), or keep one
+    // min1, location and signs; cmsg.cuh) unless staging is off or lanes are narrow, and for rows
+    // of 17 to 27 edges (1), or keep one
     // message per edge slot (0); used_compressed (host, nullable) receives the choice made
     int32_t msg_compressed = 1;
     int32_t* used_compressed = nullptr;
